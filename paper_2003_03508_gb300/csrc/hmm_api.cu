@@ -31,7 +31,7 @@ struct DevBuf {
 };
 
 struct Plan {
-    bool valid = false;
+    bool valid = false, sparse = false;
     int K = 0, n_prop = 0, n_seg = 0, precision = -1, L = 0;
     std::vector<int64_t> offsets;
     // derived
@@ -44,12 +44,17 @@ struct Plan {
     std::vector<SegFinal> segfinal;
     std::vector<int64_t> pbase;
     std::vector<ChunkDesc> chunks;
+    int strand_kp = 0;                      // 0: this shape runs on chunk products alone
+    std::vector<StrandDesc> strands;
+    std::vector<int32_t> strand_order;      // longest first
     // device copies (inside plan_buf)
     ChunkDesc *d_chunks = nullptr;
     TreeGroup *d_groups[MAX_LEVELS] = {};
     SegFinal *d_segs = nullptr;
     int64_t *d_offsets = nullptr;
     int64_t *d_pbase = nullptr;
+    StrandDesc *d_strands = nullptr;
+    int32_t *d_strand_order = nullptr;
 };
 
 }  // namespace
@@ -299,8 +304,102 @@ static bool tune_entry_valid(const TuneEntry &e) {
            e.L <= TUNE_L_MAX && e.L % OBS_WIN == 0 && e.ms >= 0.0;
 }
 
+// ---- strands (hmm_strand.cuh) ----
+
+// What a warp holds and costs, per padded state count: strands per warp,
+// warps an SM runs at once, and cycles of one step when the warp runs alone on its scheduler (latency)
+// and when others fill it (issue).
+struct StrandCost {
+    int per_warp, warps_per_sm, latency, issue;
+};
+
+static StrandCost strand_cost(int KP) {
+    switch (KP) {
+        case 4: return {strand_simt_per_warp(4), 16, 110, 40};
+        case 8: return {strand_simt_per_warp(8), 12, 160, 60};
+        case 16: return {strand_simt_per_warp(16), 12, 190, 95};
+        case 32: return {strand_simt_per_warp(32), 8, 260, 170};
+        default: return {strand_simt_per_warp(64), 8, 300, 180};
+    }
+}
+
+constexpr int STRAND_WARM = 256;        // covers the distance to meeting on tremor data (25 steps median, 200 at most)
+constexpr int STRAND_WARM_SHORT = 128;  // where a piece is short and the few that have not met can run on cheaply
+constexpr int STRAND_WARM_SPARSE = 512; // with the run-length option: rare tremors (260 steps median, 800 at most)
+
+static int strand_warm(int L, bool sparse) {
+    return sparse ? STRAND_WARM_SPARSE : L <= 512 ? STRAND_WARM_SHORT : STRAND_WARM;
+}
+
+// Piece length for a batch: the smallest modelled time over lengths growing by
+// about an eighth. One wave of warps takes (warm + L) steps, at the latency of
+// a step while a scheduler holds few warps and at their issue time beyond.
+static int choose_strand_len(int KP, int n_prop, const std::vector<int64_t> &steps, bool sparse, int n_sms) {
+    const StrandCost c = strand_cost(KP);
+    int64_t longest = 0;
+    for (int64_t n : steps) longest = std::max(longest, n);
+    const int64_t Lmax = std::max<int64_t>(OBS_WIN, (longest + OBS_WIN - 1) / OBS_WIN * OBS_WIN);
+    double best = 0.0;
+    int64_t best_L = 0;
+    for (int64_t L = OBS_WIN;; L = std::min(Lmax, (L + L / 8 + OBS_WIN) / OBS_WIN * OBS_WIN)) {
+        int64_t n = 0;
+        for (int64_t m : steps) n += (m + L - 1) / L;
+        const int64_t warps = (int64_t)n_prop * ((n + c.per_warp - 1) / c.per_warp);
+        const int64_t cap = (int64_t)n_sms * c.warps_per_sm;
+        const int64_t waves = std::max<int64_t>(1, (warps + cap - 1) / cap);
+        const int64_t resident = std::min(warps, cap);
+        const int64_t per_sched = (resident + 4 * n_sms - 1) / (4 * n_sms);
+        const double step = (double)std::max<int64_t>(c.latency, per_sched * c.issue);
+        const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm((int)L, sparse)) * step;
+        if (!best_L || t < best) {
+            best = t;
+            best_L = L;
+        }
+        if (L >= Lmax) break;
+    }
+    return (int)best_L;
+}
+
+static void build_strands(Plan &pl, bool sparse, int n_sms) {
+    pl.strands.clear();
+    pl.strand_order.clear();
+    pl.strand_kp = strand_simt_kp(pl.K);
+    std::vector<int64_t> steps;
+    for (int s = 0; s < pl.n_seg; ++s) steps.push_back(std::max<int64_t>(0, pl.offsets[s + 1] - pl.offsets[s] - 1));
+    int64_t all = 0;
+    for (int64_t n : steps) all += n;
+    // with the run-length option a short batch is done sooner by its binary
+    // powers: K=18, T=6416, 15 proposals 236 us against 266
+    if (!pl.strand_kp || pl.n_chunks == 0 || (sparse && all * pl.n_prop < (1 << 20))) {
+        pl.strand_kp = 0;
+        return;
+    }
+    const int L = choose_strand_len(pl.strand_kp, pl.n_prop, steps, sparse, n_sms);
+    for (int s = 0; s < pl.n_seg; ++s) {
+        // equal pieces of whole observation windows
+        const int64_t wins = (steps[s] + OBS_WIN - 1) / OBS_WIN;
+        const int64_t n = (steps[s] + L - 1) / L;
+        for (int64_t i = 0; i < n; ++i) {
+            const int64_t a = wins * i / n * OBS_WIN, b = std::min(steps[s], wins * (i + 1) / n * OBS_WIN);
+            const int64_t warm = std::min<int64_t>(a, strand_warm(L, sparse));
+            StrandDesc d;
+            d.pstart = pl.pbase[s] + a;
+            d.len = (int32_t)(b - a);
+            d.warm = (int32_t)warm;
+            d.seg = s;
+            d.flags = (warm == a ? SD_HEAD : 0) | (i == 0 ? SD_FIRST : 0) | (i + 1 == n ? SD_LAST : 0);
+            pl.strands.push_back(d);
+        }
+    }
+    pl.strand_order.resize(pl.strands.size());
+    for (size_t i = 0; i < pl.strands.size(); ++i) pl.strand_order[i] = (int32_t)i;
+    std::stable_sort(pl.strand_order.begin(), pl.strand_order.end(), [&](int32_t x, int32_t y) {
+        return pl.strands[x].warm + pl.strands[x].len > pl.strands[y].warm + pl.strands[y].len;
+    });
+}
+
 static void build_plan(Plan &pl, int K, int n_prop, int n_seg, const int64_t *offs, int precision,
-                       int L) {
+                       int L, bool sparse, int n_sms) {
     pl.K = K;
     pl.n_prop = n_prop;
     pl.n_seg = n_seg;
@@ -368,12 +467,14 @@ static void build_plan(Plan &pl, int K, int n_prop, int n_seg, const int64_t *of
         ++level;
     }
     pl.n_levels = level;
+    pl.sparse = sparse;
+    build_strands(pl, sparse, n_sms);
     pl.valid = true;
 }
 
 static bool plan_matches(const Plan &pl, int K, int n_prop, int n_seg, const int64_t *offs,
-                         int precision, int L) {
-    if (!pl.valid || pl.K != K || pl.n_prop != n_prop || pl.n_seg != n_seg ||
+                         int precision, int L, bool sparse) {
+    if (!pl.valid || pl.sparse != sparse || pl.K != K || pl.n_prop != n_prop || pl.n_seg != n_seg ||
         pl.precision != precision || pl.L != L)
         return false;
     return std::equal(pl.offsets.begin(), pl.offsets.end(), offs);
@@ -389,6 +490,8 @@ static int upload_plan(hmm_ctx *c, cudaStream_t st) {
     add(sizeof(SegFinal) * pl.segfinal.size());
     add(sizeof(int64_t) * pl.offsets.size());
     add(sizeof(int64_t) * pl.pbase.size());
+    add(sizeof(StrandDesc) * pl.strands.size());
+    add(sizeof(int32_t) * pl.strand_order.size());
     int rc = ensure(c, c->planbuf, bytes + 4096);
     if (rc) return rc;
     Carve cv(c->planbuf.p);
@@ -397,6 +500,8 @@ static int upload_plan(hmm_ctx *c, cudaStream_t st) {
     pl.d_segs = cv.take<SegFinal>(pl.segfinal.size());
     pl.d_offsets = cv.take<int64_t>(pl.offsets.size());
     pl.d_pbase = cv.take<int64_t>(pl.pbase.size());
+    pl.d_strands = cv.take<StrandDesc>(pl.strands.size());
+    pl.d_strand_order = cv.take<int32_t>(pl.strand_order.size());
     cudaError_t e = cudaSuccess;
     if (!pl.chunks.empty())
         e = cudaMemcpyAsync(pl.d_chunks, pl.chunks.data(), sizeof(ChunkDesc) * pl.chunks.size(), cudaMemcpyHostToDevice, st);
@@ -408,6 +513,10 @@ static int upload_plan(hmm_ctx *c, cudaStream_t st) {
         e = cudaMemcpyAsync(pl.d_offsets, pl.offsets.data(), sizeof(int64_t) * pl.offsets.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(pl.d_pbase, pl.pbase.data(), sizeof(int64_t) * pl.pbase.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !pl.strands.empty())
+        e = cudaMemcpyAsync(pl.d_strands, pl.strands.data(), sizeof(StrandDesc) * pl.strands.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !pl.strands.empty())
+        e = cudaMemcpyAsync(pl.d_strand_order, pl.strand_order.data(), sizeof(int32_t) * pl.strand_order.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host vectors may change after return
     if (e != cudaSuccess) {
         pl.valid = false;
@@ -529,6 +638,7 @@ int hmm_status(hmm_ctx *c, void *stream) {
 struct WorkPtrs {
     float *cblock = nullptr;
     int *prop_bad = nullptr, *obs_bad = nullptr;
+    StrandPtrs sp;
     float2 *packed = nullptr, *head = nullptr;
     LevelPtrs lv{};
 };
@@ -538,7 +648,21 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
     Carve cv(base);
     w->cblock = cv.take<float>((size_t)n_prop * lay.stride);
     w->prop_bad = cv.take<int>(n_prop);
-    w->obs_bad = cv.take<int>(1);
+    // cleared together at the start of a call: obs_bad and the list's length
+    w->obs_bad = cv.take<int>(2 + n_prop);
+    w->sp = StrandPtrs{};
+    if (pl.strand_kp) {
+        const size_t n = pl.strands.size(), m = (size_t)n_prop * n;
+        w->sp.n = (int)n;
+        w->sp.desc = pl.d_strands;
+        w->sp.order = pl.d_strand_order;
+        w->sp.todo = w->obs_bad + 1;
+        w->sp.route = cv.take<int>(n_prop);
+        w->sp.vs = cv.take<float>(m * pl.strand_kp);
+        w->sp.ve = cv.take<float>(m * pl.strand_kp);
+        w->sp.ex = cv.take<long long>(m);
+        w->sp.logr = cv.take<double>(m);
+    }
     w->packed = cv.take<float2>(pl.n_packed);
     w->head = cv.take<float2>(n_seg);
     w->lv = LevelPtrs{};
@@ -551,10 +675,13 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
     return cv.off;
 }
 
-int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, const float *P,
-                       const float *p, const float *mu, const float *cov, int32_t n_seg,
-                       const int64_t *offs, const float *xy, const uint8_t *tremor,
-                       const hmm_opts *opts_in, double *out, void *stream) {
+// The batched likelihood. With `products` every proposal's chunk products are
+// left in the workspace (level 0), as the boundary scans of the posterior and
+// of Viterbi read them; without, log L comes from strands where they apply.
+static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, const float *P,
+                          const float *p, const float *mu, const float *cov, int32_t n_seg,
+                          const int64_t *offs, const float *xy, const uint8_t *tremor,
+                          const hmm_opts *opts_in, double *out, bool products, void *stream) {
     if (!c) return HMM_EINVAL;
     c->last_launches = 0;
     hmm_opts opts;
@@ -604,8 +731,8 @@ int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, c
         L = tune_get(key);
         if (!L) L = choose_chunk_len(prec, n_prop, lay.KP, steps_total, c->n_sms);
     }
-    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L)) {
-        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L);
+    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0)) {
+        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, c->n_sms);
         if (c->plan.n_levels + 1 > MAX_LEVELS) {
             c->plan.valid = false;
             return fail(c, HMM_EINVAL, "too many chunks for the tree (raise chunk_len)");
@@ -635,38 +762,46 @@ int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, c
     float2 *packed = wp.packed;
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
+    // strands first; `todo` lists what is left to the chunk products (null: everything)
+    const StrandPtrs sp = products ? StrandPtrs{} : wp.sp;
+    const int *todo = sp.todo;
 
     // ---- launches ----
     // The whole sequence, on stream `s` (the caller's, or the capture stream).
     auto enqueue = [&](cudaStream_t s, int &launches) -> cudaError_t {
         launches = 0;
         prof_mark(c, HMM_PHASE_PREP, s);
-        cudaError_t r = cudaMemsetAsync(obs_bad, 0, sizeof(int), s);
-        if (r == cudaSuccess) { r = launch_prep(n_prop, K, lay, prec, opts.init_mode, pi, P, p, mu, cov, cblock, prop_bad, c->d_status, s); ++launches; }
+        cudaError_t r = cudaMemsetAsync(obs_bad, 0, 2 * sizeof(int), s);
+        if (r == cudaSuccess) { r = launch_prep(n_prop, K, lay, prec, opts.init_mode, pi, P, p, mu, cov, cblock, prop_bad, c->d_status, sp, s); ++launches; }
         prof_mark(c, HMM_PHASE_PACK, s);
         if (r == cudaSuccess && T_total > 0) { r = launch_pack(n_seg, pl.d_offsets, pl.d_pbase, T_total, xy, tremor, packed, head, obs_bad, c->d_status, s); ++launches; }
         prof_mark(c, HMM_PHASE_CHUNK, s);
+        if (r == cudaSuccess && sp.n > 0) {
+            r = launch_strand_simt(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
+            if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, cblock, packed, sp, s);
+            launches += 2;
+        }
         if (r == cudaSuccess && pl.n_chunks > 0) {
             if (min_run) {
-                r = launch_rle_table(n_prop, nb, lay, cblock, qtab, qexp, c->d_status, s);
+                r = launch_rle_table(n_prop, nb, lay, cblock, qtab, qexp, c->d_status, todo, s);
                 ++launches;
                 if (r == cudaSuccess)
                     r = launch_chunk_rle(n_prop, pl.n_chunks, renorm, min_run, nb, lay, cblock, qtab, qexp, pl.d_chunks,
-                                         packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, s);
+                                         packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, todo, s);
             } else if (prec == HMM_PREC_FP32_SIMT)
-                r = launch_chunk_simt(n_prop, pl.n_chunks, L, renorm, lay, cblock, pl.d_chunks, packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, s);
+                r = launch_chunk_simt(n_prop, pl.n_chunks, L, renorm, lay, cblock, pl.d_chunks, packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, todo, s);
             else
-                r = launch_chunk_tc(n_prop, pl.n_chunks, L, renorm, prec, lay, cblock, pl.d_chunks, packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, s);
+                r = launch_chunk_tc(n_prop, pl.n_chunks, L, renorm, prec, lay, cblock, pl.d_chunks, packed, lv.A[0], (int32_t *)lv.e[0], c->d_status, todo, s);
             ++launches;
         }
         prof_mark(c, HMM_PHASE_TREE, s);
         for (int l = 0; l < pl.n_levels && r == cudaSuccess; ++l) {
-            r = launch_tree_level(n_prop, KP, l, (int)pl.groups[l].size(), pl.d_groups[l], lv, c->d_status, s);
+            r = launch_tree_level(n_prop, KP, l, (int)pl.groups[l].size(), pl.d_groups[l], lv, c->d_status, todo, s);
             ++launches;
         }
         prof_mark(c, HMM_PHASE_FINAL, s);
         if (r == cudaSuccess) {
-            r = launch_final(n_prop, K, opts.init_mode, n_seg, pl.d_segs, head, lv, KP, pi, P, p, mu, cov, prop_bad, obs_bad, out, s);
+            r = launch_final(n_prop, K, opts.init_mode, n_seg, pl.d_segs, head, lv, KP, pi, P, p, mu, cov, prop_bad, obs_bad, out, sp, pl.strand_kp, s);
             ++launches;
         }
         prof_mark(c, HMM_PHASE_COUNT, s);
@@ -684,7 +819,7 @@ int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, c
             (uint64_t)(uintptr_t)cov, (uint64_t)(uintptr_t)xy, (uint64_t)(uintptr_t)tremor, (uint64_t)(uintptr_t)out,
             (uint64_t)(uintptr_t)c->work.p, c->plan_version, (uint64_t)n_prop, (uint64_t)K, (uint64_t)n_seg,
             (uint64_t)prec, (uint64_t)opts.init_mode, (uint64_t)renorm, (uint64_t)min_run, (uint64_t)L,
-            (uint64_t)T_total};
+            (uint64_t)T_total, (uint64_t)products};
         if (c->call_exec && c->call_key == key) {
             e = cudaGraphLaunch(c->call_exec, st);
             if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphLaunch");
@@ -743,6 +878,13 @@ int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, c
     return HMM_OK;
 }
 
+int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, const float *P,
+                       const float *p, const float *mu, const float *cov, int32_t n_seg,
+                       const int64_t *offs, const float *xy, const uint8_t *tremor,
+                       const hmm_opts *opts, double *out, void *stream) {
+    return loglik_batched(c, n_prop, K, pi, P, p, mu, cov, n_seg, offs, xy, tremor, opts, out, false, stream);
+}
+
 int hmm_loglik(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm_opts *opts,
                double *out, void *stream) {
     if (!c) return HMM_EINVAL;
@@ -769,8 +911,8 @@ static int posterior_impl(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs,
         o.chunk_len = (int32_t)std::min<int64_t>(16384, std::max<int64_t>(OBS_WIN, Lp));
     }
     // the likelihood path computes the chunk products (and log L)
-    int rc = hmm_loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
-                                obs->tremor, &o, loglik, stream);
+    int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
+                                obs->tremor, &o, loglik, true, stream);
     if (rc) return rc;
     const Plan &pl = c->plan;
     const int K = prm->K, KP = pl.lay.KP, C = std::max(1, pl.n_chunks);
@@ -863,8 +1005,8 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
         o.chunk_len = (int32_t)std::min<int64_t>(16384, std::max<int64_t>(OBS_WIN, Lp));
     }
     // parameters, observations and the chunk table (and log L) from the likelihood path
-    int rc = hmm_loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
-                                obs->tremor, &o, loglik, stream);
+    int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
+                                obs->tremor, &o, loglik, true, stream);
     if (rc) return rc;
     const Plan &pl = c->plan;
     const int KP = pl.lay.KP, C = std::max(1, pl.n_chunks);

@@ -163,10 +163,11 @@ __device__ __forceinline__ int quiet_run(const float2 *__restrict__ obs, int cap
 template <int KP>
 __global__ void __launch_bounds__(rle_threads<KP>())
 rle_table_kernel(int nb, ConstLayout lay, const float *__restrict__ cblock, float *__restrict__ qtab,
-                 int32_t *__restrict__ qexp, unsigned *__restrict__ status) {
+                 int32_t *__restrict__ qexp, unsigned *__restrict__ status, const int *__restrict__ todo) {
     __shared__ __align__(16) float sQ[KP * KP];
     __shared__ __align__(16) int32_t sR[KP];
-    const int q = blockIdx.x;
+    if (todo && (int)blockIdx.x >= todo[0]) return;
+    const int q = todo ? todo[1 + blockIdx.x] : blockIdx.x;
     const int i = threadIdx.x;
     const float *cb = cblock + (size_t)q * lay.stride;
     const float *cno = cb + lay.off_emis + EM_CNO * KP;
@@ -223,13 +224,14 @@ chunk_rle_kernel(int n_chunks, int renorm, int min_run, int nb, ConstLayout lay,
                  const float *__restrict__ cblock, const float *__restrict__ qtab,
                  const int32_t *__restrict__ qexp, const ChunkDesc *__restrict__ chunks,
                  const float2 *__restrict__ packed, float *__restrict__ A0, int32_t *__restrict__ e0,
-                 unsigned *__restrict__ status) {
+                 unsigned *__restrict__ status, const int *__restrict__ todo) {
     __shared__ __align__(16) float sP[KP * KP];
     __shared__ float sEm[EM_ROWS * KP];
     __shared__ float sL[KP];
     __shared__ __align__(16) float sD[KP];
 
-    const int q = blockIdx.y;
+    if (todo && (int)blockIdx.y >= todo[0]) return;
+    const int q = todo ? todo[1 + blockIdx.y] : blockIdx.y;
     const int ch = blockIdx.x;
     const int i = threadIdx.x;
     const bool owner = i < KP;
@@ -351,7 +353,7 @@ chunk_rle_warp_kernel(int n_chunks, int renorm, int min_run, int nb, ConstLayout
                       const float *__restrict__ cblock, const float *__restrict__ qtab,
                       const int32_t *__restrict__ qexp, const ChunkDesc *__restrict__ chunks,
                       const float2 *__restrict__ packed, float *__restrict__ A0, int32_t *__restrict__ e0,
-                      unsigned *__restrict__ status) {
+                      unsigned *__restrict__ status, const int *__restrict__ todo) {
     static_assert(KP <= 32, "one lane per row");
     extern __shared__ __align__(16) float smem[];
     float *sP = smem;                                   // KP x KP
@@ -359,7 +361,8 @@ chunk_rle_warp_kernel(int n_chunks, int renorm, int min_run, int nb, ConstLayout
     int32_t *sR = reinterpret_cast<int32_t *>(sQ + (size_t)nb * KP * KP);  // nb x KP
     float *sD = reinterpret_cast<float *>(sR + (size_t)nb * KP);           // RLE_WPC x KP
 
-    const int q = blockIdx.y;
+    if (todo && (int)blockIdx.y >= todo[0]) return;
+    const int q = todo ? todo[1 + blockIdx.y] : blockIdx.y;
     const int warp = threadIdx.x >> 5;
     const int i = threadIdx.x & 31;  // row of the running product = lane
     const int ch = blockIdx.x * RLE_WPC + warp;
@@ -530,12 +533,12 @@ int rle_levels(int L) {
 #define HMM_RLE_CASES(X) X(4) X(8) X(16) X(32) X(48) X(64) X(80)
 
 cudaError_t launch_rle_table(int n_prop, int nb, const ConstLayout &lay, const float *cblock, float *qtab,
-                             int32_t *qexp, unsigned *status, cudaStream_t st) {
+                             int32_t *qexp, unsigned *status, const int *todo, cudaStream_t st) {
     if (n_prop == 0) return cudaSuccess;
     switch (lay.KP) {
 #define HMM_RLE_T(KPV)                                                                                 \
     case KPV:                                                                                          \
-        rle_table_kernel<KPV><<<n_prop, rle_threads<KPV>(), 0, st>>>(nb, lay, cblock, qtab, qexp, status); \
+        rle_table_kernel<KPV><<<n_prop, rle_threads<KPV>(), 0, st>>>(nb, lay, cblock, qtab, qexp, status, todo); \
         return cudaGetLastError();
         HMM_RLE_CASES(HMM_RLE_T)
 #undef HMM_RLE_T
@@ -545,7 +548,7 @@ cudaError_t launch_rle_table(int n_prop, int nb, const ConstLayout &lay, const f
 
 cudaError_t launch_chunk_rle(int n_prop, int n_chunks, int renorm, int min_run, int nb, const ConstLayout &lay,
                              const float *cblock, const float *qtab, const int32_t *qexp, const ChunkDesc *chunks,
-                             const float2 *packed, float *A0, int32_t *e0, unsigned *status, cudaStream_t st) {
+                             const float2 *packed, float *A0, int32_t *e0, unsigned *status, const int *todo, cudaStream_t st) {
     if (n_chunks == 0 || n_prop == 0) return cudaSuccess;
     if (lay.KP <= 32) {
         const dim3 wgrid((n_chunks + RLE_WPC - 1) / RLE_WPC, n_prop);
@@ -559,7 +562,7 @@ cudaError_t launch_chunk_rle(int n_prop, int n_chunks, int renorm, int min_run, 
         if (e != cudaSuccess) return e;                                                                   \
         chunk_rle_warp_kernel<KPV><<<wgrid, 32 * RLE_WPC, smem, st>>>(n_chunks, renorm, min_run, nb, lay,  \
                                                                       cblock, qtab, qexp, chunks, packed,  \
-                                                                      A0, e0, status);                    \
+                                                                      A0, e0, status, todo);                    \
         return cudaGetLastError();                                                                        \
     }
             HMM_RLE_W(4) HMM_RLE_W(8) HMM_RLE_W(16) HMM_RLE_W(32)
@@ -573,7 +576,7 @@ cudaError_t launch_chunk_rle(int n_prop, int n_chunks, int renorm, int min_run, 
     case KPV:                                                                                         \
         chunk_rle_kernel<KPV><<<grid, rle_threads<KPV>(), 0, st>>>(n_chunks, renorm, min_run, nb, lay, \
                                                                    cblock, qtab, qexp, chunks, packed, \
-                                                                   A0, e0, status);                    \
+                                                                   A0, e0, status, todo);                    \
         return cudaGetLastError();
         HMM_RLE_CASES(HMM_RLE_C)
 #undef HMM_RLE_C

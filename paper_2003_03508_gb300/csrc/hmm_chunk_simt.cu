@@ -26,18 +26,20 @@ __device__ __forceinline__ void chunk_sync() {
     if constexpr (KP <= 32) __syncwarp(); else __syncthreads();
 }
 
-template <int KP, int CPC>
+template <int KP, int CPC, bool LISTED>
 __global__ void __launch_bounds__(KP *CPC)
 chunk_simt_kernel(int n_chunks, int L, int renorm, ConstLayout lay, const float *__restrict__ cblock,
                   const ChunkDesc *__restrict__ chunks, const float2 *__restrict__ packed,
-                  float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status) {
+                  float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status,
+                  const int *__restrict__ todo) {
     __shared__ __align__(16) float sP[KP * KP];
     __shared__ float sEm[EM_ROWS * KP];
     __shared__ float sL[CPC][KP];
     __shared__ __align__(16) float sD[CPC][KP];
     __shared__ float2 sObs[CPC][OBS_WIN];
 
-    const int q = blockIdx.y;
+    if (LISTED && (int)blockIdx.y >= todo[0]) return;
+    const int q = LISTED ? todo[1 + blockIdx.y] : blockIdx.y;
     const int c = threadIdx.x / KP;  // chunk slot in this CTA
     const int i = threadIdx.x % KP;  // row of the chunk product (= start state)
     const int j_chunk = blockIdx.x * CPC + c;
@@ -162,21 +164,22 @@ chunk_simt_kernel(int n_chunks, int L, int renorm, ConstLayout lay, const float 
 template <int KP, int CPC>
 static cudaError_t launch_simt_t(int n_prop, int n_chunks, int L, int renorm, const ConstLayout &lay,
                                  const float *cblock, const ChunkDesc *chunks, const float2 *packed,
-                                 float *A0, int32_t *e0, unsigned *status, cudaStream_t st) {
+                                 float *A0, int32_t *e0, unsigned *status, const int *todo, cudaStream_t st) {
     dim3 grid((n_chunks + CPC - 1) / CPC, n_prop);
-    chunk_simt_kernel<KP, CPC><<<grid, KP * CPC, 0, st>>>(n_chunks, L, renorm, lay, cblock, chunks,
-                                                          packed, A0, e0, status);
+    auto kern = todo ? chunk_simt_kernel<KP, CPC, true> : chunk_simt_kernel<KP, CPC, false>;
+    kern<<<grid, KP * CPC, 0, st>>>(n_chunks, L, renorm, lay, cblock, chunks,
+                                                          packed, A0, e0, status, todo);
     return cudaGetLastError();
 }
 
 cudaError_t launch_chunk_simt(int n_prop, int n_chunks, int L, int renorm, const ConstLayout &lay,
                               const float *cblock, const ChunkDesc *chunks, const float2 *packed,
-                              float *A0, int32_t *e0, unsigned *status, cudaStream_t st) {
+                              float *A0, int32_t *e0, unsigned *status, const int *todo, cudaStream_t st) {
     if (n_chunks == 0 || n_prop == 0) return cudaSuccess;
 #define HMM_SIMT_CASE(KPV, CPCV)                                                                 \
     case KPV:                                                                                    \
         return launch_simt_t<KPV, CPCV>(n_prop, n_chunks, L, renorm, lay, cblock, chunks, packed, \
-                                        A0, e0, status, st);
+                                        A0, e0, status, todo, st);
     switch (lay.KP) {
         HMM_SIMT_CASE(4, 32)
         HMM_SIMT_CASE(8, 16)

@@ -75,11 +75,14 @@ struct TcCfg {
     static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 
-template <int KP, int PREC, int G, int E>
+template <int KP, int PREC, int G, int E, bool LISTED>
 __global__ void __launch_bounds__(TcCfg<KP, PREC, G, E>::THREADS, 1)
 chunk_tc_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, const float *__restrict__ cblock,
                 const ChunkDesc *__restrict__ chunks, const float2 *__restrict__ packed,
-                float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status) {
+                float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status,
+                const int *__restrict__ todo) {
+    // proposals to work on: all, or those listed
+    const int np = LISTED ? todo[0] : n_prop;
     using C = TcCfg<KP, PREC, G, E>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -96,7 +99,8 @@ chunk_tc_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, const flo
     const int lane = threadIdx.x & 31;
     const int per_item = G * C::CPG;  // chunks per work item
     const int items_per_prop = (n_chunks + per_item - 1) / per_item;
-    const int n_items = n_prop * items_per_prop;
+    const int n_items = np * items_per_prop;
+    if (LISTED && (int)blockIdx.x >= n_items) return;  // the launch's grid fits the whole batch
 
     if (threadIdx.x == 0) {
         for (int g = 0; g < G; ++g) {
@@ -247,7 +251,7 @@ chunk_tc_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, const flo
             // previous item fully consumed by every epilogue warp (so every MMA
             // that read P has completed); agree on abort
             if (named_barrier_or(1, nthr_epi, *abort_flag != 0)) break;
-            const int q = item / items_per_prop;
+            const int q = LISTED ? todo[1 + item / items_per_prop] : item / items_per_prop;
             const int b = item % items_per_prop;
             const int steps = item_steps(b);
             if (ew == 0 && lane == 0) {
@@ -630,9 +634,9 @@ chunk_tc_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, const flo
 template <int KP, int PREC, int G, int E>
 cudaError_t launch_tc_t(int n_prop, int n_chunks, int renorm, const ConstLayout &lay, const float *cblock,
                         const ChunkDesc *chunks, const float2 *packed, float *A0, int32_t *e0, unsigned *status,
-                        cudaStream_t st) {
+                            const int *todo, cudaStream_t st) {
     using C = TcCfg<KP, PREC, G, E>;
-    auto kern = chunk_tc_kernel<KP, PREC, G, E>;
+    auto kern = todo ? chunk_tc_kernel<KP, PREC, G, E, true> : chunk_tc_kernel<KP, PREC, G, E, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
@@ -641,7 +645,8 @@ cudaError_t launch_tc_t(int n_prop, int n_chunks, int renorm, const ConstLayout 
     const int per_item = G * C::CPG;
     const long long n_items = (long long)n_prop * ((n_chunks + per_item - 1) / per_item);
     const int grid = (int)(n_items < sms ? n_items : sms);
-    kern<<<grid, C::THREADS, C::SMEM, st>>>(n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status);
+    kern<<<grid, C::THREADS, C::SMEM, st>>>(n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status,
+                                            todo);
     return cudaGetLastError();
 }
 
@@ -679,7 +684,7 @@ int chunk_tc_chunks_per_item(int KP, int precision) {
 cudaError_t launch_chunk_tc(int n_prop, int n_chunks, int L, int renorm, int precision,
                             const ConstLayout &lay, const float *cblock, const ChunkDesc *chunks,
                             const float2 *packed, float *A0, int32_t *e0, unsigned *status,
-                            cudaStream_t st) {
+                            const int *todo, cudaStream_t st) {
     // the observation windows are bulk copies that need every chunk to start
     // on a 64-step (512-byte) boundary of the packed sequence: chunk lengths
     // are multiples of 64 (segments are laid out on such boundaries)
@@ -687,12 +692,12 @@ cudaError_t launch_chunk_tc(int n_prop, int n_chunks, int L, int renorm, int pre
     if (n_chunks == 0 || n_prop == 0) return cudaSuccess;
     if (lay.KP > 32)
         return launch_chunk_tc_wide(n_prop, n_chunks, renorm, precision, lay, cblock, chunks, packed, A0, e0,
-                                    status, st);
+                                    status, todo, st);
 #define HMM_TC_CASE(KPV, PRECV)                                                                              \
     if (lay.KP == KPV && precision == PRECV)                                                                  \
         return launch_tc_t<KPV, PRECV, TcTile<KPV, PRECV>::G, TcTile<KPV, PRECV>::E>(n_prop, n_chunks, renorm, \
                                                                                    lay, cblock, chunks,       \
-                                                                                   packed, A0, e0, status, st);
+                                                                                   packed, A0, e0, status, todo, st);
     HMM_TC_CASE(16, HMM_PREC_TF32)
     HMM_TC_CASE(32, HMM_PREC_TF32)
     HMM_TC_CASE(16, HMM_PREC_TF32_SPLIT)

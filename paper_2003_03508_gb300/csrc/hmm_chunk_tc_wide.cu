@@ -74,11 +74,14 @@ struct WideCfg {
     static_assert(KP % KSTEP == 0 && KP % 16 == 0, "K tiling");
 };
 
-template <int KP, int PREC, int G, int E>
+template <int KP, int PREC, int G, int E, bool LISTED>
 __global__ void __launch_bounds__(WideCfg<KP, PREC, G, E>::THREADS, 1)
 chunk_tc_wide_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, const float *__restrict__ cblock,
                      const ChunkDesc *__restrict__ chunks, const float2 *__restrict__ packed,
-                     float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status) {
+                     float *__restrict__ A0, int32_t *__restrict__ e0, unsigned *__restrict__ status,
+                const int *__restrict__ todo) {
+    // proposals to work on: all, or those listed
+    const int np = LISTED ? todo[0] : n_prop;
     using C = WideCfg<KP, PREC, G, E>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -95,7 +98,8 @@ chunk_tc_wide_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, cons
     const int lane = threadIdx.x & 31;
     const int per_item = C::PI;
     const int items_per_prop = (n_chunks + per_item - 1) / per_item;
-    const int n_items = n_prop * items_per_prop;
+    const int n_items = np * items_per_prop;
+    if (LISTED && (int)blockIdx.x >= n_items) return;  // the launch's grid fits the whole batch
 
     if (threadIdx.x == 0) {
         for (int g = 0; g < G; ++g) {
@@ -257,7 +261,7 @@ chunk_tc_wide_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, cons
 
         for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
             if (named_barrier_or(1, nthr_epi, *abort_flag != 0)) break;
-            const int q = item / items_per_prop;
+            const int q = LISTED ? todo[1 + item / items_per_prop] : item / items_per_prop;
             const int b = item % items_per_prop;
             const int steps = item_steps(b);
             if (ew == 0 && lane == 0) {
@@ -479,9 +483,9 @@ chunk_tc_wide_kernel(int n_prop, int n_chunks, int renorm, ConstLayout lay, cons
 template <int KP, int PREC, int G, int E>
 cudaError_t launch_wide_t(int n_prop, int n_chunks, int renorm, const ConstLayout &lay, const float *cblock,
                           const ChunkDesc *chunks, const float2 *packed, float *A0, int32_t *e0, unsigned *status,
-                          cudaStream_t st) {
+                            const int *todo, cudaStream_t st) {
     using C = WideCfg<KP, PREC, G, E>;
-    auto kern = chunk_tc_wide_kernel<KP, PREC, G, E>;
+    auto kern = todo ? chunk_tc_wide_kernel<KP, PREC, G, E, true> : chunk_tc_wide_kernel<KP, PREC, G, E, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
@@ -490,7 +494,8 @@ cudaError_t launch_wide_t(int n_prop, int n_chunks, int renorm, const ConstLayou
     const int per_item = C::PI;
     const long long n_items = (long long)n_prop * ((n_chunks + per_item - 1) / per_item);
     const int grid = (int)(n_items < sms ? n_items : sms);
-    kern<<<grid, C::THREADS, C::SMEM, st>>>(n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status);
+    kern<<<grid, C::THREADS, C::SMEM, st>>>(n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status,
+                                            todo);
     return cudaGetLastError();
 }
 
@@ -527,12 +532,13 @@ int chunk_tc_wide_chunks_per_item(int KP, int precision) {
 
 cudaError_t launch_chunk_tc_wide(int n_prop, int n_chunks, int renorm, int precision, const ConstLayout &lay,
                                  const float *cblock, const ChunkDesc *chunks, const float2 *packed, float *A0,
-                                 int32_t *e0, unsigned *status, cudaStream_t st) {
+                                 int32_t *e0, unsigned *status,
+                            const int *todo, cudaStream_t st) {
     if (n_chunks == 0 || n_prop == 0) return cudaSuccess;
 #define HMM_WIDE_CASE(KPV, PRECV)                                                                         \
     if (lay.KP == KPV && precision == PRECV)                                                               \
         return launch_wide_t<KPV, PRECV, WideTile<KPV, PRECV>::G, WideTile<KPV, PRECV>::E>(                \
-            n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status, st);
+            n_prop, n_chunks, renorm, lay, cblock, chunks, packed, A0, e0, status, todo, st);
     HMM_WIDE_CASE(48, HMM_PREC_TF32)
     HMM_WIDE_CASE(64, HMM_PREC_TF32)
     HMM_WIDE_CASE(80, HMM_PREC_TF32)

@@ -40,6 +40,7 @@ enum {
     EM_QC = 4,   // -0.5 log2(e) sxx / det
     EM_CTR = 5,  // log2 p - log2(2 pi) - 0.5 log2 det
     EM_CNO = 6,  // log2 (1 - p)
+    EM_OFF = 7,  // [0], [1]: whole numbers next above the row maxima of EM_CTR and EM_CNO
     EM_ROWS = 8,
 };
 
@@ -58,6 +59,34 @@ struct ChunkDesc {
     int64_t pstart;  // index of the chunk's first step in `packed`
     int32_t len;     // steps in this chunk (1..L)
     int32_t seg;     // segment it belongs to
+};
+
+// One strand: the forward vector of one proposal carried over `len` steps of a
+// segment (hmm_strand.cuh). It starts `warm` steps earlier, from a flat vector
+// or, when that reaches the segment's start, from the head vector.
+struct StrandDesc {
+    int64_t pstart;  // index of the piece's first step in `packed` (a multiple of OBS_WIN)
+    int32_t len;     // steps in the piece (>= 1)
+    int32_t warm;    // steps run before the piece (a multiple of OBS_WIN)
+    int32_t seg;     // segment it belongs to
+    int32_t flags;   // SD_HEAD (starts at the head vector), SD_FIRST, SD_LAST (of its segment)
+};
+enum { SD_HEAD = 1, SD_FIRST = 2, SD_LAST = 4 };
+
+// How a proposal's log L is formed (route[q]): by strands, by chunk products
+// (listed in todo[1..], todo[0] of them), or not at all (invalid parameters)
+enum { ROUTE_STRANDS = 0, ROUTE_CHUNKS = 1, ROUTE_BAD = 2 };
+
+struct StrandPtrs {
+    const StrandDesc *desc = nullptr;  // [n], by segment and position
+    const int32_t *order = nullptr;    // [n], longest first: the warps' order
+    int n = 0;
+    float *vs = nullptr;       // [n_prop][n][KP] vector at the piece's start
+    float *ve = nullptr;       // [n_prop][n][KP] vector at its end
+    long long *ex = nullptr;   // [n_prop][n] power-of-two exponent of ve relative to vs
+    double *logr = nullptr;    // [n_prop][n] log scale of the true vector over vs at the piece's start
+    int *route = nullptr;      // [n_prop]
+    int *todo = nullptr;       // [1 + n_prop]
 };
 
 struct ConstLayout {
@@ -120,7 +149,7 @@ ConstLayout make_layout(int K, int precision);
 cudaError_t launch_prep(int n_prop, int K, const ConstLayout &lay, int precision, int init_mode,
                         const float *pi, const float *P, const float *p, const float *mu,
                         const float *cov, float *cblock, int *prop_bad, unsigned *status,
-                        cudaStream_t st);
+                        const StrandPtrs &sp, cudaStream_t st);
 
 cudaError_t launch_pack(int n_seg, const int64_t *d_offsets, const int64_t *d_pbase,
                         int64_t T_total, const float *xy, const uint8_t *tremor, float2 *packed,
@@ -128,16 +157,29 @@ cudaError_t launch_pack(int n_seg, const int64_t *d_offsets, const int64_t *d_pb
 
 cudaError_t launch_chunk_simt(int n_prop, int n_chunks, int L, int renorm, const ConstLayout &lay,
                               const float *cblock, const ChunkDesc *chunks, const float2 *packed,
-                              float *A0, int32_t *e0, unsigned *status, cudaStream_t st);
+                              float *A0, int32_t *e0, unsigned *status, const int *todo, cudaStream_t st);
+
+// Strands (hmm_strand_simt.cu) and their join (hmm_join.cu). strand_simt_kp: the
+// padded state count (0: K too large).
+int strand_simt_kp(int K);
+int strand_simt_per_warp(int KP);
+cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+                               const float *cblock, const float *pi, const float2 *head, const float2 *packed,
+                               const StrandPtrs &sp, cudaStream_t st);
+cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
+                        const float2 *packed, const StrandPtrs &sp, cudaStream_t st);
+
+// The chunk-product kernels and the tree take a list of the proposals to work
+// on, todo[0] of them in todo[1..] (null: all n_prop).
 
 // run-length shortcut (FP32 on the CUDA cores): table of M_0^(2^b), b < nb,
 // then chunk products that apply runs of >= min_run no-tremor steps from it
 int rle_levels(int L);
 cudaError_t launch_rle_table(int n_prop, int nb, const ConstLayout &lay, const float *cblock, float *qtab,
-                             int32_t *qexp, unsigned *status, cudaStream_t st);
+                             int32_t *qexp, unsigned *status, const int *todo, cudaStream_t st);
 cudaError_t launch_chunk_rle(int n_prop, int n_chunks, int renorm, int min_run, int nb, const ConstLayout &lay,
                              const float *cblock, const float *qtab, const int32_t *qexp, const ChunkDesc *chunks,
-                             const float2 *packed, float *A0, int32_t *e0, unsigned *status, cudaStream_t st);
+                             const float2 *packed, float *A0, int32_t *e0, unsigned *status, const int *todo, cudaStream_t st);
 
 bool chunk_tc_supported(int K, int precision);
 int chunk_tc_chunks_per_item(int KP, int precision);
@@ -152,11 +194,11 @@ cudaError_t launch_viterbi(int K, int init_mode, int n_chunks, int L, const Cons
                            int32_t *path, double *score, cudaStream_t st);
 cudaError_t launch_chunk_tc_wide(int n_prop, int n_chunks, int renorm, int precision, const ConstLayout &lay,
                                  const float *cblock, const ChunkDesc *chunks, const float2 *packed, float *A0,
-                                 int32_t *e0, unsigned *status, cudaStream_t st);
+                                 int32_t *e0, unsigned *status, const int *todo, cudaStream_t st);
 cudaError_t launch_chunk_tc(int n_prop, int n_chunks, int L, int renorm, int precision,
                             const ConstLayout &lay, const float *cblock, const ChunkDesc *chunks,
                             const float2 *packed, float *A0, int32_t *e0, unsigned *status,
-                            cudaStream_t st);
+                            const int *todo, cudaStream_t st);
 
 // Fisher-identity gradient and EM M-step from the E-step statistics (hmm_grad.cu)
 cudaError_t launch_fisher_grad(int K, int init_mode, const float *pi, const float *P, const float *p, const float *mu,
@@ -166,11 +208,11 @@ cudaError_t launch_em_mstep(int K, const float *pi, const float *P, const float 
                             float *cov_out, cudaStream_t st);
 
 cudaError_t launch_tree_level(int n_prop, int KP, int level, int n_groups, const TreeGroup *groups,
-                              const LevelPtrs &lv, unsigned *status, cudaStream_t st);
+                              const LevelPtrs &lv, unsigned *status, const int *todo, cudaStream_t st);
 
 cudaError_t launch_final(int n_prop, int K, int init_mode, int n_seg, const SegFinal *segs,
                          const float2 *head, const LevelPtrs &lv, int KP, const float *pi,
                          const float *P, const float *p, const float *mu, const float *cov,
-                         const int *prop_bad, const int *obs_bad, double *out, cudaStream_t st);
+                         const int *prop_bad, const int *obs_bad, double *out, const StrandPtrs &sp, int strand_kp, cudaStream_t st);
 
 }  // namespace hmm

@@ -1,0 +1,255 @@
+// Joining the strands of a segment (hmm_strand.cuh): one warp per piece that
+// is not its segment's first compares the vector its strand had at the piece's
+// start, g, with the end of the strand before, a. If a = r g within the
+// tolerance in every entry, log r is noted. Otherwise both vectors run on
+// through the piece, with exact scaling, until they meet; a piece that ends
+// before they do sends its proposal to the chunk products.
+//
+// Nearly every piece meets at once (the warm-up covers the usual distance), so
+// the kernel reads 2 KP floats a piece; the rest are a few hundred steps of
+// one warp each, bound by the latency of a step.
+#include "hmm_strand.cuh"
+
+namespace hmm {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr float JOIN_TINY = 8.470329472543003e-22f;  // 2^-70: an entry this far below the largest cannot matter (PMIN)
+constexpr int JOIN_WARPS = 4;
+
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
+    return v;
+}
+__device__ __forceinline__ float warp_min(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(FULL, v, o));
+    return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+}
+
+// NC: states per lane (KP <= 32 NC)
+template <int NC>
+__global__ void __launch_bounds__(32 * JOIN_WARPS)
+join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float tol, const float *__restrict__ cblock,
+            const float2 *__restrict__ packed, StrandPtrs sp) {
+    __shared__ __align__(16) float2 sag[JOIN_WARPS][32 * NC];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long id = (long long)blockIdx.x * JOIN_WARPS + warp;
+    const int q = (int)(id / sp.n), s = (int)(id % sp.n);
+    if (q >= n_prop || __shfl_sync(FULL, sp.route[q], 0) != ROUTE_STRANDS) return;
+    const StrandDesc d = sp.desc[s];
+    const size_t idx = (size_t)q * sp.n + s;
+    if (d.flags & SD_FIRST) {
+        if (lane == 0) sp.logr[idx] = 0.0;
+        return;
+    }
+    float a[NC], g[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int k = lane + 32 * c;
+        a[c] = k < K ? sp.ve[(idx - 1) * KP + k] : 0.0f;
+        g[c] = k < K ? sp.vs[idx * KP + k] : 0.0f;
+    }
+    auto met = [&]() {
+        float lo = INFINITY, hi = 0.0f;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (a[c] > JOIN_TINY || g[c] > JOIN_TINY) {
+                const float r = a[c] / g[c];
+                lo = fminf(lo, r);
+                hi = fmaxf(hi, r);
+            }
+        lo = warp_min(lo);
+        hi = warp_max(hi);
+        return hi <= lo * (1.0f + tol);  // false for NaN
+    };
+    int ea = 0, eg = 0;  // exponents gathered while running on (both in [1, 2) at the start)
+    long long de = 0;
+    bool ok = met();
+    if (!ok) {
+        const float *cb = cblock + (size_t)q * lay.stride;
+        const float *em = cb + lay.off_emis;
+        const int KPl = lay.KP;
+        auto load_p = [&](int i, int k) {
+            float v = i < KPl && k < KPl ? cb[lay.off_p32 + i * KPl + k] : 0.0f;
+            if (round_tf32) {
+                uint32_t r;
+                asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
+                v = __uint_as_float(r);
+            }
+            return v;
+        };
+        f32x2 pc[NC == 1 ? 32 : 1];  // this lane's column of P, each entry twice
+        if (NC == 1) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const float v = load_p(i, lane);
+                pc[NC == 1 ? i : 0] = pack2(v, v);
+            }
+        }
+        float c[NC][7];
+        float offt, offn;
+        strand_offsets(em, KPl, offt, offn);
+#pragma unroll
+        for (int n = 0; n < NC; ++n) {
+            const int k = lane + 32 * n;
+#pragma unroll
+            for (int r = 0; r < 7; ++r) c[n][r] = k < K ? em[r * KPl + k] : r >= EM_CTR ? -INFINITY : 0.0f;
+            c[n][EM_CTR] -= offt;
+            c[n][EM_CNO] -= offn;
+        }
+        // log2 emission factor of state lane + 32 n, relative to the whole offsets
+        auto emission = [&](int n, float x, float y) {
+            const float dx = x - c[n][EM_MUX], dy = y - c[n][EM_MUY];
+            const float l = fmaf(fmaf(c[n][EM_QA], dx, c[n][EM_QB] * dy), dx, fmaf(c[n][EM_QC] * dy, dy, c[n][EM_CTR]));
+            return isnan(x) ? c[n][EM_CNO] : l;
+        };
+        // one step of both vectors: (a, g) <- ((a, g) P) f
+        auto step = [&](const float (&f)[NC]) {
+#pragma unroll
+            for (int n = 0; n < NC; ++n) sag[warp][lane + 32 * n] = make_float2(a[n], g[n]);
+            __syncwarp();
+            f32x2 acc[NC][4];
+#pragma unroll
+            for (int n = 0; n < NC; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0ull;
+            if (NC == 1) {
+#pragma unroll
+                for (int i = 0; i < 32; i += 2) {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sag[warp][i]);
+                    acc[0][i & 2] = fma2(x.x, pc[NC == 1 ? i : 0], acc[0][i & 2]);
+                    acc[0][(i & 2) + 1] = fma2(x.y, pc[NC == 1 ? i + 1 : 0], acc[0][(i & 2) + 1]);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = 0; i < 32 * NC; i += 2) {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sag[warp][i]);
+#pragma unroll
+                    for (int n = 0; n < NC; ++n) {
+                        const float v = load_p(i, lane + 32 * n), w = load_p(i + 1, lane + 32 * n);
+                        acc[n][0] = fma2(x.x, pack2(v, v), acc[n][0]);
+                        acc[n][1] = fma2(x.y, pack2(w, w), acc[n][1]);
+                    }
+                }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                unpack2(add2(add2(acc[n][0], acc[n][1]), add2(acc[n][2], acc[n][3])), a[n], g[n]);
+                a[n] *= f[n];
+                g[n] *= f[n];
+            }
+        };
+        // both back to [1, 2); false when one left the range
+        auto rescale = [&]() {
+            float ma = 0.0f, mg = 0.0f;
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                ma = fmaxf(ma, a[n]);
+                mg = fmaxf(mg, g[n]);
+            }
+            ma = warp_max(ma);
+            mg = warp_max(mg);
+            if (!(ma >= STRAND_SHRINK && mg >= STRAND_SHRINK && ma <= STRAND_GROW && mg <= STRAND_GROW)) return false;
+            const int xa = float_exponent(ma), xg = float_exponent(mg);
+            const float fa = pow2f(-xa), fg = pow2f(-xg);
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                a[n] *= fa;
+                g[n] *= fg;
+            }
+            ea += xa;
+            eg += xg;
+            return true;
+        };
+        bool alive = true;
+        for (int t0 = 0; t0 < d.len && !ok && alive; t0 += 32) {
+            // 32 steps' observations, one per lane (the packed sequence is padded to whole windows)
+            const float2 ob = packed[d.pstart + t0 + lane];
+            for (int t = t0; t < min(t0 + 32, d.len) && !ok && alive; t += 4) {
+                const int m = min(4, d.len - t);
+                float ka[NC], kg[NC];
+#pragma unroll
+                for (int n = 0; n < NC; ++n) {
+                    ka[n] = a[n];
+                    kg[n] = g[n];
+                }
+                bool fine = m == 4;
+                if (fine) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float x = __shfl_sync(FULL, ob.x, t - t0 + j), y = __shfl_sync(FULL, ob.y, t - t0 + j);
+                        float f[NC];
+#pragma unroll
+                        for (int n = 0; n < NC; ++n) f[n] = ex2(emission(n, x, y));
+                        step(f);
+                    }
+                    fine = rescale();
+                }
+                if (!fine) {
+                    // step by step with exact scaling (as in the strands)
+#pragma unroll
+                    for (int n = 0; n < NC; ++n) {
+                        a[n] = ka[n];
+                        g[n] = kg[n];
+                    }
+                    for (int j = 0; j < m && alive; ++j) {
+                        const float x = __shfl_sync(FULL, ob.x, t - t0 + j), y = __shfl_sync(FULL, ob.y, t - t0 + j);
+                        float f[NC], mx = -INFINITY;
+#pragma unroll
+                        for (int n = 0; n < NC; ++n) {
+                            f[n] = emission(n, x, y);
+                            mx = fmaxf(mx, f[n]);
+                        }
+                        mx = warp_max(mx);
+                        alive = mx + (isnan(x) ? offn : offt) >= -(float)EXP_LIMIT;
+                        const float fm = alive ? floorf(mx) : 0.0f;
+#pragma unroll
+                        for (int n = 0; n < NC; ++n) f[n] = ex2(f[n] - fm);
+                        step(f);
+                        alive = alive && rescale();
+                    }
+                }
+                ok = alive && met();
+            }
+            de += (long long)ea - eg;
+            ea = eg = 0;
+        }
+    }
+    double sa = 0.0, sg = 0.0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        sa += a[c];
+        sg += g[c];
+    }
+    sa = warp_sum(sa);
+    sg = warp_sum(sg);
+    if (lane == 0) {
+        if (ok) sp.logr[idx] = log(sa / sg) + 0.69314718055994530942 * (double)(de + ea - eg);
+        else send_to_chunks(sp, q);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
+                        const float2 *packed, const StrandPtrs &sp, cudaStream_t st) {
+    if (sp.n == 0) return cudaSuccess;
+    // FP32 vectors that have met differ by their rounding only, a few 2^-20
+    const float tol = 3.0517578125e-5f;  // 2^-15
+    const bool rt = precision == HMM_PREC_TF32;
+    const long long warps = (long long)n_prop * sp.n;
+    const unsigned grid = (unsigned)((warps + JOIN_WARPS - 1) / JOIN_WARPS);
+    if (KP <= 32) join_kernel<1><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
+    else if (KP <= 64) join_kernel<2><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
+    else join_kernel<3><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
+    return cudaGetLastError();
+}
+
+}  // namespace hmm

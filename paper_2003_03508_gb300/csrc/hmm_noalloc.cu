@@ -203,19 +203,19 @@ extern "C" int hmm_loglik_noalloc(const hmm_params *prm, const hmm_obs *obs, dou
     }
     if (e == cudaSuccess)
         e = launch_prep(1, K, lay, HMM_PREC_FP32_SIMT, 0, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov,
-                        cblock, prop_bad, status, st);
+                        cblock, prop_bad, status, StrandPtrs{}, st);
     if (e == cudaSuccess && T > 0)
         e = launch_pack(1, offs, pbase, T, obs->xy, obs->tremor, packed, head, obs_bad, status, st);
     if (e == cudaSuccess && C > 0)
-        e = launch_chunk_simt(1, C, NA_L, 4, lay, cblock, chunks, packed, lv.A[0], (int32_t *)lv.e[0], status, st);
+        e = launch_chunk_simt(1, C, NA_L, 4, lay, cblock, chunks, packed, lv.A[0], (int32_t *)lv.e[0], status, nullptr, st);
     int gbase = 0;
     for (int l = 0; l < L.n_levels && e == cudaSuccess; ++l) {
-        e = launch_tree_level(1, lay.KP, l, L.n_groups[l], groups + gbase, lv, status, st);
+        e = launch_tree_level(1, lay.KP, l, L.n_groups[l], groups + gbase, lv, status, nullptr, st);
         gbase += L.n_groups[l];
     }
     if (e == cudaSuccess)
         e = launch_final(1, K, HMM_INIT_EMIT_FIRST, 1, segs, head, lv, lay.KP, prm->pi, prm->P, prm->p_tremor,
-                         prm->mu, prm->cov, prop_bad, obs_bad, out_dev, st);
+                         prm->mu, prm->cov, prop_bad, obs_bad, out_dev, StrandPtrs{}, 0, st);
     if (e == cudaSuccess) {
         noalloc_status_kernel<<<1, 1, 0, st>>>(status, out_dev);
         e = cudaGetLastError();

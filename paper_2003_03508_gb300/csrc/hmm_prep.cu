@@ -11,7 +11,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
-#include "hmm_internal.cuh"
+#include "hmm_strand.cuh"
 
 namespace hmm {
 
@@ -57,7 +57,7 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
                             const float *__restrict__ P, const float *__restrict__ p,
                             const float *__restrict__ mu, const float *__restrict__ cov,
                             float *__restrict__ cblock, int *__restrict__ prop_bad,
-                            unsigned *__restrict__ status) {
+                            unsigned *__restrict__ status, StrandPtrs sp) {
     const int q = blockIdx.x;
     const int KP = lay.KP;
     pi += (size_t)q * K;
@@ -66,8 +66,8 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
     mu += (size_t)q * 2 * K;
     cov += (size_t)q * 3 * K;
     float *cb = cblock + (size_t)q * lay.stride;
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
+    __shared__ int bad, small;
+    if (threadIdx.x == 0) bad = small = 0;
     __syncthreads();
 
     // rows of P: non-negative, finite, summing to 1 within 1e-5
@@ -77,6 +77,7 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
         for (int j = 0; j < K; ++j) {
             float v = P[i * K + j];
             ok = ok && isfinite(v) && v >= 0.0f;
+            if (v < STRAND_PMIN) small = 1;
             s += v;
         }
         if (!ok || fabs(s - 1.0) > 1e-5) bad = 1;
@@ -123,7 +124,6 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
         em[EM_QC * KP + k] = qc;
         em[EM_CTR * KP + k] = ctr;
         em[EM_CNO * KP + k] = cno;
-        em[7 * KP + k] = 0.f;
     }
     // P padded to KP x KP (FP32, row-major) and the tensor-core images
     for (int idx = threadIdx.x; idx < KP * KP; idx += blockDim.x) {
@@ -145,19 +145,45 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        prop_bad[q] = bad;
-        if (bad) atomicOr(status, ST_EINVAL);
+    if (threadIdx.x < 32) {
+        // EM_OFF: the emissions' largest constants, rounded up to whole numbers
+        float *em = cb + lay.off_emis;
+        float mt = -INFINITY, mn = -INFINITY;
+        for (int k = threadIdx.x; k < K; k += 32) {
+            mt = fmaxf(mt, em[EM_CTR * KP + k]);
+            mn = fmaxf(mn, em[EM_CNO * KP + k]);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+            mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        }
+        if (threadIdx.x == 0) {
+            mt = isfinite(mt) ? ceilf(mt) : 0.0f;
+            mn = isfinite(mn) ? ceilf(mn) : 0.0f;
+            em[EM_OFF * KP] = mt;
+            em[EM_OFF * KP + 1] = mn;
+            prop_bad[q] = bad;
+            if (bad) atomicOr(status, ST_EINVAL);
+            if (sp.route) {
+                // strands need P's entries above STRAND_PMIN and constants of ordinary size
+                const bool fits = !small && fabsf(mt) <= 1000.0f && fabsf(mn) <= 1000.0f;
+                sp.route[q] = bad ? ROUTE_BAD : ROUTE_STRANDS;
+                if (!bad && !fits) {
+                    sp.route[q] = ROUTE_CHUNKS;
+                    sp.todo[1 + atomicAdd(&sp.todo[0], 1)] = q;
+                }
+            }
+        }
     }
 }
 
 cudaError_t launch_prep(int n_prop, int K, const ConstLayout &lay, int precision, int init_mode,
                         const float *pi, const float *P, const float *p, const float *mu,
                         const float *cov, float *cblock, int *prop_bad, unsigned *status,
-                        cudaStream_t st) {
+                        const StrandPtrs &sp, cudaStream_t st) {
     (void)init_mode;
     prep_kernel<<<n_prop, 128, 0, st>>>(K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad,
-                                        status);
+                                        status, sp);
     return cudaGetLastError();
 }
 

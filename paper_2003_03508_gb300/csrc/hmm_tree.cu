@@ -31,7 +31,8 @@ constexpr int TREE_THREADS = 256;
 template <bool E32>
 __global__ void __launch_bounds__(TREE_THREADS)
 tree_level_kernel(int KP, int level, const TreeGroup *__restrict__ groups, LevelPtrs lv,
-                  unsigned *__restrict__ status) {
+                  unsigned *__restrict__ status, const int *__restrict__ todo) {
+    if (todo && (int)blockIdx.y >= todo[0]) return;
     extern __shared__ __align__(16) float smem[];
     float *X = smem;
     float *Y = X + KP * KP;
@@ -39,7 +40,7 @@ tree_level_kernel(int KP, int level, const TreeGroup *__restrict__ groups, Level
     long long *ey = ex + KP;
     long long *mrow = ey + KP;  // m_i of the current product
 
-    const int q = blockIdx.y;
+    const int q = todo ? todo[1 + blockIdx.y] : blockIdx.y;
     const TreeGroup g = groups[blockIdx.x];
     const size_t nin = (size_t)lv.n[level];
     const float *Ain = lv.A[level] + (size_t)q * nin * KP * KP;
@@ -149,16 +150,16 @@ tree_level_kernel(int KP, int level, const TreeGroup *__restrict__ groups, Level
 }
 
 cudaError_t launch_tree_level(int n_prop, int KP, int level, int n_groups, const TreeGroup *groups,
-                              const LevelPtrs &lv, unsigned *status, cudaStream_t st) {
+                              const LevelPtrs &lv, unsigned *status, const int *todo, cudaStream_t st) {
     if (n_groups == 0) return cudaSuccess;
     size_t smem = (size_t)2 * KP * KP * sizeof(float) + 3 * KP * sizeof(long long);
     dim3 grid(n_groups, n_prop);
     if (level == 0) {
         cudaFuncSetAttribute(tree_level_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        tree_level_kernel<true><<<grid, TREE_THREADS, smem, st>>>(KP, level, groups, lv, status);
+        tree_level_kernel<true><<<grid, TREE_THREADS, smem, st>>>(KP, level, groups, lv, status, todo);
     } else {
         cudaFuncSetAttribute(tree_level_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        tree_level_kernel<false><<<grid, TREE_THREADS, smem, st>>>(KP, level, groups, lv, status);
+        tree_level_kernel<false><<<grid, TREE_THREADS, smem, st>>>(KP, level, groups, lv, status, todo);
     }
     return cudaGetLastError();
 }
@@ -197,7 +198,7 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
              const float2 *__restrict__ head, LevelPtrs lv, const float *__restrict__ pi,
              const float *__restrict__ P, const float *__restrict__ p, const float *__restrict__ mu,
              const float *__restrict__ cov, const int *__restrict__ prop_bad,
-             const int *__restrict__ obs_bad, double *__restrict__ out) {
+             const int *__restrict__ obs_bad, StrandPtrs sp, int strand_kp, double *__restrict__ out) {
     __shared__ double red[FINAL_THREADS];
     __shared__ double lpi0[80];   // log of the initial vector
     __shared__ double w[80];      // log h_i + ex_i ln 2
@@ -223,8 +224,26 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
     }
     __syncthreads();
     double total = 0.0;
+    // strands: each contributes its exponents and its scale over the strand
+    // before; a segment's last one the sum of its vector as well
+    const bool strands = sp.route && sp.route[q] == ROUTE_STRANDS;
+    if (strands) {
+        double part = 0.0;
+        for (int i = tid; i < sp.n; i += FINAL_THREADS) {
+            const size_t idx = (size_t)q * sp.n + i;
+            double v = (double)sp.ex[idx] * LN2 + sp.logr[idx];
+            if (sp.desc[i].flags & SD_LAST) {
+                double a = 0.0;
+                for (int k = 0; k < K; ++k) a += (double)sp.ve[idx * strand_kp + k];
+                v += log(a);
+            }
+            part += v;
+        }
+        total = block_sum_fixed(part, red);
+    }
     for (int s = 0; s < n_seg; ++s) {
         const SegFinal sf = segs[s];
+        if (strands && sf.T > 1) continue;
         double ll;
         if (sf.T == 0) {
             double a = 0.0;
@@ -288,9 +307,10 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
 cudaError_t launch_final(int n_prop, int K, int init_mode, int n_seg, const SegFinal *segs,
                          const float2 *head, const LevelPtrs &lv, int KP, const float *pi,
                          const float *P, const float *p, const float *mu, const float *cov,
-                         const int *prop_bad, const int *obs_bad, double *out, cudaStream_t st) {
+                         const int *prop_bad, const int *obs_bad, double *out, const StrandPtrs &sp, int strand_kp,
+                         cudaStream_t st) {
     final_kernel<<<n_prop, FINAL_THREADS, 0, st>>>(K, KP, init_mode, n_seg, segs, head, lv, pi, P, p,
-                                                   mu, cov, prop_bad, obs_bad, out);
+                                                   mu, cov, prop_bad, obs_bad, sp, strand_kp, out);
     return cudaGetLastError();
 }
 
