@@ -45,6 +45,7 @@ struct Plan {
     std::vector<int64_t> pbase;
     std::vector<ChunkDesc> chunks;
     int strand_kp = 0;                      // 0: this shape runs on chunk products alone
+    bool strand_tensor = false;             // strands on the tensor cores
     std::vector<StrandDesc> strands;
     std::vector<int32_t> strand_order;      // longest first
     // device copies (inside plan_buf)
@@ -306,56 +307,70 @@ static bool tune_entry_valid(const TuneEntry &e) {
 
 // ---- strands (hmm_strand.cuh) ----
 
-// What a warp holds and costs, per padded state count: strands per warp,
-// warps an SM runs at once, and cycles of one step when the warp runs alone on its scheduler (latency)
+// What a warp holds and costs, per kernel and padded state count: strands per
+// warp, warps an SM runs at once, whether warps come in fours of one proposal,
+// and cycles of one step when the warp runs alone on its scheduler (latency)
 // and when others fill it (issue).
 struct StrandCost {
-    int per_warp, warps_per_sm, latency, issue;
+    int per_warp, warps_per_sm, fours, latency, issue;
 };
 
-static StrandCost strand_cost(int KP) {
+static StrandCost strand_cost(bool tensor, int KP, int precision) {
+    if (tensor) {
+        switch (KP) {
+            case 16: return {strand_mma_per_warp(16), 16, 0, 330, precision == HMM_PREC_TF32 ? 155 : 200};
+            case 32: return {strand_mma_per_warp(32), 8, 0, 480, precision == HMM_PREC_TF32 ? 300 : precision == HMM_PREC_BF16 ? 400 : 450};
+            case 48: return {strand_mma_per_warp(48), 8, 1, 2000, 1900};
+            case 64: return {strand_mma_per_warp(64), 8, 1, 3300, 3100};
+            default: return {strand_mma_per_warp(80), 8, 1, 4500, 4200};
+        }
+    }
     switch (KP) {
-        case 4: return {strand_simt_per_warp(4), 16, 110, 40};
-        case 8: return {strand_simt_per_warp(8), 12, 160, 60};
-        case 16: return {strand_simt_per_warp(16), 12, 190, 95};
-        case 32: return {strand_simt_per_warp(32), 8, 260, 170};
-        default: return {strand_simt_per_warp(64), 8, 300, 180};
+        case 4: return {strand_simt_per_warp(4), 16, 0, 150, 60};
+        case 8: return {strand_simt_per_warp(8), 12, 0, 230, 110};
+        case 16: return {strand_simt_per_warp(16), 12, 0, 300, 190};
+        case 32: return {strand_simt_per_warp(32), 8, 0, 400, 250};
+        default: return {strand_simt_per_warp(64), 8, 0, 430, 260};
     }
 }
 
-constexpr int STRAND_WARM = 256;        // covers the distance to meeting on tremor data (25 steps median, 200 at most)
-constexpr int STRAND_WARM_SHORT = 128;  // where a piece is short and the few that have not met can run on cheaply
-constexpr int STRAND_WARM_SPARSE = 512; // with the run-length option: rare tremors (260 steps median, 800 at most)
+// Warm-up steps. Vectors on tremor data meet after 25 steps at the median and
+// 200 at most; the join carries those that have not met at less than the cost
+// of a longer warm-up for all (K=32, 64 segments, 64 proposals: 1273 us at 128,
+// 1365 at 256; K=25, T=2^20, one chain: 119 us at 64, 131 at 128). With the
+// run-length option tremors are rare: 260 at the median, 800 at most.
+static int strand_warm(int L, bool sparse) { return sparse ? 512 : L <= 512 ? 64 : 128; }
 
-static int strand_warm(int L, bool sparse) {
-    return sparse ? STRAND_WARM_SPARSE : L <= 512 ? STRAND_WARM_SHORT : STRAND_WARM;
-}
-
-// Piece length for a batch: the smallest modelled time over lengths growing by
-// about an eighth. One wave of warps takes (warm + L) steps, at the latency of
-// a step while a scheduler holds few warps and at their issue time beyond.
-static int choose_strand_len(int KP, int n_prop, const std::vector<int64_t> &steps, bool sparse, int n_sms) {
-    const StrandCost c = strand_cost(KP);
-    int64_t longest = 0;
-    for (int64_t n : steps) longest = std::max(longest, n);
-    const int64_t Lmax = std::max<int64_t>(OBS_WIN, (longest + OBS_WIN - 1) / OBS_WIN * OBS_WIN);
-    double best = 0.0;
+// Piece length for a batch: the smallest modelled time over the lengths that
+// fill 1, 2, .. warps of a proposal (about an eighth more each beyond 32). One
+// wave of warps takes (warm + L) steps, at the latency of a step while a
+// scheduler holds few warps and at their issue time beyond.
+static int choose_strand_len(const StrandCost &c, int n_prop, const std::vector<int64_t> &steps, bool sparse, int n_sms,
+                             double &best) {
+    int64_t longest = 0, all = 0;
+    for (int64_t n : steps) {
+        longest = std::max(longest, n);
+        all += n;
+    }
+    const int64_t cap = (int64_t)n_sms * c.warps_per_sm;
     int64_t best_L = 0;
-    for (int64_t L = OBS_WIN;; L = std::min(Lmax, (L + L / 8 + OBS_WIN) / OBS_WIN * OBS_WIN)) {
+    for (int64_t w = 1;; w += 1 + w / 32) {
+        const int64_t slots = w * (c.fours ? 4 : 1) * c.per_warp;
+        const int64_t L = std::max<int64_t>(OBS_WIN, ((all + slots - 1) / slots + OBS_WIN - 1) / OBS_WIN * OBS_WIN);
         int64_t n = 0;
         for (int64_t m : steps) n += (m + L - 1) / L;
-        const int64_t warps = (int64_t)n_prop * ((n + c.per_warp - 1) / c.per_warp);
-        const int64_t cap = (int64_t)n_sms * c.warps_per_sm;
+        int64_t wpp = (n + c.per_warp - 1) / c.per_warp;
+        if (c.fours) wpp = (wpp + 3) / 4 * 4;
+        const int64_t warps = (int64_t)n_prop * wpp;
         const int64_t waves = std::max<int64_t>(1, (warps + cap - 1) / cap);
-        const int64_t resident = std::min(warps, cap);
-        const int64_t per_sched = (resident + 4 * n_sms - 1) / (4 * n_sms);
+        const int64_t per_sched = (std::min(warps, cap) + 4 * n_sms - 1) / (4 * n_sms);
         const double step = (double)std::max<int64_t>(c.latency, per_sched * c.issue);
         const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm((int)L, sparse)) * step;
         if (!best_L || t < best) {
             best = t;
             best_L = L;
         }
-        if (L >= Lmax) break;
+        if (L == OBS_WIN) break;
     }
     return (int)best_L;
 }
@@ -363,7 +378,8 @@ static int choose_strand_len(int KP, int n_prop, const std::vector<int64_t> &ste
 static void build_strands(Plan &pl, bool sparse, int n_sms) {
     pl.strands.clear();
     pl.strand_order.clear();
-    pl.strand_kp = strand_simt_kp(pl.K);
+    pl.strand_tensor = false;
+    pl.strand_kp = pl.precision == HMM_PREC_FP32_SIMT ? strand_simt_kp(pl.K) : pl.lay.KP;
     std::vector<int64_t> steps;
     for (int s = 0; s < pl.n_seg; ++s) steps.push_back(std::max<int64_t>(0, pl.offsets[s + 1] - pl.offsets[s] - 1));
     int64_t all = 0;
@@ -374,7 +390,24 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
         pl.strand_kp = 0;
         return;
     }
-    const int L = choose_strand_len(pl.strand_kp, pl.n_prop, steps, sparse, n_sms);
+    double cost = 0.0;
+    int L = 0;
+    if (pl.precision != HMM_PREC_FP32_SIMT) {
+        pl.strand_tensor = true;
+        L = choose_strand_len(strand_cost(true, pl.lay.KP, pl.precision), pl.n_prop, steps, sparse, n_sms, cost);
+    }
+    if (strand_simt_kp(pl.K)) {
+        // the CUDA cores' strands are quicker by the step: for a batch too
+        // small to fill the tensor cores' rows
+        double other = 0.0;
+        const int L2 = choose_strand_len(strand_cost(false, strand_simt_kp(pl.K), pl.precision), pl.n_prop, steps,
+                                         sparse, n_sms, other);
+        if (!L || other < cost) {
+            L = L2;
+            pl.strand_tensor = false;
+            pl.strand_kp = strand_simt_kp(pl.K);
+        }
+    }
     for (int s = 0; s < pl.n_seg; ++s) {
         // equal pieces of whole observation windows
         const int64_t wins = (steps[s] + OBS_WIN - 1) / OBS_WIN;
@@ -662,6 +695,8 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
         w->sp.ve = cv.take<float>(m * pl.strand_kp);
         w->sp.ex = cv.take<long long>(m);
         w->sp.logr = cv.take<double>(m);
+        w->sp.jump = cv.take<int>(m);
+        w->sp.jumps = cv.take<int>(n_prop);
     }
     w->packed = cv.take<float2>(pl.n_packed);
     w->head = cv.take<float2>(n_seg);
@@ -777,7 +812,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         if (r == cudaSuccess && T_total > 0) { r = launch_pack(n_seg, pl.d_offsets, pl.d_pbase, T_total, xy, tremor, packed, head, obs_bad, c->d_status, s); ++launches; }
         prof_mark(c, HMM_PHASE_CHUNK, s);
         if (r == cudaSuccess && sp.n > 0) {
-            r = launch_strand_simt(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
+            auto strands = pl.strand_tensor ? launch_strand_mma : launch_strand_simt;
+            r = strands(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
             if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, cblock, packed, sp, s);
             launches += 2;
         }

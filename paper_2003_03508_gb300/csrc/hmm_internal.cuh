@@ -40,8 +40,15 @@ enum {
     EM_QC = 4,   // -0.5 log2(e) sxx / det
     EM_CTR = 5,  // log2 p - log2(2 pi) - 0.5 log2 det
     EM_CNO = 6,  // log2 (1 - p)
-    EM_OFF = 7,  // [0], [1]: whole numbers next above the row maxima of EM_CTR and EM_CNO
     EM_ROWS = 8,
+    // the strands' form of the same density (hmm_strand.cuh)
+    EM_OFF = 8,  // [0], [1]: whole numbers next above the row maxima of EM_CTR and EM_CNO; [2], [3]: centre of the states
+    EM_UX = 9,   // u = ux x + uy y + u0, w = wy y + w0, x and y from the centre: log2 density = ctr - u^2 - w^2
+    EM_UY = 10,
+    EM_U0 = 11,
+    EM_WY = 12,
+    EM_W0 = 13,
+    EM_ALL = 14,
 };
 
 // a step whose best state has log2-emission below -EXP_LIMIT is not representable
@@ -84,14 +91,16 @@ struct StrandPtrs {
     float *vs = nullptr;       // [n_prop][n][KP] vector at the piece's start
     float *ve = nullptr;       // [n_prop][n][KP] vector at its end
     long long *ex = nullptr;   // [n_prop][n] power-of-two exponent of ve relative to vs
-    double *logr = nullptr;    // [n_prop][n] log scale of the true vector over vs at the piece's start
+    double *logr = nullptr;    // [n_prop][n] log scale of the true vector over the strand of piece `jump`
+    int *jump = nullptr;       // [n_prop][n] piece where the vectors met: itself, a later one, or -1 (at the segment's end)
+    int *jumps = nullptr;      // [n_prop] some piece's jump is not itself
     int *route = nullptr;      // [n_prop]
     int *todo = nullptr;       // [1 + n_prop]
 };
 
 struct ConstLayout {
     int KP;         // padded state count used by the chunk kernel
-    int off_emis;   // EM_ROWS * KP floats
+    int off_emis;   // EM_ALL * KP floats
     int off_p32;    // KP * KP floats, row-major, zero padded
     int off_tc;     // tensor-core B-operand images (path dependent)
     int tc_floats;  // size of the tensor-core section
@@ -166,6 +175,10 @@ int strand_simt_per_warp(int KP);
 cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                                const float *cblock, const float *pi, const float2 *head, const float2 *packed,
                                const StrandPtrs &sp, cudaStream_t st);
+int strand_mma_per_warp(int KP);
+cudaError_t launch_strand_mma(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+                              const float *cblock, const float *pi, const float2 *head, const float2 *packed,
+                              const StrandPtrs &sp, cudaStream_t st);
 cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
                         const float2 *packed, const StrandPtrs &sp, cudaStream_t st);
 

@@ -2,8 +2,10 @@
 // is not its segment's first compares the vector its strand had at the piece's
 // start, g, with the end of the strand before, a. If a = r g within the
 // tolerance in every entry, log r is noted. Otherwise both vectors run on
-// through the piece, with exact scaling, until they meet; a piece that ends
-// before they do sends its proposal to the chunk products.
+// through the piece, with exact scaling, until they meet. Where the piece ends
+// first, a goes on against the strand of the next piece, and the pieces passed
+// over are taken from it (jump); after JOIN_MOST steps the proposal is sent to
+// the chunk products.
 //
 // Nearly every piece meets at once (the warm-up covers the usual distance), so
 // the kernel reads 2 KP floats a piece; the rest are a few hundred steps of
@@ -17,6 +19,7 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr float JOIN_TINY = 8.470329472543003e-22f;  // 2^-70: an entry this far below the largest cannot matter (PMIN)
 constexpr int JOIN_WARPS = 4;
+constexpr int JOIN_MOST = 2048;
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
@@ -44,10 +47,13 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
     const long long id = (long long)blockIdx.x * JOIN_WARPS + warp;
     const int q = (int)(id / sp.n), s = (int)(id % sp.n);
     if (q >= n_prop || __shfl_sync(FULL, sp.route[q], 0) != ROUTE_STRANDS) return;
-    const StrandDesc d = sp.desc[s];
+    StrandDesc d = sp.desc[s];
     const size_t idx = (size_t)q * sp.n + s;
     if (d.flags & SD_FIRST) {
-        if (lane == 0) sp.logr[idx] = 0.0;
+        if (lane == 0) {
+            sp.logr[idx] = 0.0;
+            sp.jump[idx] = s;
+        }
         return;
     }
     float a[NC], g[NC];
@@ -70,8 +76,11 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
         hi = warp_max(hi);
         return hi <= lo * (1.0f + tol);  // false for NaN
     };
-    int ea = 0, eg = 0;  // exponents gathered while running on (both in [1, 2) at the start)
-    long long de = 0;
+    int ea = 0, eg = 0;  // exponents gathered while running on: a's from this piece's start, g's from piece `at`'s
+    long long xa = 0, xg = 0;  // their sums
+    long long off = 0;  // whole offsets of the current piece's steps: common to both vectors
+    int at = s;
+    bool over = false;  // the segment ended before the vectors met
     bool ok = met();
     if (!ok) {
         const float *cb = cblock + (size_t)q * lay.stride;
@@ -95,8 +104,8 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
             }
         }
         float c[NC][7];
-        float offt, offn;
-        strand_offsets(em, KPl, offt, offn);
+        const float offt = em[EM_OFF * KPl], offn = em[EM_OFF * KPl + 1];
+        const int ct = (int)offt, cn = (int)offn;
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
             const int k = lane + 32 * n;
@@ -157,19 +166,39 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
             ma = warp_max(ma);
             mg = warp_max(mg);
             if (!(ma >= STRAND_SHRINK && mg >= STRAND_SHRINK && ma <= STRAND_GROW && mg <= STRAND_GROW)) return false;
-            const int xa = float_exponent(ma), xg = float_exponent(mg);
-            const float fa = pow2f(-xa), fg = pow2f(-xg);
+            const int pa = float_exponent(ma), pg = float_exponent(mg);
+            const float fa = pow2f(-pa), fg = pow2f(-pg);
 #pragma unroll
             for (int n = 0; n < NC; ++n) {
                 a[n] *= fa;
                 g[n] *= fg;
             }
-            ea += xa;
-            eg += xg;
+            ea += pa;
+            eg += pg;
             return true;
         };
         bool alive = true;
-        for (int t0 = 0; t0 < d.len && !ok && alive; t0 += 32) {
+        int t0 = 0;
+        for (int done = 0; !ok && alive && done < JOIN_MOST; done += 32, t0 += 32) {
+            if (t0 >= d.len) {
+                // this piece is over: on against the next one's strand
+                xa += off;
+                off = xg = 0;
+                if (d.flags & SD_LAST) {
+                    over = true;
+                    break;
+                }
+                ++at;
+                d = sp.desc[at];
+                t0 = 0;
+#pragma unroll
+                for (int n = 0; n < NC; ++n) {
+                    const int k = lane + 32 * n;
+                    g[n] = k < K ? sp.vs[((size_t)q * sp.n + at) * KP + k] : 0.0f;
+                }
+                ok = met();
+                if (ok) break;
+            }
             // 32 steps' observations, one per lane (the packed sequence is padded to whole windows)
             const float2 ob = packed[d.pstart + t0 + lane];
             for (int t = t0; t < min(t0 + 32, d.len) && !ok && alive; t += 4) {
@@ -181,11 +210,13 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                     kg[n] = g[n];
                 }
                 bool fine = m == 4;
+                int o4 = 0;
                 if (fine) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float x = __shfl_sync(FULL, ob.x, t - t0 + j), y = __shfl_sync(FULL, ob.y, t - t0 + j);
                         float f[NC];
+                        o4 += isnan(x) ? cn : ct;
 #pragma unroll
                         for (int n = 0; n < NC; ++n) f[n] = ex2(emission(n, x, y));
                         step(f);
@@ -193,6 +224,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                     fine = rescale();
                 }
                 if (!fine) {
+                    o4 = 0;
                     // step by step with exact scaling (as in the strands)
 #pragma unroll
                     for (int n = 0; n < NC; ++n) {
@@ -210,15 +242,18 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                         mx = warp_max(mx);
                         alive = mx + (isnan(x) ? offn : offt) >= -(float)EXP_LIMIT;
                         const float fm = alive ? floorf(mx) : 0.0f;
+                        o4 += (int)fm + (isnan(x) ? cn : ct);
 #pragma unroll
                         for (int n = 0; n < NC; ++n) f[n] = ex2(f[n] - fm);
                         step(f);
                         alive = alive && rescale();
                     }
                 }
+                off += o4;
                 ok = alive && met();
             }
-            de += (long long)ea - eg;
+            xa += ea;
+            xg += eg;
             ea = eg = 0;
         }
     }
@@ -231,8 +266,13 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
     sa = warp_sum(sa);
     sg = warp_sum(sg);
     if (lane == 0) {
-        if (ok) sp.logr[idx] = log(sa / sg) + 0.69314718055994530942 * (double)(de + ea - eg);
-        else send_to_chunks(sp, q);
+        if (ok || over) {
+            sp.logr[idx] = log(ok ? sa / sg : sa) + 0.69314718055994530942 * (double)(xa - xg);
+            sp.jump[idx] = ok ? at : -1;
+            if (at != s || over) sp.jumps[q] = 1;
+        } else {
+            send_to_chunks(sp, q);
+        }
     }
 }
 
@@ -241,9 +281,11 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
 cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
                         const float2 *packed, const StrandPtrs &sp, cudaStream_t st) {
     if (sp.n == 0) return cudaSuccess;
-    // FP32 vectors that have met differ by their rounding only, a few 2^-20
+    // FP32 vectors that have met differ by their rounding only, a few 2^-20.
+    // Vectors carried with TF32 operands differ by more, and run on here, in
+    // FP32, for the ten or twenty steps that take the difference away.
     const float tol = 3.0517578125e-5f;  // 2^-15
-    const bool rt = precision == HMM_PREC_TF32;
+    const bool rt = precision == HMM_PREC_TF32;  // P as the strands have it
     const long long warps = (long long)n_prop * sp.n;
     const unsigned grid = (unsigned)((warps + JOIN_WARPS - 1) / JOIN_WARPS);
     if (KP <= 32) join_kernel<1><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);

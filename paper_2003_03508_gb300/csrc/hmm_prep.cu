@@ -27,7 +27,7 @@ ConstLayout make_layout(int K, int precision) {
     }
     L.KP = KP;
     L.off_emis = 0;
-    L.off_p32 = round_up(EM_ROWS * KP, 32);
+    L.off_p32 = round_up(EM_ALL * KP, 32);
     L.off_tc = round_up(L.off_p32 + KP * KP, 32);
     switch (precision) {
         case HMM_PREC_TF32: L.tc_floats = KP * KP; break;            // P_hi (tf32)
@@ -67,7 +67,24 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
     cov += (size_t)q * 3 * K;
     float *cb = cblock + (size_t)q * lay.stride;
     __shared__ int bad, small;
+    __shared__ float centre[2];
     if (threadIdx.x == 0) bad = small = 0;
+    if (threadIdx.x < 32) {
+        // the states' centre: the strands take coordinates from it
+        float sx = 0.0f, sy = 0.0f;
+        for (int k = threadIdx.x; k < K; k += 32) {
+            sx += mu[2 * k] / (float)K;
+            sy += mu[2 * k + 1] / (float)K;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        }
+        if (threadIdx.x == 0) {
+            centre[0] = sx;
+            centre[1] = sy;
+        }
+    }
     __syncthreads();
 
     // rows of P: non-negative, finite, summing to 1 within 1e-5
@@ -97,6 +114,7 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
     for (int k = threadIdx.x; k < KP; k += blockDim.x) {
         float mx = 0.f, my = 0.f, qa = 0.f, qb = 0.f, qc = 0.f;
         float ctr = -INFINITY, cno = -INFINITY;
+        double ux = 0.0, uy = 0.0, u0 = 0.0, wy = 0.0, w0 = 0.0;
         if (k < K) {
             double pk = p[k];
             double sxx = cov[3 * k], sxy = cov[3 * k + 1], syy = cov[3 * k + 2];
@@ -114,6 +132,13 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
                 qc = (float)(-0.5 * LOG2E * sxx / det);
                 ctr = (float)(log2(pk) - LOG2_2PI - 0.5 * log2(det));
                 cno = (float)log2(1.0 - pk);
+                // the quadratic form as two squares (Cholesky factor of the precision matrix)
+                ux = sqrt(0.5 * LOG2E * syy / det);
+                uy = -ux * sxy / syy;
+                wy = sqrt(0.5 * LOG2E / syy);
+                const double cx = (double)mx - centre[0], cy = (double)my - centre[1];
+                u0 = -(ux * cx + uy * cy);
+                w0 = -wy * cy;
             }
         }
         float *em = cb + lay.off_emis;
@@ -124,6 +149,11 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
         em[EM_QC * KP + k] = qc;
         em[EM_CTR * KP + k] = ctr;
         em[EM_CNO * KP + k] = cno;
+        em[EM_UX * KP + k] = (float)ux;
+        em[EM_UY * KP + k] = (float)uy;
+        em[EM_U0 * KP + k] = (float)u0;
+        em[EM_WY * KP + k] = (float)wy;
+        em[EM_W0 * KP + k] = (float)w0;
     }
     // P padded to KP x KP (FP32, row-major) and the tensor-core images
     for (int idx = threadIdx.x; idx < KP * KP; idx += blockDim.x) {
@@ -162,12 +192,15 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
             mn = isfinite(mn) ? ceilf(mn) : 0.0f;
             em[EM_OFF * KP] = mt;
             em[EM_OFF * KP + 1] = mn;
+            em[EM_OFF * KP + 2] = centre[0];
+            em[EM_OFF * KP + 3] = centre[1];
             prop_bad[q] = bad;
             if (bad) atomicOr(status, ST_EINVAL);
             if (sp.route) {
                 // strands need P's entries above STRAND_PMIN and constants of ordinary size
                 const bool fits = !small && fabsf(mt) <= 1000.0f && fabsf(mn) <= 1000.0f;
                 sp.route[q] = bad ? ROUTE_BAD : ROUTE_STRANDS;
+                sp.jumps[q] = 0;
                 if (!bad && !fits) {
                     sp.route[q] = ROUTE_CHUNKS;
                     sp.todo[1 + atomicAdd(&sp.todo[0], 1)] = q;

@@ -1,5 +1,6 @@
-// Strands on the CUDA cores (FP32): every precision for few long chains, and
-// HMM_PREC_FP32_SIMT for batches. See hmm_strand.cuh for the method.
+// Strands on the CUDA cores (FP32): HMM_PREC_FP32_SIMT, and the other precisions
+// where the batch has too few strands for the tensor cores' rows (with P rounded
+// to TF32 for HMM_PREC_TF32). See hmm_strand.cuh for the method.
 //
 // A strand is carried by G threads. Each holds the four columns of P it is
 // responsible for (KP / H of their rows) in registers, as pairs over the row
@@ -79,12 +80,12 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
             }
             p[c][i] = pack2(v[0], v[1]);
         }
-    float offt, offn;
-    strand_offsets(em, KPl, offt, offn);
-    const int ct = (int)offt, cn = (int)offn;
+    StrandBase base;
+    base.load(em, KPl);
+    const int ct = (int)base.offt, cn = (int)base.offn;
     Emis2 ec[NS / 2];
 #pragma unroll
-    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u, offt, offn);
+    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u, base.offt, base.offn);
 
     // this thread's strands
     const float4 *obs[R];
@@ -112,7 +113,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
         const bool tr = !isnan(o.x);
         float l[NS], m = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < NS / 2; ++u) ec[u].eval(o.x, o.y, tr, l[2 * u], l[2 * u + 1]);
+        for (int u = 0; u < NS / 2; ++u) ec[u].eval(o.x - base.cx, o.y - base.cy, tr, l[2 * u], l[2 * u + 1]);
 #pragma unroll
         for (int u = 0; u < NS; ++u) {
             const int k = own + u;
@@ -132,7 +133,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
 #pragma unroll
         for (int o = 1; o < G; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
         if (at_head) {
-            if (m + (tr ? offt : offn) >= -(float)EXP_LIMIT) {
+            if (m + base.off(tr) >= -(float)EXP_LIMIT) {
                 const float fm = floorf(m);
                 e32[r] = (int)fm + (tr ? ct : cn);
 #pragma unroll
@@ -175,8 +176,11 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
                     a = t.x;
                     b = t.y;
                 }
+                // a and b each four times in a row: their registers are read once
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[c] = fma2(b, p[c][2 * i + 1], fma2(a, p[c][2 * i], acc[c]));
+                for (int c = 0; c < 4; ++c) acc[c] = fma2(a, p[c][2 * i], acc[c]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[c] = fma2(b, p[c][2 * i + 1], acc[c]);
             }
             float s[4];
 #pragma unroll
@@ -213,6 +217,11 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
         for (int r = 0; r < R; ++r) {
             ox[r][0] = na[r].x; oy[r][0] = na[r].y; ox[r][1] = na[r].z; oy[r][1] = na[r].w;
             ox[r][2] = nb[r].x; oy[r][2] = nb[r].y; ox[r][3] = nb[r].z; oy[r][3] = nb[r].w;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                ox[r][j] -= base.cx;
+                oy[r][j] -= base.cy;
+            }
             if (4 * (w + 1) < total[r]) {
                 na[r] = obs[r][2 * (w + 1)];
                 nb[r] = obs[r][2 * (w + 1) + 1];
@@ -275,7 +284,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
                     for (int u = 0; u < NS; ++u) m = fmaxf(m, l[u]);
 #pragma unroll
                     for (int o = 1; o < G; o <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
-                    const bool emits = m + (tr ? offt : offn) >= -(float)EXP_LIMIT;
+                    const bool emits = m + base.off(tr) >= -(float)EXP_LIMIT;
                     const float fm = emits ? floorf(m) : 0.0f;
                     float z[NS], mx = 0.0f;
 #pragma unroll

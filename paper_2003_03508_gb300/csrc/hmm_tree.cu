@@ -228,16 +228,33 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
     // before; a segment's last one the sum of its vector as well
     const bool strands = sp.route && sp.route[q] == ROUTE_STRANDS;
     if (strands) {
-        double part = 0.0;
-        for (int i = tid; i < sp.n; i += FINAL_THREADS) {
-            const size_t idx = (size_t)q * sp.n + i;
-            double v = (double)sp.ex[idx] * LN2 + sp.logr[idx];
-            if (sp.desc[i].flags & SD_LAST) {
+        // piece i, with the exponents and, if it is the last, the vector of strand e
+        auto piece = [&](int i, int e) {
+            const size_t at = (size_t)q * sp.n + e;
+            double v = (double)sp.ex[at] * LN2 + sp.logr[(size_t)q * sp.n + i];
+            if (sp.desc[e].flags & SD_LAST) {
                 double a = 0.0;
-                for (int k = 0; k < K; ++k) a += (double)sp.ve[idx * strand_kp + k];
+                for (int k = 0; k < K; ++k) a += (double)sp.ve[at * strand_kp + k];
                 v += log(a);
             }
-            part += v;
+            return v;
+        };
+        double part = 0.0;
+        if (!sp.jumps[q]) {
+            for (int i = tid; i < sp.n; i += FINAL_THREADS) part += piece(i, i);
+        } else if (tid == 0) {
+            // some pieces are passed over: in order
+            for (int i = 0; i < sp.n;) {
+                const int j = sp.jump[(size_t)q * sp.n + i];
+                if (j >= 0) {
+                    part += piece(i, j);
+                    i = j + 1;
+                } else {
+                    part += sp.logr[(size_t)q * sp.n + i];
+                    while (!(sp.desc[i].flags & SD_LAST)) ++i;
+                    ++i;
+                }
+            }
         }
         total = block_sum_fixed(part, red);
     }
