@@ -313,16 +313,17 @@ static bool tune_entry_valid(const TuneEntry &e) {
 // and when others fill it (issue).
 struct StrandCost {
     int per_warp, warps_per_sm, fours, latency, issue;
+    bool tensor = false;
 };
 
 static StrandCost strand_cost(bool tensor, int KP, int precision) {
     if (tensor) {
         switch (KP) {
-            case 16: return {strand_mma_per_warp(16), 16, 0, 330, precision == HMM_PREC_TF32 ? 155 : 200};
-            case 32: return {strand_mma_per_warp(32), 8, 0, 480, precision == HMM_PREC_TF32 ? 300 : precision == HMM_PREC_BF16 ? 400 : 450};
-            case 48: return {strand_mma_per_warp(48), 8, 1, 2000, 1900};
-            case 64: return {strand_mma_per_warp(64), 8, 1, 3300, 3100};
-            default: return {strand_mma_per_warp(80), 8, 1, 4500, 4200};
+            case 16: return {strand_mma_per_warp(16), 16, 0, 330, precision == HMM_PREC_TF32 ? 155 : 200, true};
+            case 32: return {strand_mma_per_warp(32), 8, 0, 480, precision == HMM_PREC_TF32 ? 300 : precision == HMM_PREC_BF16 ? 400 : 450, true};
+            case 48: return {strand_mma_per_warp(48), 8, 1, 2000, 1900, true};
+            case 64: return {strand_mma_per_warp(64), 8, 1, 3300, 3100, true};
+            default: return {strand_mma_per_warp(80), 8, 1, 4500, 4200, true};
         }
     }
     switch (KP) {
@@ -339,7 +340,7 @@ static StrandCost strand_cost(bool tensor, int KP, int precision) {
 // of a longer warm-up for all (K=32, 64 segments, 64 proposals: 1273 us at 128,
 // 1365 at 256; K=25, T=2^20, one chain: 119 us at 64, 131 at 128). With the
 // run-length option tremors are rare: 260 at the median, 800 at most.
-static int strand_warm(int L, bool sparse) { return sparse ? 512 : L <= 512 ? 64 : 128; }
+static int strand_warm(int L, bool sparse, bool tensor) { return sparse ? 512 : L <= 512 && !tensor ? 64 : 128; }
 
 // Piece length for a batch: the smallest modelled time over the lengths that
 // fill 1, 2, .. warps of a proposal (about an eighth more each beyond 32). One
@@ -365,7 +366,7 @@ static int choose_strand_len(const StrandCost &c, int n_prop, const std::vector<
         const int64_t waves = std::max<int64_t>(1, (warps + cap - 1) / cap);
         const int64_t per_sched = (std::min(warps, cap) + 4 * n_sms - 1) / (4 * n_sms);
         const double step = (double)std::max<int64_t>(c.latency, per_sched * c.issue);
-        const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm((int)L, sparse)) * step;
+        const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm((int)L, sparse, c.tensor)) * step;
         if (!best_L || t < best) {
             best = t;
             best_L = L;
@@ -414,7 +415,7 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
         const int64_t n = (steps[s] + L - 1) / L;
         for (int64_t i = 0; i < n; ++i) {
             const int64_t a = wins * i / n * OBS_WIN, b = std::min(steps[s], wins * (i + 1) / n * OBS_WIN);
-            const int64_t warm = std::min<int64_t>(a, strand_warm(L, sparse));
+            const int64_t warm = std::min<int64_t>(a, strand_warm(L, sparse, pl.strand_tensor));
             StrandDesc d;
             d.pstart = pl.pbase[s] + a;
             d.len = (int32_t)(b - a);
@@ -814,7 +815,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         if (r == cudaSuccess && sp.n > 0) {
             auto strands = pl.strand_tensor ? launch_strand_mma : launch_strand_simt;
             r = strands(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
-            if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, cblock, packed, sp, s);
+            if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, pl.strand_tensor, cblock, packed, sp, s);
             launches += 2;
         }
         if (r == cudaSuccess && pl.n_chunks > 0) {

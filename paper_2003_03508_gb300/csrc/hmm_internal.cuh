@@ -179,7 +179,7 @@ int strand_mma_per_warp(int KP);
 cudaError_t launch_strand_mma(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                               const float *cblock, const float *pi, const float2 *head, const float2 *packed,
                               const StrandPtrs &sp, cudaStream_t st);
-cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
+cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, bool tensor, const float *cblock,
                         const float2 *packed, const StrandPtrs &sp, cudaStream_t st);
 
 // The chunk-product kernels and the tree take a list of the proposals to work

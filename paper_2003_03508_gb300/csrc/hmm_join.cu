@@ -20,6 +20,7 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr float JOIN_TINY = 8.470329472543003e-22f;  // 2^-70: an entry this far below the largest cannot matter (PMIN)
 constexpr int JOIN_WARPS = 4;
 constexpr int JOIN_MOST = 2048;
+constexpr float JOIN_TOL = 3.0517578125e-5f;  // 2^-15: what FP32 vectors run on to
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
@@ -40,7 +41,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // NC: states per lane (KP <= 32 NC)
 template <int NC>
 __global__ void __launch_bounds__(32 * JOIN_WARPS)
-join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float tol, const float *__restrict__ cblock,
+join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float tol0, const float *__restrict__ cblock,
             const float2 *__restrict__ packed, StrandPtrs sp) {
     __shared__ __align__(16) float2 sag[JOIN_WARPS][32 * NC];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -63,7 +64,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
         a[c] = k < K ? sp.ve[(idx - 1) * KP + k] : 0.0f;
         g[c] = k < K ? sp.vs[idx * KP + k] : 0.0f;
     }
-    auto met = [&]() {
+    auto met = [&](float tol) {
         float lo = INFINITY, hi = 0.0f;
 #pragma unroll
         for (int c = 0; c < NC; ++c)
@@ -81,7 +82,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
     long long off = 0;  // whole offsets of the current piece's steps: common to both vectors
     int at = s;
     bool over = false;  // the segment ended before the vectors met
-    bool ok = met();
+    bool ok = met(tol0);
     if (!ok) {
         const float *cb = cblock + (size_t)q * lay.stride;
         const float *em = cb + lay.off_emis;
@@ -196,7 +197,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                     const int k = lane + 32 * n;
                     g[n] = k < K ? sp.vs[((size_t)q * sp.n + at) * KP + k] : 0.0f;
                 }
-                ok = met();
+                ok = met(JOIN_TOL);
                 if (ok) break;
             }
             // 32 steps' observations, one per lane (the packed sequence is padded to whole windows)
@@ -250,7 +251,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                     }
                 }
                 off += o4;
-                ok = alive && met();
+                ok = alive && met(JOIN_TOL);
             }
             xa += ea;
             xg += eg;
@@ -278,13 +279,16 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
 
 }  // namespace
 
-cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, const float *cblock,
+cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, bool tensor, const float *cblock,
                         const float2 *packed, const StrandPtrs &sp, cudaStream_t st) {
     if (sp.n == 0) return cudaSuccess;
-    // FP32 vectors that have met differ by their rounding only, a few 2^-20.
-    // Vectors carried with TF32 operands differ by more, and run on here, in
-    // FP32, for the ten or twenty steps that take the difference away.
-    const float tol = 3.0517578125e-5f;  // 2^-15
+    // Vectors that have met differ by the rounding of their strands: a few
+    // 2^-20 in FP32, 2^-11 with TF32 operands, 2^-16 with BF16 hi + lo. What is
+    // taken as met at a piece's start is wider by eight; the ratio of the sums
+    // then carries the rounding of one step, where the piece has that of 64 and
+    // more. The rest runs on in FP32 to JOIN_TOL (K=80 BF16, 32 proposals:
+    // 1000 us when every boundary had to).
+    const float tol = !tensor ? JOIN_TOL : precision == HMM_PREC_BF16 ? 2.44140625e-4f : 3.90625e-3f;
     const bool rt = precision == HMM_PREC_TF32;  // P as the strands have it
     const long long warps = (long long)n_prop * sp.n;
     const unsigned grid = (unsigned)((warps + JOIN_WARPS - 1) / JOIN_WARPS);
