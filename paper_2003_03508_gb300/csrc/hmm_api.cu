@@ -31,7 +31,7 @@ struct DevBuf {
 };
 
 struct Plan {
-    bool valid = false, sparse = false;
+    bool valid = false, sparse = false, smooth = false;
     int K = 0, n_prop = 0, n_seg = 0, precision = -1, L = 0;
     std::vector<int64_t> offsets;
     // derived
@@ -46,6 +46,7 @@ struct Plan {
     std::vector<ChunkDesc> chunks;
     int strand_kp = 0;                      // 0: this shape runs on chunk products alone
     bool strand_tensor = false;             // strands on the tensor cores
+    int strand_warm = 0;
     std::vector<StrandDesc> strands;
     std::vector<int32_t> strand_order;      // longest first
     // device copies (inside plan_buf)
@@ -393,7 +394,11 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     }
     double cost = 0.0;
     int L = 0;
-    if (pl.precision != HMM_PREC_FP32_SIMT) {
+    if (pl.smooth && !strand_simt_kp(pl.K)) {
+        pl.strand_kp = 0;
+        return;
+    }
+    if (pl.precision != HMM_PREC_FP32_SIMT && !pl.smooth) {
         pl.strand_tensor = true;
         L = choose_strand_len(strand_cost(true, pl.lay.KP, pl.precision), pl.n_prop, steps, sparse, n_sms, cost);
     }
@@ -409,13 +414,17 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
             pl.strand_kp = strand_simt_kp(pl.K);
         }
     }
+    // every row of a posterior is used: pieces and warm-ups long enough that the
+    // vectors have met before a piece ends
+    if (pl.smooth) L = std::max(L, 128);
+    pl.strand_warm = pl.smooth ? 128 : strand_warm(L, sparse, pl.strand_tensor);
     for (int s = 0; s < pl.n_seg; ++s) {
         // equal pieces of whole observation windows
         const int64_t wins = (steps[s] + OBS_WIN - 1) / OBS_WIN;
         const int64_t n = (steps[s] + L - 1) / L;
         for (int64_t i = 0; i < n; ++i) {
             const int64_t a = wins * i / n * OBS_WIN, b = std::min(steps[s], wins * (i + 1) / n * OBS_WIN);
-            const int64_t warm = std::min<int64_t>(a, strand_warm(L, sparse, pl.strand_tensor));
+            const int64_t warm = std::min<int64_t>(a, pl.strand_warm);
             StrandDesc d;
             d.pstart = pl.pbase[s] + a;
             d.len = (int32_t)(b - a);
@@ -433,7 +442,7 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
 }
 
 static void build_plan(Plan &pl, int K, int n_prop, int n_seg, const int64_t *offs, int precision,
-                       int L, bool sparse, int n_sms) {
+                       int L, bool sparse, bool smooth, int n_sms) {
     pl.K = K;
     pl.n_prop = n_prop;
     pl.n_seg = n_seg;
@@ -502,13 +511,14 @@ static void build_plan(Plan &pl, int K, int n_prop, int n_seg, const int64_t *of
     }
     pl.n_levels = level;
     pl.sparse = sparse;
+    pl.smooth = smooth;
     build_strands(pl, sparse, n_sms);
     pl.valid = true;
 }
 
 static bool plan_matches(const Plan &pl, int K, int n_prop, int n_seg, const int64_t *offs,
-                         int precision, int L, bool sparse) {
-    if (!pl.valid || pl.sparse != sparse || pl.K != K || pl.n_prop != n_prop || pl.n_seg != n_seg ||
+                         int precision, int L, bool sparse, bool smooth) {
+    if (!pl.valid || pl.sparse != sparse || pl.smooth != smooth || pl.K != K || pl.n_prop != n_prop || pl.n_seg != n_seg ||
         pl.precision != precision || pl.L != L)
         return false;
     return std::equal(pl.offsets.begin(), pl.offsets.end(), offs);
@@ -711,13 +721,21 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
     return cv.off;
 }
 
-// The batched likelihood. With `products` every proposal's chunk products are
-// left in the workspace (level 0), as the boundary scans of the posterior and
-// of Viterbi read them; without, log L comes from strands where they apply.
+// What a call of the likelihood path is for. LOGLIK: log L, by strands where
+// they apply. PRODUCTS: every proposal's chunk products as well, left in the
+// workspace (level 0) for the boundary scans of Viterbi. SMOOTH: the posterior
+// and the statistics of one sequence too (`out2`), by strands or, where these
+// do not apply, by scans over the chunk products.
+enum class Mode { LOGLIK, PRODUCTS, SMOOTH };
+struct SmoothOut {
+    float *gamma;
+    double *stats;
+};
+
 static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, const float *P,
                           const float *p, const float *mu, const float *cov, int32_t n_seg,
                           const int64_t *offs, const float *xy, const uint8_t *tremor,
-                          const hmm_opts *opts_in, double *out, bool products, void *stream) {
+                          const hmm_opts *opts_in, double *out, Mode mode, const SmoothOut *out2, void *stream) {
     if (!c) return HMM_EINVAL;
     c->last_launches = 0;
     hmm_opts opts;
@@ -767,8 +785,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         L = tune_get(key);
         if (!L) L = choose_chunk_len(prec, n_prop, lay.KP, steps_total, c->n_sms);
     }
-    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0)) {
-        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, c->n_sms);
+    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode == Mode::SMOOTH)) {
+        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode == Mode::SMOOTH, c->n_sms);
         if (c->plan.n_levels + 1 > MAX_LEVELS) {
             c->plan.valid = false;
             return fail(c, HMM_EINVAL, "too many chunks for the tree (raise chunk_len)");
@@ -799,8 +817,43 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
     // strands first; `todo` lists what is left to the chunk products (null: everything)
-    const StrandPtrs sp = products ? StrandPtrs{} : wp.sp;
+    const StrandPtrs sp = mode == Mode::PRODUCTS ? StrandPtrs{} : wp.sp;
     const int *todo = sp.todo;
+    SmoothPtrs sm;
+    float *fvec = nullptr, *bvec = nullptr;
+    double *scan_part = nullptr, *scan_g0 = nullptr;
+    if (mode == Mode::SMOOTH) {
+        auto carve = [&](void *base) {
+            Carve cv(base);
+            const size_t C = std::max(1, pl.n_chunks), T = (size_t)T_total, n = (size_t)sp.n, kp = (size_t)pl.strand_kp;
+            const size_t part = out2->stats ? (size_t)K * K + 7 * K : 0;
+            fvec = cv.take<float>(C * KP);
+            bvec = cv.take<float>(C * KP);
+            scan_part = cv.take<double>(C * part);
+            scan_g0 = cv.take<double>(part ? K : 0);
+            if (n) {
+                sm.alpha = cv.take<float>(T * kp);
+                sm.u = part ? cv.take<float>(T * kp) : nullptr;
+                sm.bs = cv.take<float>(n * kp);
+                sm.be = cv.take<float>(n * kp);
+                sm.carry = cv.take<float>(n * kp);
+                sm.unmet = cv.take<int>(n);
+                sm.part = cv.take<double>(SMOOTH_PARTS * part);
+                sm.g0 = cv.take<double>(part ? K : 0);
+            }
+            return cv.off;
+        };
+        rc = ensure(c, c->fb, carve(nullptr) + 256);
+        if (rc) return rc;
+        carve(c->fb.p);
+        sm.warm = pl.strand_warm;
+        sm.gamma = out2->gamma;
+        sm.stats = out2->stats;
+        if (!out2->stats) {
+            scan_part = scan_g0 = nullptr;
+            sm.part = sm.g0 = nullptr;
+        }
+    }
 
     // ---- launches ----
     // The whole sequence, on stream `s` (the caller's, or the capture stream).
@@ -813,10 +866,14 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         if (r == cudaSuccess && T_total > 0) { r = launch_pack(n_seg, pl.d_offsets, pl.d_pbase, T_total, xy, tremor, packed, head, obs_bad, c->d_status, s); ++launches; }
         prof_mark(c, HMM_PHASE_CHUNK, s);
         if (r == cudaSuccess && sp.n > 0) {
-            auto strands = pl.strand_tensor ? launch_strand_mma : launch_strand_simt;
-            r = strands(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
+            if (pl.strand_tensor) r = launch_strand_mma(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
+            else r = launch_strand_simt(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, sm.alpha, s);
             if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, pl.strand_tensor, cblock, packed, sp, s);
             launches += 2;
+            if (r == cudaSuccess && sm.alpha) {
+                r = launch_smooth(K, pl.strand_kp, steps_total, lay, cblock, head, packed, sp, sm, s);
+                launches += 5 + (sm.stats ? 2 : 0);
+            }
         }
         if (r == cudaSuccess && pl.n_chunks > 0) {
             if (min_run) {
@@ -841,6 +898,12 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             r = launch_final(n_prop, K, opts.init_mode, n_seg, pl.d_segs, head, lv, KP, pi, P, p, mu, cov, prop_bad, obs_bad, out, sp, pl.strand_kp, s);
             ++launches;
         }
+        if (r == cudaSuccess && mode == Mode::SMOOTH) {
+            r = launch_posterior(K, KP, opts.init_mode, pl.n_chunks, L, pl.d_chunks, pi, P, cblock + lay.off_emis, head,
+                                 packed, lv.A[0], (const int32_t *)lv.e[0], fvec, bvec, out2->gamma, scan_part, scan_g0,
+                                 out2->stats, todo, s);
+            launches += 1 + (pl.n_chunks > 0 ? 1 : 0) + (out2->stats && pl.n_chunks > 0 ? 1 : 0);
+        }
         prof_mark(c, HMM_PHASE_COUNT, s);
         return r;
     };
@@ -856,7 +919,9 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             (uint64_t)(uintptr_t)cov, (uint64_t)(uintptr_t)xy, (uint64_t)(uintptr_t)tremor, (uint64_t)(uintptr_t)out,
             (uint64_t)(uintptr_t)c->work.p, c->plan_version, (uint64_t)n_prop, (uint64_t)K, (uint64_t)n_seg,
             (uint64_t)prec, (uint64_t)opts.init_mode, (uint64_t)renorm, (uint64_t)min_run, (uint64_t)L,
-            (uint64_t)T_total, (uint64_t)products};
+            (uint64_t)T_total, (uint64_t)mode,
+            (uint64_t)(uintptr_t)c->fb.p, (uint64_t)(uintptr_t)(out2 ? out2->gamma : nullptr),
+            (uint64_t)(uintptr_t)(out2 ? out2->stats : nullptr)};
         if (c->call_exec && c->call_key == key) {
             e = cudaGraphLaunch(c->call_exec, st);
             if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphLaunch");
@@ -919,7 +984,7 @@ int hmm_loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi, c
                        const float *p, const float *mu, const float *cov, int32_t n_seg,
                        const int64_t *offs, const float *xy, const uint8_t *tremor,
                        const hmm_opts *opts, double *out, void *stream) {
-    return loglik_batched(c, n_prop, K, pi, P, p, mu, cov, n_seg, offs, xy, tremor, opts, out, false, stream);
+    return loglik_batched(c, n_prop, K, pi, P, p, mu, cov, n_seg, offs, xy, tremor, opts, out, Mode::LOGLIK, nullptr, stream);
 }
 
 int hmm_loglik(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm_opts *opts,
@@ -947,32 +1012,9 @@ static int posterior_impl(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs,
         const int64_t Lp = ((int64_t)std::sqrt(3.0 * (double)obs->T) + OBS_WIN - 1) / OBS_WIN * OBS_WIN;
         o.chunk_len = (int32_t)std::min<int64_t>(16384, std::max<int64_t>(OBS_WIN, Lp));
     }
-    // the likelihood path computes the chunk products (and log L)
-    int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
-                                obs->tremor, &o, loglik, true, stream);
-    if (rc) return rc;
-    const Plan &pl = c->plan;
-    const int K = prm->K, KP = pl.lay.KP, C = std::max(1, pl.n_chunks);
-    WorkPtrs wp;
-    carve_work(c->work.p, 1, 1, pl.lay, pl, &wp);
-    size_t fb_bytes = sizeof(float) * 2 * (size_t)C * KP + 256;
-    if (stats) fb_bytes += sizeof(double) * ((size_t)C * (K * K + 7 * K) + K) + 256;
-    rc = ensure(c, c->fb, fb_bytes);
-    if (rc) return rc;
-    float *fvec = (float *)c->fb.p;
-    float *bvec = fvec + (size_t)C * KP;
-    double *part = nullptr, *g0 = nullptr;
-    if (stats) {
-        part = (double *)(((uintptr_t)(bvec + (size_t)C * KP) + 255) & ~(uintptr_t)255);
-        g0 = part + (size_t)C * (K * K + 7 * K);
-    }
-    cudaError_t e = launch_posterior(K, KP, o.init_mode, pl.n_chunks, pl.L, pl.d_chunks, prm->pi, prm->P,
-                                     wp.cblock + pl.lay.off_emis, wp.head, wp.packed, wp.lv.A[0],
-                                     (const int32_t *)wp.lv.e[0], fvec, bvec, gamma, part, g0, stats,
-                                     (cudaStream_t)stream);
-    c->last_launches += 1 + (pl.n_chunks > 0 ? 1 : 0) + (stats && pl.n_chunks > 0 ? 1 : 0);
-    if (e != cudaSuccess) return cuda_fail(c, e, "posterior launch");
-    return HMM_OK;
+    const SmoothOut so{gamma, stats};
+    return loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
+                          obs->tremor, &o, loglik, Mode::SMOOTH, &so, stream);
 }
 
 int hmm_posterior(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm_opts *opts, float *gamma,
@@ -1043,7 +1085,7 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     }
     // parameters, observations and the chunk table (and log L) from the likelihood path
     int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
-                                obs->tremor, &o, loglik, true, stream);
+                                obs->tremor, &o, loglik, Mode::PRODUCTS, nullptr, stream);
     if (rc) return rc;
     const Plan &pl = c->plan;
     const int KP = pl.lay.KP, C = std::max(1, pl.n_chunks);

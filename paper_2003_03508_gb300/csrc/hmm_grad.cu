@@ -109,16 +109,24 @@ __global__ void __launch_bounds__(GT) em_mstep_kernel(int K, const float *__rest
                                                       float *cov_out) {
     const StatsView st(stats, K);
     __shared__ double g0sum;
-    if (threadIdx.x == 0) {
+    // sums over a row, a warp each
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto row_sum = [&](const double *row) {
         double s = 0.0;
-        for (int k = 0; k < K; ++k) s += st.G0[k];
-        g0sum = s;
+        for (int j = lane; j < K; j += 32) s += row[j];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    };
+    if (warp == 0) {
+        const double s = row_sum(st.G0);
+        if (lane == 0) g0sum = s;
+    }
+    for (int i = warp; i < K; i += GT / 32) {
+        const double rs = row_sum(st.N + i * K);
+        for (int j = lane; j < K; j += 32) P_out[i * K + j] = rs > 0.0 ? (float)(st.N[i * K + j] / rs) : P[i * K + j];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < K; i += GT) {
-        double rs = 0.0;
-        for (int j = 0; j < K; ++j) rs += st.N[i * K + j];
-        for (int j = 0; j < K; ++j) P_out[i * K + j] = rs > 0.0 ? (float)(st.N[i * K + j] / rs) : P[i * K + j];
         pi_out[i] = g0sum > 0.0 ? (float)(st.G0[i] / g0sum) : pi[i];
         const double g = st.Gr[i], gs = st.Gs[i];
         p_out[i] = gs > 0.0 ? (float)(g / gs) : p[i];

@@ -98,6 +98,23 @@ struct StrandPtrs {
     int *todo = nullptr;       // [1 + n_prop]
 };
 
+// The posterior of one sequence by strands (hmm_smooth.cu). Row t belongs to
+// observation t; u's row t to the step from t to t + 1.
+constexpr int SMOOTH_PARTS = 456;  // partial sums of the E-step statistics
+struct SmoothPtrs {
+    int warm = 0;              // warm-up steps of the backward strands
+    float *alpha = nullptr;    // [T][KP] forward vectors, any scale (null: no posterior)
+    float *gamma = nullptr;    // [T][K]
+    float *u = nullptr;        // [T][KP] d o b / S of every step (null: no statistics)
+    float *bs = nullptr;       // [n][KP] backward vector at the piece's end
+    float *be = nullptr;       // [n][KP] and at its start
+    float *carry = nullptr;    // [n][KP] true vector where a piece ended unmet
+    int *unmet = nullptr;      // [n] 2 x rows written again, + 1 where the piece ended first
+    double *part = nullptr;    // [SMOOTH_PARTS][K K + 7 K]
+    double *g0 = nullptr;      // [K]
+    double *stats = nullptr;   // K K + 8 K, as hmm_expected_stats
+};
+
 struct ConstLayout {
     int KP;         // padded state count used by the chunk kernel
     int off_emis;   // EM_ALL * KP floats
@@ -174,7 +191,9 @@ int strand_simt_kp(int K);
 int strand_simt_per_warp(int KP);
 cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                                const float *cblock, const float *pi, const float2 *head, const float2 *packed,
-                               const StrandPtrs &sp, cudaStream_t st);
+                               const StrandPtrs &sp, float *alpha, cudaStream_t st);
+cudaError_t launch_smooth(int K, int KP, int64_t steps, const ConstLayout &lay, const float *cblock, const float2 *head,
+                          const float2 *packed, const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st);
 int strand_mma_per_warp(int KP);
 cudaError_t launch_strand_mma(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                               const float *cblock, const float *pi, const float2 *head, const float2 *packed,
@@ -199,7 +218,8 @@ int chunk_tc_chunks_per_item(int KP, int precision);
 cudaError_t launch_posterior(int K, int KP, int init_mode, int n_chunks, int L, const ChunkDesc *chunks,
                              const float *pi, const float *P, const float *em, const float2 *head,
                              const float2 *packed, const float *A0, const int32_t *e0, float *fvec, float *bvec,
-                             float *gamma, double *stats_part, double *g0, double *stats, cudaStream_t st);
+                             float *gamma, double *stats_part, double *g0, double *stats, const int *todo,
+                             cudaStream_t st);
 int chunk_tc_wide_chunks_per_item(int KP, int precision);
 cudaError_t launch_viterbi(int K, int init_mode, int n_chunks, int L, const ConstLayout &lay, const ChunkDesc *chunks,
                            const float *pi, const float *P, const float *cblock, const float2 *head,

@@ -17,7 +17,6 @@ namespace hmm {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr float JOIN_TINY = 8.470329472543003e-22f;  // 2^-70: an entry this far below the largest cannot matter (PMIN)
 constexpr int JOIN_WARPS = 4;
 constexpr int JOIN_MOST = 2048;
 constexpr float JOIN_TOL = 3.0517578125e-5f;  // 2^-15: what FP32 vectors run on to
@@ -68,7 +67,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
         float lo = INFINITY, hi = 0.0f;
 #pragma unroll
         for (int c = 0; c < NC; ++c)
-            if (a[c] > JOIN_TINY || g[c] > JOIN_TINY) {
+            if (a[c] > STRAND_TINY || g[c] > STRAND_TINY) {
                 const float r = a[c] / g[c];
                 lo = fminf(lo, r);
                 hi = fmaxf(hi, r);

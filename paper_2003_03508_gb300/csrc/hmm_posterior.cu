@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(FB_THREADS) fb_scan_kernel(int K, int KP, int 
                                                              const float *__restrict__ pi, const float *__restrict__ P,
                                                              const float *__restrict__ em, const float2 *__restrict__ head,
                                                              const float *__restrict__ A0, const int32_t *__restrict__ e0,
-                                                             float *fvec, float *bvec, float *gamma) {
+                                                             float *fvec, float *bvec, float *gamma, const int *todo) {
+    if (todo && todo[0] == 0) return;  // done by strands
     extern __shared__ float sA[];           // KP x KP
     float *vec = sA + KP * KP;              // KP
     float *red = vec + KP;                  // FB_THREADS / 32
@@ -162,7 +163,8 @@ __global__ void __launch_bounds__(FB_THREADS) fb_chunk_kernel(int K, int KP, int
                                                               const float2 *__restrict__ packed,
                                                               const float *__restrict__ fvec,
                                                               const float *__restrict__ bvec, float *gamma,
-                                                              double *stats_part, double *g0) {
+                                                              double *stats_part, double *g0, const int *todo) {
+    if (todo && todo[0] == 0) return;
     extern __shared__ double sN[];           // K x K expected transitions (with statistics, FP64)
     float *sP = reinterpret_cast<float *>(sN + (stats_part ? K * K : 0));  // K x K (row-major)
     float *sPT = sP + K * K;                 // its transpose
@@ -253,7 +255,8 @@ __global__ void __launch_bounds__(FB_THREADS) fb_chunk_kernel(int K, int KP, int
 // stats = [N (K x K), G0, Gs, Gr, Sx, Sy, Sxx, Sxy, Syy]: the chunks'
 // partial sums added in chunk order (one thread per entry)
 __global__ void fb_stats_reduce_kernel(int K, int n_chunks, const double *__restrict__ part,
-                                       const double *__restrict__ g0, double *stats) {
+                                       const double *__restrict__ g0, double *stats, const int *todo) {
+    if (todo && todo[0] == 0) return;
     const int n = K * K + N_MOM * K;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
         double acc = 0.0;
@@ -269,7 +272,8 @@ __global__ void fb_stats_reduce_kernel(int K, int n_chunks, const double *__rest
 cudaError_t launch_posterior(int K, int KP, int init_mode, int n_chunks, int L, const ChunkDesc *chunks,
                              const float *pi, const float *P, const float *em, const float2 *head,
                              const float2 *packed, const float *A0, const int32_t *e0, float *fvec, float *bvec,
-                             float *gamma, double *stats_part, double *g0, double *stats, cudaStream_t st) {
+                             float *gamma, double *stats_part, double *g0, double *stats, const int *todo,
+                             cudaStream_t st) {
     const size_t scan_smem = sizeof(float) * ((size_t)KP * KP + KP + FB_THREADS / 32) + sizeof(int) * FB_THREADS / 32;
     const size_t chunk_smem = (stats_part ? sizeof(double) * (size_t)K * K : 0) +
                               sizeof(float) * (2 * (size_t)K * K + 2 * KP + FB_THREADS / 32);
@@ -278,12 +282,12 @@ cudaError_t launch_posterior(int K, int KP, int init_mode, int n_chunks, int L, 
     e = cudaFuncSetAttribute(fb_chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chunk_smem);
     if (e != cudaSuccess) return e;
     fb_scan_kernel<<<2, FB_THREADS, scan_smem, st>>>(K, KP, init_mode, n_chunks, pi, P, em, head, A0, e0, fvec,
-                                                      bvec, gamma);
+                                                      bvec, gamma, todo);
     if (n_chunks > 0)
         fb_chunk_kernel<<<n_chunks, FB_THREADS, chunk_smem, st>>>(K, KP, init_mode, L, chunks, pi, P, em, head,
-                                                                   packed, fvec, bvec, gamma, stats_part, g0);
+                                                                   packed, fvec, bvec, gamma, stats_part, g0, todo);
     if (stats && n_chunks > 0)
-        fb_stats_reduce_kernel<<<(K * K + N_MOM * K + 255) / 256, 256, 0, st>>>(K, n_chunks, stats_part, g0, stats);
+        fb_stats_reduce_kernel<<<(K * K + N_MOM * K + 255) / 256, 256, 0, st>>>(K, n_chunks, stats_part, g0, stats, todo);
     return cudaGetLastError();
 }
 

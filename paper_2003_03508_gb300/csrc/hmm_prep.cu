@@ -53,7 +53,9 @@ __device__ __forceinline__ int kmajor_offset(int n, int k, int KP, int elems16) 
     return (n >> 3) * sbo_elems + (k / elems16) * (8 * elems16) + (n & 7) * elems16 + (k % elems16);
 }
 
-__global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *__restrict__ pi,
+constexpr int PREP_THREADS = 256;
+
+__global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout lay, int precision, const float *__restrict__ pi,
                             const float *__restrict__ P, const float *__restrict__ p,
                             const float *__restrict__ mu, const float *__restrict__ cov,
                             float *__restrict__ cblock, int *__restrict__ prop_bad,
@@ -87,26 +89,22 @@ __global__ void prep_kernel(int K, ConstLayout lay, int precision, const float *
     }
     __syncthreads();
 
-    // rows of P: non-negative, finite, summing to 1 within 1e-5
-    for (int i = threadIdx.x; i < K; i += blockDim.x) {
+    // rows of P and pi: non-negative, finite, summing to 1 within 1e-5 (a warp
+    // per row; row K is pi)
+    for (int i = threadIdx.x >> 5; i <= K; i += blockDim.x >> 5) {
+        const float *row = i < K ? P + i * K : pi;
+        const int lane = threadIdx.x & 31;
         double s = 0.0;
-        bool ok = true;
-        for (int j = 0; j < K; ++j) {
-            float v = P[i * K + j];
+        bool ok = true, tiny = false;
+        for (int j = lane; j < K; j += 32) {
+            const float v = row[j];
             ok = ok && isfinite(v) && v >= 0.0f;
-            if (v < STRAND_PMIN) small = 1;
+            tiny = tiny || v < STRAND_PMIN;
             s += v;
         }
-        if (!ok || fabs(s - 1.0) > 1e-5) bad = 1;
-    }
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        bool ok = true;
-        for (int k = 0; k < K; ++k) {
-            ok = ok && isfinite(pi[k]) && pi[k] >= 0.0f;
-            s += pi[k];
-        }
-        if (!ok || fabs(s - 1.0) > 1e-5) bad = 1;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (!ok || (lane == 0 && !(fabs(s - 1.0) <= 1e-5))) bad = 1;
+        if (i < K && tiny) small = 1;
     }
     // per-state emission constants (log2 domain), padded states emit nothing
     const double LOG2E = 1.4426950408889634074;
@@ -215,7 +213,7 @@ cudaError_t launch_prep(int n_prop, int K, const ConstLayout &lay, int precision
                         const float *cov, float *cblock, int *prop_bad, unsigned *status,
                         const StrandPtrs &sp, cudaStream_t st) {
     (void)init_mode;
-    prep_kernel<<<n_prop, 128, 0, st>>>(K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad,
+    prep_kernel<<<n_prop, PREP_THREADS, 0, st>>>(K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad,
                                         status, sp);
     return cudaGetLastError();
 }

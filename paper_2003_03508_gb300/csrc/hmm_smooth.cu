@@ -1,0 +1,584 @@
+// Posterior probabilities and E-step statistics of one sequence by strands
+// (hmm_strand.cuh), in place of two scans over chunk products on one CTA.
+//
+// The forward strands keep their vector of every step (alpha, any scale). The
+// backward vectors b_t = P (d_{t+1} o b_{t+1}) of a piece are carried the same
+// way: from a flat vector some steps behind the piece (or from the sequence's
+// end, where it is exact) down to the piece's start, checked against the
+// strand of the piece behind where the two meet. Each step in the piece gives
+//     w = d_t o b_t,  y = P w,  S = sum_i alpha_{t-1}(i) y(i),
+//     gamma_{t-1} = alpha_{t-1} o y / S,
+// and w / S is what the expected transition counts need:
+//     N_ij = P_ij sum_t alpha_{t-1}(i) w_t(j) / S_t,
+// a K x T by T x K product taken over blocks of 64 steps in FP32 and summed in
+// FP64. The gamma-weighted moments are taken about each state's mean, so that
+// their FP32 block sums lose nothing to the coordinates' size.
+//
+// Vectors that have not met at a piece's edge run on from the true one, and the
+// rows passed are written again (rows_join_kernel).
+//
+// What bounds it: a step of a lone warp, 0.2 us, times warm-up and piece, in
+// each direction; at T = 2^20 also the FMA pipe (K=25: 130 us a direction). The
+// rows are written once and read once or twice: 0.27 GB at K=32, T=2^20, 40 us.
+#include "hmm_strand_simt.cuh"
+
+namespace hmm {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// ---- backward strands ----
+template <class C>
+__global__ void __launch_bounds__(32 * STRAND_WPC, C::MIN_CTAS)
+strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float *__restrict__ cb,
+                   const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm) {
+    constexpr int KP = C::KP, NS = C::NS;
+    __shared__ __align__(16) float sv[STRAND_WPC][2 * C::PER_WARP * C::STRIDE];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wid = blockIdx.x * STRAND_WPC + warp;
+    if (wid * C::PER_WARP >= sp.n) return;
+    if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
+    const float *em = cb + lay.off_emis;
+    const int KPl = lay.KP;
+
+    SimtStrand<C> S;
+    S.init(sv[warp], lane);
+    S.load(cb + lay.off_p32, KPl, true, false);
+    const int own = S.own;
+    StrandBase base;
+    base.load(em, KPl);
+    Emis2 ec[NS / 2];
+#pragma unroll
+    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u, base.offt, base.offn);
+
+    const int k = wid * C::PER_WARP + S.slot;
+    const int sid = k < sp.n ? k : -1;
+    const StrandDesc d = sp.desc[sid < 0 ? 0 : sid];
+    const int64_t a = d.pstart, b = a + d.len;                // the piece's steps
+    const int64_t e = sid < 0 ? a : min(b + (int64_t)warm, steps);  // where the strand starts
+    const int64_t wtop = (e + 3) / 4 - 1;
+    const int mine = sid < 0 ? 0 : (int)(wtop - a / 4 + 1);
+    int nwin = mine;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nwin = max(nwin, __shfl_xor_sync(FULL, nwin, o));
+    bool bad = false;
+    float v[NS];
+#pragma unroll
+    for (int u = 0; u < NS; ++u) v[u] = own + u < K ? 1.0f : 0.0f;
+
+    // gamma's row t of the strand's own states from alpha's row and y
+    auto put_gamma = [&](int64_t t, const float (&al)[NS], const float (&y)[NS], float r) {
+        float *g = sm.gamma + t * K + own;
+        if ((K & 3) == 0 && NS == 4) {
+            if (own < K) *reinterpret_cast<float4 *>(g) = make_float4(al[0] * y[0] * r, al[1] * y[1] * r, al[NS - 2] * y[NS - 2] * r, al[NS - 1] * y[NS - 1] * r);
+        } else {
+#pragma unroll
+            for (int u = 0; u < NS; ++u)
+                if (own + u < K) g[u] = al[u] * y[u] * r;
+        }
+    };
+    {  // the sequence's last row
+        const bool last = sid >= 0 && (d.flags & SD_LAST);
+        float al[NS], t = 0.0f;
+#pragma unroll
+        for (int u = 0; u < NS; ++u) al[u] = 0.0f;
+        if (last) S.fetch(sm.alpha + steps * KP, al);
+#pragma unroll
+        for (int u = 0; u < NS; ++u) t += al[u];
+        t = S.sum_all(t);
+        if (last) put_gamma(steps, al, v, 1.0f / t);
+    }
+
+    const float4 *obs = reinterpret_cast<const float4 *>(packed);
+    float4 na = make_float4(0.f, 0.f, 0.f, 0.f), nb = na;
+    if (mine > 0) {
+        na = obs[2 * wtop];
+        nb = obs[2 * wtop + 1];
+    }
+    for (int it = 0; it < nwin; ++it) {
+        const int64_t w = wtop - it;
+        const bool act = it < mine;
+        const float ox[4] = {na.x - base.cx, na.z - base.cx, nb.x - base.cx, nb.z - base.cx};
+        const float oy[4] = {na.y - base.cy, na.w - base.cy, nb.y - base.cy, nb.w - base.cy};
+        if (it + 1 < mine) {
+            na = obs[2 * (w - 1)];
+            nb = obs[2 * (w - 1) + 1];
+        }
+        if (act && 4 * (w + 1) == b && !(d.flags & SD_LAST)) S.store(sm.bs + (size_t)sid * KP, v);  // the piece begins
+        const bool own_steps = act && 4 * w < b;
+        const int valid = act ? (int)min((int64_t)4, e - 4 * w) : 0;
+        if (it + 1 < mine && 4 * (w - 1) < b) {
+            // alpha's rows of the next window
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(sm.alpha + (4 * (w - 1) + j) * KP + own));
+        }
+        float keep[NS];
+#pragma unroll
+        for (int u = 0; u < NS; ++u) keep[u] = v[u];
+#pragma unroll
+        for (int j = 3; j >= 0; --j) {
+            const int64_t i = 4 * w + j;
+            float f[NS], y[NS], al[NS], s = 0.0f;
+#pragma unroll
+            for (int u = 0; u < NS; ++u) al[u] = 0.0f;
+            if (own_steps && valid == 4) S.fetch(sm.alpha + i * KP, al);
+#pragma unroll
+            for (int u = 0; u < NS / 2; ++u) ec[u].eval(ox[j], oy[j], !isnan(ox[j]), f[2 * u], f[2 * u + 1]);
+#pragma unroll
+            for (int u = 0; u < NS; ++u) f[u] = ex2(f[u]) * v[u];
+            S.mul(f, y);
+#pragma unroll
+            for (int u = 0; u < NS; ++u) s = fmaf(al[u], y[u], s);
+            s = S.sum_all(s);
+            if (own_steps && valid == 4) {
+                const float r = rcp(s);
+                put_gamma(i, al, y, r);
+                if (sm.u) {
+#pragma unroll
+                    for (int u = 0; u < NS; ++u) f[u] *= r;
+                    S.store(sm.u + i * KP, f);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < NS; ++u) v[u] = y[u];
+        }
+        const float m = S.max_all(S.max_own(v));
+        const bool fine = valid == 4 && m >= STRAND_SHRINK_KEEP && m <= STRAND_GROW;
+        const bool redo = act && !fine;
+        const float sc = pow2f(-float_exponent(m));
+#pragma unroll
+        for (int u = 0; u < NS; ++u) v[u] = fine ? v[u] * sc : keep[u];
+        if (__any_sync(FULL, redo)) {
+            for (int j = 3; j >= 0; --j) {
+                const int64_t i = 4 * w + j;
+                const float x = j == 0 ? ox[0] : j == 1 ? ox[1] : j == 2 ? ox[2] : ox[3];
+                const float yy = j == 0 ? oy[0] : j == 1 ? oy[1] : j == 2 ? oy[2] : oy[3];
+                const bool todo = redo && j < valid;
+                float l[NS], y[NS], al[NS], s = 0.0f;
+#pragma unroll
+                for (int u = 0; u < NS; ++u) al[u] = 0.0f;
+                if (todo && own_steps) S.fetch(sm.alpha + i * KP, al);
+#pragma unroll
+                for (int u = 0; u < NS / 2; ++u) ec[u].eval(x, yy, !isnan(x), l[2 * u], l[2 * u + 1]);
+                float mx = S.max_all(S.max_own(l));
+                const bool emits = mx + base.off(!isnan(x)) >= -(float)EXP_LIMIT;
+                const float fm = emits ? floorf(mx) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < NS; ++u) l[u] = ex2(l[u] - fm) * v[u];
+                S.mul(l, y);
+                mx = S.max_all(S.max_own(y));
+                const bool can = emits && mx >= STRAND_SHRINK && mx <= STRAND_GROW;
+                const float sy = can ? pow2f(-float_exponent(mx)) : 1.0f;
+#pragma unroll
+                for (int u = 0; u < NS; ++u) {
+                    y[u] *= sy;
+                    l[u] *= sy;
+                    s = fmaf(al[u], y[u], s);
+                }
+                s = S.sum_all(s);
+                if (todo && can) {
+#pragma unroll
+                    for (int u = 0; u < NS; ++u) v[u] = y[u];
+                    if (own_steps) {
+                        const float r = rcp(s);
+                        put_gamma(i, al, y, r);
+                        if (sm.u) {
+#pragma unroll
+                            for (int u = 0; u < NS; ++u) l[u] *= r;
+                            S.store(sm.u + i * KP, l);
+                        }
+                    }
+                } else if (todo) {
+                    bad = true;
+                }
+            }
+        }
+    }
+    if (sid < 0) return;
+    S.store(sm.be + (size_t)sid * KP, v);
+    if (lane % C::G == 0 && bad) send_to_chunks(sp, 0);
+}
+
+// ---- pieces whose vectors had not met at their edge: rows written again ----
+// BACK = false: strand c's first rows of alpha, from the end of strand c - 1.
+// BACK = true: strand c's last rows of gamma (and u), from the end of strand
+// c + 1. One warp per piece, one step after another with exact scaling. A piece
+// that ends first is noted with its true vector (unmet, carry), and a second
+// launch (`chain`) takes those on through the pieces that follow once every
+// piece has written its rows; after ROWS_MOST steps, or where two of them
+// touch, the sequence is left to the chunk products.
+constexpr int64_t ROWS_MOST = 16384;
+
+template <int NC, bool BACK>
+__global__ void __launch_bounds__(128)
+rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__restrict__ cb,
+                 const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm) {
+    __shared__ float2 sag[4][32 * NC];
+    constexpr float tol = 3.0517578125e-5f;  // 2^-15, as in the likelihood's join
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
+    const float *em = cb + lay.off_emis, *P = cb + lay.off_p32;
+    const int KPl = lay.KP;
+    float a[NC], g[NC];
+    auto all_max = [&](float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
+        return v;
+    };
+    auto all_sum = [&](float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        return v;
+    };
+    auto met = [&]() {
+        float lo = INFINITY, hi = 0.0f;
+#pragma unroll
+        for (int n = 0; n < NC; ++n)
+            if (a[n] > STRAND_TINY || g[n] > STRAND_TINY) {
+                const float r = a[n] / g[n];
+                lo = fminf(lo, r);
+                hi = fmaxf(hi, r);
+            }
+        return all_max(hi) <= -all_max(-lo) * (1.0f + tol);
+    };
+    auto fetch = [&](const float *row, float (&x)[NC]) {
+#pragma unroll
+        for (int n = 0; n < NC; ++n) x[n] = lane + 32 * n < K ? row[lane + 32 * n] : 0.0f;
+    };
+    float pc[NC == 1 ? 32 : 1];  // this lane's column of P (row, backward)
+    // runs a and piece c's own vector through the piece, writing a's rows, at
+    // least `least` of them: 1 they met, 0 the piece ended, -1 out of range
+    int rows = 0;
+    auto run = [&](int c, int least) {
+        const StrandDesc d = sp.desc[c];
+        fetch((BACK ? sm.bs : sp.vs) + (size_t)c * KP, g);
+        rows = 0;
+        if (least == 0 && met()) return 1;
+        if (NC == 1) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) pc[NC == 1 ? j : 0] = j < K && lane < K ? (BACK ? P[lane * KPl + j] : P[j * KPl + lane]) : 0.0f;
+        }
+        for (int &s = rows; s < least || (s & 3) || !met(); ++s) {
+            if (s >= d.len) return 0;
+            const int64_t i = BACK ? d.pstart + d.len - 1 - s : d.pstart + s;
+            const float2 o = packed[i];
+            const bool tr = !isnan(o.x);
+            float f[NC], wa[NC], mx = -INFINITY;
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                const int k = lane + 32 * n;
+                f[n] = k < K ? log2_emission(em, KPl, k, o.x, o.y, tr) : -INFINITY;
+                mx = fmaxf(mx, f[n]);
+            }
+            mx = all_max(mx);
+            if (!(mx >= -(float)EXP_LIMIT)) return -1;
+            const float fm = floorf(mx);
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                f[n] = ex2(f[n] - fm);
+                wa[n] = BACK ? a[n] * f[n] : a[n];
+                sag[warp][lane + 32 * n] = make_float2(wa[n], BACK ? g[n] * f[n] : g[n]);
+                a[n] = g[n] = 0.0f;
+            }
+            __syncwarp();
+            if (NC == 1) {
+                f32x2 t[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float p = pc[NC == 1 ? j : 0];
+                    t[j & 3] = fma2(*reinterpret_cast<const f32x2 *>(&sag[warp][j]), pack2(p, p), t[j & 3]);
+                }
+                unpack2(add2(add2(t[0], t[1]), add2(t[2], t[3])), a[0], g[0]);
+            } else {
+#pragma unroll 8
+                for (int j = 0; j < 32 * NC; ++j) {
+                    const float2 x = sag[warp][j];
+#pragma unroll
+                    for (int n = 0; n < NC; ++n) {
+                        const int k = lane + 32 * n;
+                        const float p = k < K && j < K ? (BACK ? P[k * KPl + j] : P[j * KPl + k]) : 0.0f;
+                        a[n] = fmaf(x.x, p, a[n]);
+                        g[n] = fmaf(x.y, p, g[n]);
+                    }
+                }
+            }
+            __syncwarp();
+            float ma = 0.0f, mg = 0.0f;
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                if (!BACK) {
+                    a[n] *= f[n];
+                    g[n] *= f[n];
+                }
+                ma = fmaxf(ma, a[n]);
+                mg = fmaxf(mg, g[n]);
+            }
+            ma = all_max(ma);
+            mg = all_max(mg);
+            if (!(ma >= STRAND_SHRINK && mg >= STRAND_SHRINK && ma <= STRAND_GROW && mg <= STRAND_GROW)) return -1;
+            const float fa = pow2f(-float_exponent(ma)), fg = pow2f(-float_exponent(mg));
+            float z = 0.0f, al[NC];
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                const int k = lane + 32 * n;
+                a[n] *= fa;
+                g[n] *= fg;
+                wa[n] *= fa;
+                if (BACK) {
+                    al[n] = k < K ? sm.alpha[i * KP + k] : 0.0f;
+                    z = fmaf(al[n], a[n], z);
+                } else if (k < KP) {
+                    sm.alpha[(i + 1) * KP + k] = a[n];
+                }
+            }
+            if (BACK) {
+                const float r = 1.0f / all_sum(z);
+#pragma unroll
+                for (int n = 0; n < NC; ++n) {
+                    const int k = lane + 32 * n;
+                    if (k < K) sm.gamma[i * K + k] = al[n] * a[n] * r;
+                    if (k < KP && sm.u) sm.u[i * KP + k] = wa[n] * r;
+                }
+            }
+        }
+        return 1;
+    };
+    if (!chain) {
+        const int c = blockIdx.x * 4 + warp;
+        if (c >= sp.n) return;
+        int how = 1;
+        if (!(sp.desc[c].flags & (BACK ? SD_LAST : SD_FIRST))) {
+            fetch(BACK ? sm.be + (size_t)(c + 1) * KP : sp.ve + (size_t)(c - 1) * KP, a);
+            how = run(c, 0);
+        }
+        if (how == 0)
+#pragma unroll
+            for (int n = 0; n < NC; ++n)
+                if (lane + 32 * n < K) sm.carry[(size_t)c * KP + lane + 32 * n] = a[n];
+        if (lane == 0) {
+            sm.unmet[c] = 2 * rows + (how == 0 ? 1 : 0);
+            if (how < 0) send_to_chunks(sp, 0);
+        }
+        return;
+    }
+    // one warp per piece: those unmet whose neighbour behind had met (its end is
+    // the true vector) go on, up to the next such piece
+    const int x0 = blockIdx.x * 4 + warp;  // in the recursion's direction
+    if (x0 >= sp.n) return;
+    auto piece = [&](int x) { return BACK ? sp.n - 1 - x : x; };
+    auto starts = [&](int x) { return (sm.unmet[piece(x)] & 1) && (x == 0 || !(sm.unmet[piece(x - 1)] & 1)); };
+    if (!starts(x0)) return;
+    fetch(sm.carry + (size_t)piece(x0) * KP, a);
+    int how = 0;
+    int64_t spent = 0;
+    for (int x = x0 + 1; x < sp.n && how == 0; ++x) {
+        // (all the rows that the piece's own run wrote, from a vector that was not the true one)
+        how = starts(x) || spent > ROWS_MOST ? -1 : run(piece(x), sm.unmet[piece(x)] >> 1);
+        spent += sp.desc[piece(x)].len;
+    }
+    if (how < 0 && lane == 0) send_to_chunks(sp, 0);
+}
+
+// ---- E-step statistics ----
+constexpr int SX_THREADS = 256, SX_BLOCK = 64;
+
+// One CTA per range of steps: sum of alpha_i (x) u_i times P, and the gamma
+// moments about the states' means, FP32 within a block of 64 steps and FP64
+// across blocks; the CTAs' sums are added in order by a later kernel.
+template <int KP>
+__global__ void __launch_bounds__(SX_THREADS)
+stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__restrict__ cb,
+             const float2 *__restrict__ head, const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm,
+             double *__restrict__ part, double *__restrict__ g0) {
+    constexpr int CQ = KP / 4;                                        // column quads
+    constexpr int NR = KP * CQ <= SX_THREADS ? 1 : KP * CQ / SX_THREADS;  // rows of N per thread
+    constexpr int SL = KP * CQ <= SX_THREADS ? SX_THREADS / (KP * CQ) : 1;  // step slices of N
+    constexpr int MS = SX_THREADS / KP;                               // step slices of the moments
+    __shared__ __align__(16) float sA[SX_BLOCK][KP], sU[SX_BLOCK][KP];
+    __shared__ float2 sO[SX_BLOCK];
+    __shared__ double red[SX_THREADS][4];
+    if (sp.route[0] != ROUTE_STRANDS) return;
+    const int tid = threadIdx.x;
+    const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(i0 + per, steps);
+    const float *em = cb + lay.off_emis;
+    double *out = part + (size_t)blockIdx.x * (K * K + 7 * K);
+
+    const int cq = tid % CQ, row = (tid / CQ) % (KP / NR), sl = tid / (CQ * (KP / NR));
+    double acc[NR][4] = {};
+    const int mk = tid % KP, msl = tid / KP;
+    const float mx = mk < K ? em[EM_MUX * lay.KP + mk] : 0.0f, my = mk < K ? em[EM_MUY * lay.KP + mk] : 0.0f;
+    double mom[7] = {};
+    // gamma rows: i + 1 for each of this CTA's steps i, and row 0 for the first CTA
+    auto add = [&](float (&s)[7], float g, float2 o) {
+        s[0] += g;
+        if (!isnan(o.x)) {
+            const float dx = o.x - mx, dy = o.y - my;
+            s[1] += g;
+            s[2] = fmaf(g, dx, s[2]);
+            s[3] = fmaf(g, dy, s[3]);
+            s[4] = fmaf(g * dx, dx, s[4]);
+            s[5] = fmaf(g * dx, dy, s[5]);
+            s[6] = fmaf(g * dy, dy, s[6]);
+        }
+    };
+    for (int64_t b = i0; b < i1; b += SX_BLOCK) {
+        const int n = (int)min((int64_t)SX_BLOCK, i1 - b);
+        __syncthreads();
+        for (int x = tid; x < SX_BLOCK * CQ; x += SX_THREADS) {
+            const int s = x / CQ;
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            reinterpret_cast<float4 *>(&sA[0][0])[x] = s < n ? reinterpret_cast<const float4 *>(sm.alpha + b * KP)[x] : zero;
+            reinterpret_cast<float4 *>(&sU[0][0])[x] = s < n ? reinterpret_cast<const float4 *>(sm.u + b * KP)[x] : zero;
+        }
+        for (int x = tid; x < n; x += SX_THREADS) sO[x] = packed[b + x];
+        __syncthreads();
+        float t[NR][4] = {};
+        if (sl < SL) {
+            for (int s = sl; s < SX_BLOCK; s += SL) {
+                const float4 u = *reinterpret_cast<const float4 *>(&sU[s][4 * cq]);
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const float al = sA[s][row + r * (KP / NR)];
+                    t[r][0] = fmaf(al, u.x, t[r][0]);
+                    t[r][1] = fmaf(al, u.y, t[r][1]);
+                    t[r][2] = fmaf(al, u.z, t[r][2]);
+                    t[r][3] = fmaf(al, u.w, t[r][3]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[r][c] += t[r][c];
+        }
+        if (msl < MS && mk < K) {
+            float m[7] = {};
+            for (int s = msl; s < n; s += MS) add(m, sm.gamma[(b + s + 1) * K + mk], sO[s]);
+#pragma unroll
+            for (int c = 0; c < 7; ++c) mom[c] += m[c];
+        }
+    }
+    if (blockIdx.x == 0 && msl == 0 && mk < K) {
+        float m[7] = {};
+        const float g = sm.gamma[mk];
+        add(m, g, head[0]);
+#pragma unroll
+        for (int c = 0; c < 7; ++c) mom[c] += m[c];
+        g0[mk] = g;
+    }
+    // the slices together, in order
+    const float *P = cb + lay.off_p32;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) red[tid][c] = acc[r][c];
+        __syncthreads();
+        if (sl == 0) {
+            const int i = row + r * (KP / NR);
+            for (int c = 0; c < 4; ++c) {
+                const int j = 4 * cq + c;
+                double v = 0.0;
+                for (int x = 0; x < SL; ++x) v += red[tid + x * CQ * (KP / NR)][c];
+                if (i < K && j < K) out[i * K + j] = v * (double)P[i * lay.KP + j];
+            }
+        }
+    }
+    double s[7];
+    for (int c = 0; c < 7; ++c) {
+        __syncthreads();
+        red[tid][0] = mom[c];
+        __syncthreads();
+        s[c] = 0.0;
+        if (msl == 0)
+            for (int x = 0; x < MS; ++x) s[c] += red[tid + x * KP][0];
+    }
+    if (msl == 0 && mk < K) {
+        // back from the mean: S_x = sum g dx + mx sum g, and so on
+        const double ux = mx, uy = my;
+        const double v[7] = {s[0], s[1], s[2] + ux * s[1], s[3] + uy * s[1],
+                             s[4] + 2.0 * ux * s[2] + ux * ux * s[1],
+                             s[5] + ux * s[3] + uy * s[2] + ux * uy * s[1],
+                             s[6] + 2.0 * uy * s[3] + uy * uy * s[1]};
+        for (int c = 0; c < 7; ++c) out[K * K + c * K + mk] = v[c];
+    }
+}
+
+// stats = [N, G0, Gs, Gr, Sx, Sy, Sxx, Sxy, Syy]: a warp per entry adds the
+// CTAs' sums in a fixed order
+__global__ void stats_sum_kernel(int K, int n_parts, const double *__restrict__ part, const double *__restrict__ g0,
+                                 const int *__restrict__ route, double *stats) {
+    if (route[0] != ROUTE_STRANDS) return;
+    const int n = K * K + 7 * K;
+    const int lane = threadIdx.x & 31;
+    for (int e = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; e < n; e += gridDim.x * (blockDim.x / 32)) {
+        double acc = 0.0;
+        for (int c = lane; c < n_parts; c += 32) acc += part[(size_t)c * n + e];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+        if (lane == 0) stats[e < K * K ? e : e + K] = acc;
+    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) stats[K * K + k] = g0[k];
+}
+
+template <int KP>
+cudaError_t back_t(int K, int64_t steps, const ConstLayout &lay, const float *cb, const float2 *packed,
+                   const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st) {
+    using C = SimtTile<KP>;
+    const int warps = (sp.n + C::PER_WARP - 1) / C::PER_WARP;
+    strand_back_kernel<C><<<(warps + STRAND_WPC - 1) / STRAND_WPC, 32 * STRAND_WPC, 0, st>>>(K, steps, sm.warm, lay, cb,
+                                                                                           packed, sp, sm);
+    return cudaGetLastError();
+}
+
+template <int KP>
+cudaError_t stats_t(int K, int64_t steps, const ConstLayout &lay, const float *cb, const float2 *head,
+                    const float2 *packed, const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st) {
+    const int64_t blocks = (steps + SX_BLOCK - 1) / SX_BLOCK;
+    const int64_t per = (blocks + SMOOTH_PARTS - 1) / SMOOTH_PARTS * SX_BLOCK;
+    const int ctas = (int)((steps + per - 1) / per);
+    stats_kernel<KP><<<ctas, SX_THREADS, 0, st>>>(K, steps, per, lay, cb, head, packed, sp, sm, sm.part, sm.g0);
+    stats_sum_kernel<<<(K * K + 7 * K + 7) / 8, 256, 0, st>>>(K, ctas, sm.part, sm.g0, sp.route, sm.stats);
+    return cudaGetLastError();
+}
+
+template <bool BACK>
+cudaError_t join_t(int K, int KP, const ConstLayout &lay, const float *cb, const float2 *packed, const StrandPtrs &sp,
+                   const SmoothPtrs &sm, cudaStream_t st) {
+    auto kern = KP <= 32 ? rows_join_kernel<1, BACK> : rows_join_kernel<2, BACK>;
+    kern<<<(sp.n + 3) / 4, 128, 0, st>>>(K, KP, false, lay, cb, packed, sp, sm);
+    kern<<<(sp.n + 3) / 4, 128, 0, st>>>(K, KP, true, lay, cb, packed, sp, sm);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_smooth(int K, int KP, int64_t steps, const ConstLayout &lay, const float *cblock, const float2 *head,
+                          const float2 *packed, const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st) {
+    cudaError_t e = join_t<false>(K, KP, lay, cblock, packed, sp, sm, st);
+    if (e != cudaSuccess) return e;
+#define HMM_SMOOTH_CASE(KPV)                                                       \
+    case KPV:                                                                      \
+        e = back_t<KPV>(K, steps, lay, cblock, packed, sp, sm, st);                \
+        if (e == cudaSuccess) e = join_t<true>(K, KP, lay, cblock, packed, sp, sm, st); \
+        if (e == cudaSuccess && sm.stats) e = stats_t<KPV>(K, steps, lay, cblock, head, packed, sp, sm, st); \
+        return e;
+    switch (KP) {
+        HMM_SMOOTH_CASE(4)
+        HMM_SMOOTH_CASE(8)
+        HMM_SMOOTH_CASE(16)
+        HMM_SMOOTH_CASE(32)
+        HMM_SMOOTH_CASE(64)
+        default: return cudaErrorInvalidValue;
+    }
+#undef HMM_SMOOTH_CASE
+}
+
+}  // namespace hmm

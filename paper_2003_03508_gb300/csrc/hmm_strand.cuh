@@ -35,6 +35,8 @@ namespace hmm {
 
 constexpr float STRAND_PMIN = 9.094947017729282e-13f;   // 2^-40
 constexpr float STRAND_SHRINK = 8.673617379884035e-19f; // 2^-60
+constexpr float STRAND_SHRINK_KEEP = 5.960464477539063e-08f;  // 2^-24: where every step's vector is kept
+constexpr float STRAND_TINY = 8.470329472543003e-22f;   // 2^-70: an entry this far below the largest cannot matter (PMIN)
 constexpr float STRAND_GROW = 1.2676506002282294e30f;   // 2^100
 
 typedef unsigned long long f32x2;  // two packed floats

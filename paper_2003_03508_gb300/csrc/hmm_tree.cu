@@ -166,7 +166,8 @@ cudaError_t launch_tree_level(int n_prop, int KP, int level, int n_groups, const
 
 // ---------------------------------------------------------------- final
 
-constexpr int FINAL_THREADS = 128;
+constexpr int FINAL_THREADS = 256;
+constexpr int SKIP_WORDS = 512;
 
 __device__ double block_sum_fixed(double v, double *red) {
     // deterministic: fixed pairing in shared memory
@@ -200,6 +201,7 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
              const float *__restrict__ cov, const int *__restrict__ prop_bad,
              const int *__restrict__ obs_bad, StrandPtrs sp, int strand_kp, double *__restrict__ out) {
     __shared__ double red[FINAL_THREADS];
+    __shared__ unsigned skip[SKIP_WORDS];
     __shared__ double lpi0[80];   // log of the initial vector
     __shared__ double w[80];      // log h_i + ex_i ln 2
     const int q = blockIdx.x;
@@ -212,29 +214,40 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
     const double LN2 = 0.69314718055994530942;
     const double LOG_2PI = 1.8378770664093454836;
 
-    for (int j = tid; j < K; j += FINAL_THREADS) {
-        double v;
-        if (init_mode == HMM_INIT_TRANSITION_FIRST) {
-            v = 0.0;
-            for (int i = 0; i < K; ++i) v += (double)pi[i] * (double)P[i * K + j];
-        } else {
-            v = pi[j];
+    // strands leave only segments of at most one observation to the head vector
+    const bool strands = sp.route && sp.route[q] == ROUTE_STRANDS;
+    bool heads = !strands;
+    for (int x = tid; strands && x < n_seg; x += FINAL_THREADS) heads = heads || segs[x].T <= 1;
+    heads = __syncthreads_or(heads);
+    if (heads)
+        for (int j = tid; j < K; j += FINAL_THREADS) {
+            double v;
+            if (init_mode == HMM_INIT_TRANSITION_FIRST) {
+                v = 0.0;
+                for (int i = 0; i < K; ++i) v += (double)pi[i] * (double)P[i * K + j];
+            } else {
+                v = pi[j];
+            }
+            lpi0[j] = log(v);
         }
-        lpi0[j] = log(v);
-    }
     __syncthreads();
     double total = 0.0;
     // strands: each contributes its exponents and its scale over the strand
     // before; a segment's last one the sum of its vector as well
-    const bool strands = sp.route && sp.route[q] == ROUTE_STRANDS;
     if (strands) {
         // piece i, with the exponents and, if it is the last, the vector of strand e
         auto piece = [&](int i, int e) {
             const size_t at = (size_t)q * sp.n + e;
             double v = (double)sp.ex[at] * LN2 + sp.logr[(size_t)q * sp.n + i];
             if (sp.desc[e].flags & SD_LAST) {
+                // (rows are multiples of 16 bytes; entries past K are zero)
+                const float4 *row = reinterpret_cast<const float4 *>(sp.ve + at * strand_kp);
                 double a = 0.0;
-                for (int k = 0; k < K; ++k) a += (double)sp.ve[at * strand_kp + k];
+#pragma unroll 4
+                for (int k = 0; k < strand_kp / 4; ++k) {
+                    const float4 x = row[k];
+                    a += ((double)x.x + x.y) + ((double)x.z + x.w);
+                }
                 v += log(a);
             }
             return v;
@@ -242,23 +255,44 @@ final_kernel(int K, int KP, int init_mode, int n_seg, const SegFinal *__restrict
         double part = 0.0;
         if (!sp.jumps[q]) {
             for (int i = tid; i < sp.n; i += FINAL_THREADS) part += piece(i, i);
-        } else if (tid == 0) {
-            // some pieces are passed over: in order
-            for (int i = 0; i < sp.n;) {
-                const int j = sp.jump[(size_t)q * sp.n + i];
-                if (j >= 0) {
-                    part += piece(i, j);
-                    i = j + 1;
-                } else {
-                    part += sp.logr[(size_t)q * sp.n + i];
-                    while (!(sp.desc[i].flags & SD_LAST)) ++i;
-                    ++i;
+        } else {
+            // some pieces are passed over: those that jump, in order, each for
+            // the pieces it covers (skip), then the rest
+            const int *jump = sp.jump + (size_t)q * sp.n;
+            for (int base = 0, cur = 0; base < sp.n; base += 32 * SKIP_WORDS) {
+                const int n = min(sp.n - base, 32 * SKIP_WORDS);
+                __syncthreads();
+                for (int w = tid; w < SKIP_WORDS; w += FINAL_THREADS) skip[w] = 0u;
+                __syncthreads();
+                for (int i = tid; i < n; i += FINAL_THREADS)
+                    if (jump[base + i] != base + i) atomicOr(&skip[i >> 5], 1u << (i & 31));
+                __syncthreads();
+                if (tid == 0) {
+                    // (what an earlier round's last jump covers of this one)
+                    for (int x = base; x < min(cur, base + n); ++x) skip[(x - base) >> 5] |= 1u << ((x - base) & 31);
+                    for (int w = 0; 32 * w < n; ++w)
+                        for (unsigned m = skip[w]; m; m &= m - 1) {
+                            const int i = base + 32 * w + __ffs(m) - 1;
+                            if (i < cur) continue;
+                            int to = jump[i];
+                            if (to >= 0) {
+                                part += piece(i, to);
+                            } else {
+                                part += sp.logr[(size_t)q * sp.n + i];
+                                for (to = i; !(sp.desc[to].flags & SD_LAST);) ++to;
+                            }
+                            for (int x = i; x <= min(to, base + n - 1); ++x) skip[(x - base) >> 5] |= 1u << ((x - base) & 31);
+                            cur = to + 1;
+                        }
                 }
+                __syncthreads();
+                for (int i = tid; i < n; i += FINAL_THREADS)
+                    if (!(skip[i >> 5] >> (i & 31) & 1u)) part += piece(base + i, base + i);
             }
         }
         total = block_sum_fixed(part, red);
     }
-    for (int s = 0; s < n_seg; ++s) {
+    for (int s = 0; heads && s < n_seg; ++s) {
         const SegFinal sf = segs[s];
         if (strands && sf.T > 1) continue;
         double ll;
