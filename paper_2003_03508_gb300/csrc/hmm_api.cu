@@ -341,13 +341,18 @@ static StrandCost strand_cost(bool tensor, int KP, int precision) {
 // of a longer warm-up for all (K=32, 64 segments, 64 proposals: 1273 us at 128,
 // 1365 at 256; K=25, T=2^20, one chain: 119 us at 64, 131 at 128). With the
 // run-length option tremors are rare: 260 at the median, 800 at most.
-static int strand_warm(int L, bool sparse, bool tensor) { return sparse ? 512 : L <= 512 && !tensor ? 64 : 128; }
+// (The join's step is dearer beyond 32 states: K=45, T=9000, 20 proposals 470 to
+// 1260 us at 512, 220 to 690 at 768.)
+static int strand_warm(int K, int L, bool sparse, bool tensor) {
+    if (sparse) return K <= 32 ? 512 : 768;
+    return L <= 512 && !tensor ? 64 : 128;
+}
 
 // Piece length for a batch: the smallest modelled time over the lengths that
 // fill 1, 2, .. warps of a proposal (about an eighth more each beyond 32). One
 // wave of warps takes (warm + L) steps, at the latency of a step while a
 // scheduler holds few warps and at their issue time beyond.
-static int choose_strand_len(const StrandCost &c, int n_prop, const std::vector<int64_t> &steps, bool sparse, int n_sms,
+static int choose_strand_len(const StrandCost &c, int K, int n_prop, const std::vector<int64_t> &steps, bool sparse, int n_sms,
                              double &best) {
     int64_t longest = 0, all = 0;
     for (int64_t n : steps) {
@@ -367,7 +372,7 @@ static int choose_strand_len(const StrandCost &c, int n_prop, const std::vector<
         const int64_t waves = std::max<int64_t>(1, (warps + cap - 1) / cap);
         const int64_t per_sched = (std::min(warps, cap) + 4 * n_sms - 1) / (4 * n_sms);
         const double step = (double)std::max<int64_t>(c.latency, per_sched * c.issue);
-        const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm((int)L, sparse, c.tensor)) * step;
+        const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm(K, (int)L, sparse, c.tensor)) * step;
         if (!best_L || t < best) {
             best = t;
             best_L = L;
@@ -384,11 +389,7 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     pl.strand_kp = pl.precision == HMM_PREC_FP32_SIMT ? strand_simt_kp(pl.K) : pl.lay.KP;
     std::vector<int64_t> steps;
     for (int s = 0; s < pl.n_seg; ++s) steps.push_back(std::max<int64_t>(0, pl.offsets[s + 1] - pl.offsets[s] - 1));
-    int64_t all = 0;
-    for (int64_t n : steps) all += n;
-    // with the run-length option a short batch is done sooner by its binary
-    // powers: K=18, T=6416, 15 proposals 236 us against 266
-    if (!pl.strand_kp || pl.n_chunks == 0 || (sparse && all * pl.n_prop < (1 << 20))) {
+    if (!pl.strand_kp || pl.n_chunks == 0) {
         pl.strand_kp = 0;
         return;
     }
@@ -400,13 +401,13 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     }
     if (pl.precision != HMM_PREC_FP32_SIMT && !pl.smooth) {
         pl.strand_tensor = true;
-        L = choose_strand_len(strand_cost(true, pl.lay.KP, pl.precision), pl.n_prop, steps, sparse, n_sms, cost);
+        L = choose_strand_len(strand_cost(true, pl.lay.KP, pl.precision), pl.K, pl.n_prop, steps, sparse, n_sms, cost);
     }
     if (strand_simt_kp(pl.K)) {
         // the CUDA cores' strands are quicker by the step: for a batch too
         // small to fill the tensor cores' rows
         double other = 0.0;
-        const int L2 = choose_strand_len(strand_cost(false, strand_simt_kp(pl.K), pl.precision), pl.n_prop, steps,
+        const int L2 = choose_strand_len(strand_cost(false, strand_simt_kp(pl.K), pl.precision), pl.K, pl.n_prop, steps,
                                          sparse, n_sms, other);
         if (!L || other < cost) {
             L = L2;
@@ -417,7 +418,7 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     // every row of a posterior is used: pieces and warm-ups long enough that the
     // vectors have met before a piece ends
     if (pl.smooth) L = std::max(L, 128);
-    pl.strand_warm = pl.smooth ? 128 : strand_warm(L, sparse, pl.strand_tensor);
+    pl.strand_warm = pl.smooth ? 128 : strand_warm(pl.K, L, sparse, pl.strand_tensor);
     for (int s = 0; s < pl.n_seg; ++s) {
         // equal pieces of whole observation windows
         const int64_t wins = (steps[s] + OBS_WIN - 1) / OBS_WIN;
@@ -722,11 +723,10 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
 }
 
 // What a call of the likelihood path is for. LOGLIK: log L, by strands where
-// they apply. PRODUCTS: every proposal's chunk products as well, left in the
-// workspace (level 0) for the boundary scans of Viterbi. SMOOTH: the posterior
-// and the statistics of one sequence too (`out2`), by strands or, where these
-// do not apply, by scans over the chunk products.
-enum class Mode { LOGLIK, PRODUCTS, SMOOTH };
+// they apply. PATH: log L of one sequence with a plan that Viterbi's strands
+// share. SMOOTH: the posterior and the statistics of one sequence too (`out2`),
+// by strands or, where these do not apply, by scans over the chunk products.
+enum class Mode { LOGLIK, PATH, SMOOTH };
 struct SmoothOut {
     float *gamma;
     double *stats;
@@ -785,8 +785,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         L = tune_get(key);
         if (!L) L = choose_chunk_len(prec, n_prop, lay.KP, steps_total, c->n_sms);
     }
-    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode == Mode::SMOOTH)) {
-        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode == Mode::SMOOTH, c->n_sms);
+    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode != Mode::LOGLIK)) {
+        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode != Mode::LOGLIK, c->n_sms);
         if (c->plan.n_levels + 1 > MAX_LEVELS) {
             c->plan.valid = false;
             return fail(c, HMM_EINVAL, "too many chunks for the tree (raise chunk_len)");
@@ -817,7 +817,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
     // strands first; `todo` lists what is left to the chunk products (null: everything)
-    const StrandPtrs sp = mode == Mode::PRODUCTS ? StrandPtrs{} : wp.sp;
+    const StrandPtrs sp = wp.sp;
     const int *todo = sp.todo;
     SmoothPtrs sm;
     float *fvec = nullptr, *bvec = nullptr;
@@ -1085,29 +1085,53 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     }
     // parameters, observations and the chunk table (and log L) from the likelihood path
     int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
-                                obs->tremor, &o, loglik, Mode::PRODUCTS, nullptr, stream);
+                                obs->tremor, &o, loglik, Mode::PATH, nullptr, stream);
     if (rc) return rc;
     const Plan &pl = c->plan;
-    const int KP = pl.lay.KP, C = std::max(1, pl.n_chunks);
+    const int K = prm->K, KP = pl.lay.KP;
+    const size_t C = std::max(1, pl.n_chunks), n = pl.strand_kp ? pl.strands.size() : 0, kp = (size_t)pl.strand_kp;
     WorkPtrs wp;
     carve_work(c->work.p, 1, 1, pl.lay, pl, &wp);
-    Carve cv(nullptr);
-    cv.take<float>((size_t)C * KP * KP);
-    cv.take<double>((size_t)C * KP);
-    cv.take<int32_t>((size_t)C * KP);
-    cv.take<int32_t>((size_t)C + 1);
-    cv.take<uint8_t>((size_t)C * pl.L * KP);
-    rc = ensure(c, c->fb, cv.off + 1024);
+    VitPtrs vp;
+    float *V = nullptr;
+    double *voff = nullptr;
+    int32_t *ptr = nullptr, *bstate = nullptr;
+    uint8_t *bp = nullptr;
+    auto carve = [&](void *base) {
+        Carve cv(base);
+        V = cv.take<float>(C * KP * KP);
+        voff = cv.take<double>(C * KP);
+        ptr = cv.take<int32_t>(C * KP);
+        bstate = cv.take<int32_t>(C + 1);
+        bp = cv.take<uint8_t>(C * pl.L * KP);
+        if (n) {
+            vp.lp = cv.take<float>(kp * kp);
+            vp.lp64 = cv.take<double>(kp * kp);
+            vp.em64 = cv.take<double>((size_t)K * 8);
+            vp.vs = cv.take<float>(n * kp);
+            vp.ve = cv.take<float>(n * kp);
+            vp.carry = cv.take<float>(n * kp);
+            vp.unmet = cv.take<int>(n);
+            vp.bstate = cv.take<int>(n);
+            vp.map = cv.take<uint8_t>(n * kp);
+            vp.bp = cv.take<uint8_t>((size_t)pl.n_packed * kp);
+            vp.part = cv.take<double>(n);
+            vp.chunks = cv.take<int>(1);
+        }
+        return cv.off;
+    };
+    rc = ensure(c, c->fb, carve(nullptr) + 1024);
     if (rc) return rc;
-    Carve vc(c->fb.p);
-    float *V = vc.take<float>((size_t)C * KP * KP);
-    double *voff = vc.take<double>((size_t)C * KP);
-    int32_t *ptr = vc.take<int32_t>((size_t)C * KP);
-    int32_t *bstate = vc.take<int32_t>((size_t)C + 1);
-    uint8_t *bp = vc.take<uint8_t>((size_t)C * pl.L * KP);
-    cudaError_t e = launch_viterbi(prm->K, o.init_mode, pl.n_chunks, pl.L, pl.lay, pl.d_chunks, prm->pi, prm->P,
-                                   wp.cblock, wp.head, wp.packed, V, voff, ptr, bstate, bp, path, score,
-                                   (cudaStream_t)stream);
+    carve(c->fb.p);
+    cudaError_t e = cudaSuccess;
+    if (n) {
+        e = launch_vit_strands(K, pl.strand_kp, o.init_mode, pl.lay, wp.cblock, prm->pi, prm->P, prm->p_tremor, prm->mu,
+                               prm->cov, wp.head, wp.packed, wp.sp, vp, path, score, (cudaStream_t)stream);
+        c->last_launches += 8;
+    }
+    if (e == cudaSuccess)
+        e = launch_viterbi(K, o.init_mode, pl.n_chunks, pl.L, pl.lay, pl.d_chunks, prm->pi, prm->P, wp.cblock, wp.head,
+                           wp.packed, V, voff, ptr, bstate, bp, path, score, vp.chunks, (cudaStream_t)stream);
     c->last_launches += pl.n_chunks > 0 ? 3 : 2;
     if (e != cudaSuccess) return cuda_fail(c, e, "viterbi launch");
     return HMM_OK;

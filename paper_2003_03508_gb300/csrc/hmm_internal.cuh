@@ -115,6 +115,22 @@ struct SmoothPtrs {
     double *stats = nullptr;   // K K + 8 K, as hmm_expected_stats
 };
 
+// The most probable path by strands (hmm_vit_strand.cu). Row i belongs to step i.
+struct VitPtrs {
+    float *lp = nullptr;       // [KP][KP] log2 P
+    double *lp64 = nullptr;    // [KP][KP] log P
+    double *em64 = nullptr;    // [K][8] emission constants of the score
+    float *vs = nullptr;       // [n][KP] vector at the piece's start
+    float *ve = nullptr;       // [n][KP] and at its end
+    float *carry = nullptr;    // [n][KP] true vector where a piece ended unmet
+    int *unmet = nullptr;      // [n] 2 x rows written again, + 1 where the piece ended first
+    int *bstate = nullptr;     // [n] state at the piece's end
+    uint8_t *map = nullptr;    // [n][KP] leaving state -> state before the piece
+    uint8_t *bp = nullptr;     // [steps][KP] back-pointers
+    double *part = nullptr;    // [n] the pieces' parts of the score
+    int *chunks = nullptr;     // set: the chunk products take the sequence
+};
+
 struct ConstLayout {
     int KP;         // padded state count used by the chunk kernel
     int off_emis;   // EM_ALL * KP floats
@@ -194,6 +210,10 @@ cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayo
                                const StrandPtrs &sp, float *alpha, cudaStream_t st);
 cudaError_t launch_smooth(int K, int KP, int64_t steps, const ConstLayout &lay, const float *cblock, const float2 *head,
                           const float2 *packed, const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st);
+cudaError_t launch_vit_strands(int K, int KP, int init_mode, const ConstLayout &lay, const float *cb, const float *pi,
+                               const float *P, const float *p, const float *mu, const float *cov, const float2 *head,
+                               const float2 *packed, const StrandPtrs &sp, const VitPtrs &vp, int32_t *path,
+                               double *score, cudaStream_t st);
 int strand_mma_per_warp(int KP);
 cudaError_t launch_strand_mma(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                               const float *cblock, const float *pi, const float2 *head, const float2 *packed,
@@ -224,7 +244,7 @@ int chunk_tc_wide_chunks_per_item(int KP, int precision);
 cudaError_t launch_viterbi(int K, int init_mode, int n_chunks, int L, const ConstLayout &lay, const ChunkDesc *chunks,
                            const float *pi, const float *P, const float *cblock, const float2 *head,
                            const float2 *packed, float *V, double *voff, int32_t *ptr, int32_t *bstate, uint8_t *bp,
-                           int32_t *path, double *score, cudaStream_t st);
+                           int32_t *path, double *score, const int *todo, cudaStream_t st);
 cudaError_t launch_chunk_tc_wide(int n_prop, int n_chunks, int renorm, int precision, const ConstLayout &lay,
                                  const float *cblock, const ChunkDesc *chunks, const float2 *packed, float *A0,
                                  int32_t *e0, unsigned *status, const int *todo, cudaStream_t st);

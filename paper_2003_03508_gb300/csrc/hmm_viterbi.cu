@@ -27,7 +27,8 @@ template <int KP, int CPC>
 __global__ void __launch_bounds__(KP *CPC)
 vit_chunk_kernel(int n_chunks, ConstLayout lay, const float *__restrict__ cblock,
                  const ChunkDesc *__restrict__ chunks, const float2 *__restrict__ packed, float *__restrict__ V,
-                 double *__restrict__ voff) {
+                 double *__restrict__ voff, const int *__restrict__ todo) {
+    if (todo && *todo == 0) return;  // done by strands
     __shared__ float sLP[KP * KP];
     __shared__ float sEm[EM_ROWS * KP];
     __shared__ float sL[CPC][KP];
@@ -111,7 +112,8 @@ __global__ void __launch_bounds__(VT) vit_scan_kernel(int K, int KP, int init_mo
                                                       const float *__restrict__ em, const float2 *__restrict__ head,
                                                       const float *__restrict__ V, const double *__restrict__ voff,
                                                       int32_t *__restrict__ ptr, int32_t *__restrict__ bstate,
-                                                      double *__restrict__ score) {
+                                                      double *__restrict__ score, const int *__restrict__ todo) {
+    if (todo && *todo == 0) return;
     __shared__ double d[128];
     __shared__ double red[VT];
     __shared__ int ired[VT];
@@ -187,7 +189,8 @@ __global__ void __launch_bounds__(VT) vit_path_kernel(int K, int KP, int L, cons
                                                       const float *__restrict__ cblock, ConstLayout lay,
                                                       const float2 *__restrict__ packed,
                                                       const int32_t *__restrict__ bstate, uint8_t *__restrict__ bp,
-                                                      int32_t *__restrict__ path) {
+                                                      int32_t *__restrict__ path, const int *__restrict__ todo) {
+    if (todo && *todo == 0) return;
     extern __shared__ float sLP[];  // K x K log2 P
     float *sd = sLP + K * K;        // K
     float *red = sd + K;            // VT
@@ -243,9 +246,9 @@ __global__ void __launch_bounds__(VT) vit_path_kernel(int K, int KP, int L, cons
 
 template <int KP, int CPC>
 cudaError_t launch_vit_chunk_t(int n_chunks, const ConstLayout &lay, const float *cblock, const ChunkDesc *chunks,
-                               const float2 *packed, float *V, double *voff, cudaStream_t st) {
+                               const float2 *packed, float *V, double *voff, const int *todo, cudaStream_t st) {
     const int blocks = (n_chunks + CPC - 1) / CPC;
-    vit_chunk_kernel<KP, CPC><<<blocks, KP * CPC, 0, st>>>(n_chunks, lay, cblock, chunks, packed, V, voff);
+    vit_chunk_kernel<KP, CPC><<<blocks, KP * CPC, 0, st>>>(n_chunks, lay, cblock, chunks, packed, V, voff, todo);
     return cudaGetLastError();
 }
 
@@ -254,24 +257,24 @@ cudaError_t launch_vit_chunk_t(int n_chunks, const ConstLayout &lay, const float
 cudaError_t launch_viterbi(int K, int init_mode, int n_chunks, int L, const ConstLayout &lay, const ChunkDesc *chunks,
                            const float *pi, const float *P, const float *cblock, const float2 *head,
                            const float2 *packed, float *V, double *voff, int32_t *ptr, int32_t *bstate, uint8_t *bp,
-                           int32_t *path, double *score, cudaStream_t st) {
+                           int32_t *path, double *score, const int *todo, cudaStream_t st) {
     const int KP = lay.KP;
     cudaError_t e = cudaSuccess;
     if (n_chunks > 0) {
         switch (KP) {
-            case 4: e = launch_vit_chunk_t<4, 32>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 8: e = launch_vit_chunk_t<8, 16>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 16: e = launch_vit_chunk_t<16, 8>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 32: e = launch_vit_chunk_t<32, 4>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 48: e = launch_vit_chunk_t<48, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 64: e = launch_vit_chunk_t<64, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
-            case 80: e = launch_vit_chunk_t<80, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, st); break;
+            case 4: e = launch_vit_chunk_t<4, 32>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 8: e = launch_vit_chunk_t<8, 16>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 16: e = launch_vit_chunk_t<16, 8>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 32: e = launch_vit_chunk_t<32, 4>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 48: e = launch_vit_chunk_t<48, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 64: e = launch_vit_chunk_t<64, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
+            case 80: e = launch_vit_chunk_t<80, 2>(n_chunks, lay, cblock, chunks, packed, V, voff, todo, st); break;
             default: return cudaErrorInvalidValue;
         }
         if (e != cudaSuccess) return e;
     }
     vit_scan_kernel<<<1, VT, 0, st>>>(K, KP, init_mode, n_chunks, pi, P, cblock + lay.off_emis, head, V, voff, ptr,
-                                      bstate, score);
+                                      bstate, score, todo);
     if (n_chunks == 0) {
         // one observation: the path is the best entering state
         return cudaMemcpyAsync(path, bstate, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
@@ -279,7 +282,7 @@ cudaError_t launch_viterbi(int K, int init_mode, int n_chunks, int L, const Cons
     const size_t smem = sizeof(float) * ((size_t)K * K + K + VT);
     e = cudaFuncSetAttribute(vit_path_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    vit_path_kernel<<<n_chunks, VT, smem, st>>>(K, KP, L, chunks, cblock, lay, packed, bstate, bp, path);
+    vit_path_kernel<<<n_chunks, VT, smem, st>>>(K, KP, L, chunks, cblock, lay, packed, bstate, bp, path, todo);
     return cudaGetLastError();
 }
 
