@@ -18,8 +18,8 @@
 // terms that do not depend on the network dropped). Optimiser: Adam
 // (Kingma & Ba, ICLR 2015) with bias correction.
 //
-// All GEMMs are FP32 SIMT tiles: the network costs about 1 MFLOP per chain
-// and iteration, against ~10^10 for one likelihood evaluation.
+// All products are FP32 on the CUDA cores: the network costs about 1 MFLOP per
+// chain and iteration.
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -31,58 +31,160 @@ namespace mlp {
 
 constexpr float FSIG_LO = -6.0f, FSIG_HI = 3.0f;
 
-// C[m][n] = alpha * sum_k A(m,k) B(k,n) (+ bias[n]) (relu), beta C + ...
+// C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n]) (relu) (zero where mask[m][n] <= 0)
 // A(m,k) = TA ? A[k*lda + m] : A[m*lda + k];  B(k,n) = TB ? B[n*ldb + k] : B[k*ldb + n]
+// With `colsum` the CTAs of the first column block also write sum_k A(m,k).
+//
+// One CTA per 32 x 32 block of C, 256 threads as four slices of the k range of
+// a tile, 4 x 4 outputs a thread, the next tile's loads in flight while the
+// present one is multiplied. The matrices are small (512 x 256 x 351): what
+// counts is the latency of the k loop, not the FMA rate, so the slices shorten
+// it fourfold: 12 us a product of 512 x 256 x 256, about 25 with a thread per
+// four outputs and 32 k steps a tile. (Standardising the input as it is loaded
+// was tried: its divisions stand in the loop, 34 us a product, so a pass of its
+// own does it.)
 constexpr int TILE = 32;
 
+struct Gemm {
+    int M, N, K;
+    const float *A;
+    int lda, ta;
+    const float *B;
+    int ldb, tb;
+    float *C;
+    int ldc;
+    const float *bias = nullptr;
+    int relu = 0;
+    const float *mask = nullptr;     // [M][N], row stride ldc
+    float *colsum = nullptr;         // [M]
+};
+
+struct GemmShared {
+    float a[TILE * 36], b[TILE * 36], red[3][TILE * TILE];
+};
+
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(TILE * 8) gemm_kernel(int M, int N, int K, const float *__restrict__ A, int lda,
-                                                         const float *__restrict__ B, int ldb, float *__restrict__ C,
-                                                         int ldc, const float *__restrict__ bias, int relu,
-                                                         float beta) {
-    __shared__ float sA[TILE][TILE + 1];
-    __shared__ float sB[TILE][TILE + 1];
-    const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;  // 32 x 8 threads, 4 rows each
-    const int m0 = blockIdx.y * TILE, n0 = blockIdx.x * TILE;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k0 = 0; k0 < K; k0 += TILE) {
-        for (int r = ty; r < TILE; r += 8) {
-            const int m = m0 + r, k = k0 + tx;
-            sA[r][tx] = (m < M && k < K) ? (TA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k]) : 0.f;
-            const int kk = k0 + r, n = n0 + tx;
-            sB[r][tx] = (kk < K && n < N) ? (TB ? B[(size_t)n * ldb + kk] : B[(size_t)kk * ldb + n]) : 0.f;
+__device__ __forceinline__ void gemm_tile(const Gemm &g, int bx, int by, GemmShared &sh) {
+    // operands as the loads find them: [k][i] rows where the index along i is
+    // contiguous in memory, else [i][k] (odd stride)
+    float *const sA = sh.a, *const sB = sh.b;
+    float(*const red)[TILE * TILE] = sh.red;
+    const int tid = threadIdx.x;
+    const int m0 = by * TILE, n0 = bx * TILE;
+    const int lx = tid % TILE, ly = tid / TILE;  // loads: 8 rows at a time
+    const int ks = tid >> 6, t = tid & 63, tm = (t >> 3) * 4, tn = (t & 7) * 4;
+    float ra[4], rb[4];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int y = ly + 8 * r;
+            const int m = TA ? m0 + lx : m0 + y, ka = TA ? k0 + y : k0 + lx;
+            float v = 0.0f;
+            if (m < g.M && ka < g.K) v = TA ? g.A[(size_t)ka * g.lda + m] : g.A[(size_t)m * g.lda + ka];
+            ra[r] = v;
+            const int n = TB ? n0 + y : n0 + lx, kb = TB ? k0 + lx : k0 + y;
+            v = 0.0f;
+            if (n < g.N && kb < g.K) v = TB ? g.B[(size_t)n * g.ldb + kb] : g.B[(size_t)kb * g.ldb + n];
+            rb[r] = v;
+        }
+    };
+    float acc[4][4] = {};
+    float csum = 0.0f;  // thread tid < 32: row m0 + tid of A
+    const bool sums = g.colsum && bx == 0;
+    load(0);
+    for (int k0 = 0; k0 < g.K; k0 += TILE) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int y = ly + 8 * r;
+            sA[TA ? y * 36 + lx : y * 33 + lx] = ra[r];
+            sB[TB ? y * 33 + lx : y * 36 + lx] = rb[r];
         }
         __syncthreads();
+        if (k0 + TILE < g.K) load(k0 + TILE);
+#pragma unroll
+        for (int j = 0; j < TILE / 4; ++j) {
+            const int k = ks * (TILE / 4) + j;
+            float a[4], b[4];
+            if (TA) {
+                const float4 v = *reinterpret_cast<const float4 *>(&sA[k * 36 + tm]);
+                a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i] = sA[(tm + i) * 33 + k];
+            }
+            if (!TB) {
+                const float4 v = *reinterpret_cast<const float4 *>(&sB[k * 36 + tn]);
+                b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) b[i] = sB[(tn + i) * 33 + k];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int l = 0; l < 4; ++l) acc[i][l] = fmaf(a[i], b[l], acc[i][l]);
+        }
+        if (sums && tid < TILE) {
 #pragma unroll 8
-        for (int k = 0; k < TILE; ++k) {
-            const float b = sB[k][tx];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] = fmaf(sA[ty + 8 * i][k], b, acc[i]);
+            for (int k = 0; k < TILE; ++k) csum += sA[TA ? k * 36 + tid : tid * 33 + k];
         }
         __syncthreads();
     }
-    const int n = n0 + tx;
-    if (n >= N) return;
+    // the four slices' sums, in order
+    if (ks) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty + 8 * i;
-        if (m >= M) continue;
-        float v = acc[i];
-        if (bias) v += bias[n];
-        if (relu) v = fmaxf(v, 0.f);
-        float *c = C + (size_t)m * ldc + n;
-        *c = beta != 0.f ? beta * *c + v : v;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) red[ks - 1][(tm + i) * TILE + tn + l] = acc[i][l];
     }
+    __syncthreads();
+    if (ks == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                const int m = m0 + tm + i, n = n0 + tn + l, x = (tm + i) * TILE + tn + l;
+                if (m >= g.M || n >= g.N) continue;
+                float v = ((acc[i][l] + red[0][x]) + red[1][x]) + red[2][x];
+                if (g.bias) v += g.bias[n];
+                if (g.relu) v = fmaxf(v, 0.0f);
+                if (g.mask && !(g.mask[(size_t)m * g.ldc + n] > 0.0f)) v = 0.0f;
+                g.C[(size_t)m * g.ldc + n] = v;
+            }
+    }
+    if (sums && tid < TILE && m0 + tid < g.M) g.colsum[m0 + tid] = csum;
 }
 
-static cudaError_t gemm(bool ta, bool tb, int M, int N, int K, const float *A, int lda, const float *B, int ldb,
-                        float *C, int ldc, const float *bias, int relu, float beta, cudaStream_t st) {
-    dim3 grid((N + TILE - 1) / TILE, (M + TILE - 1) / TILE), block(TILE * 8);
-    if (!ta && !tb) gemm_kernel<false, false><<<grid, block, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, beta);
-    else if (!ta && tb) gemm_kernel<false, true><<<grid, block, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, beta);
-    else if (ta && !tb) gemm_kernel<true, false><<<grid, block, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, beta);
-    else gemm_kernel<true, true><<<grid, block, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, relu, beta);
+// one or two independent products in one launch (blockIdx.z)
+__global__ void __launch_bounds__(256) gemm_kernel(Gemm g0, Gemm g1) {
+    __shared__ __align__(16) GemmShared sh;
+    const Gemm &g = blockIdx.z ? g1 : g0;
+    const int bx = blockIdx.x, by = blockIdx.y;
+    if (bx * TILE >= g.N || by * TILE >= g.M) return;
+    if (g.ta) gemm_tile<true, false>(g, bx, by, sh);
+    else if (g.tb) gemm_tile<false, true>(g, bx, by, sh);
+    else gemm_tile<false, false>(g, bx, by, sh);
+}
+
+static cudaError_t gemm(const Gemm &g, cudaStream_t st) {
+    gemm_kernel<<<dim3((g.N + TILE - 1) / TILE, (g.M + TILE - 1) / TILE, 1), 256, 0, st>>>(g, g);
     return cudaGetLastError();
+}
+
+static cudaError_t gemm2(const Gemm &a, const Gemm &b, cudaStream_t st) {
+    const int nx = ((a.N > b.N ? a.N : b.N) + TILE - 1) / TILE, ny = ((a.M > b.M ? a.M : b.M) + TILE - 1) / TILE;
+    gemm_kernel<<<dim3(nx, ny, 2), 256, 0, st>>>(a, b);
+    return cudaGetLastError();
+}
+
+static Gemm product(bool ta, bool tb, int M, int N, int K, const float *A, int lda, const float *B, int ldb, float *C,
+                    int ldc) {
+    Gemm g{};
+    g.M = M; g.N = N; g.K = K;
+    g.A = A; g.lda = lda; g.ta = ta;
+    g.B = B; g.ldb = ldb; g.tb = tb;
+    g.C = C; g.ldc = ldc;
+    return g;
 }
 
 // x = (theta - m) / s
@@ -135,21 +237,6 @@ __global__ void mean_kernel(int B, const double *v, double *out) {
         __syncthreads();
     }
     if (threadIdx.x == 0) *out = red[0] / B;
-}
-
-// dZ = dA * (Z > 0) in place on dA (the forward kept post-activation A; A > 0 iff Z > 0)
-__global__ void relu_back_kernel(size_t n, const float *act, float *grad) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (!(act[i] > 0.f)) grad[i] = 0.f;
-}
-
-// db[n] = sum_b dZ[b][n]
-__global__ void colsum_kernel(int B, int N, const float *dz, float *db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += dz[(size_t)b * N + n];
-    db[n] = s;
 }
 
 __global__ void adam_kernel(size_t n, float *p, const float *g, float *m, float *v, float lr, float b1, float b2,
@@ -244,55 +331,53 @@ static int ensure_batch(hmm_mlp *m, int B) {
     return HMM_OK;
 }
 
-// forward of B standardised rows x into out, through the given activation buffers
-static cudaError_t forward_ext(hmm_mlp *m, int B, const float *x, float *a1, float *a2, float *out, cudaStream_t st) {
+// forward of B states theta into out, through the given buffers
+static cudaError_t forward_ext(hmm_mlp *m, int B, const float *theta, float *x, float *a1, float *a2, float *out,
+                               cudaStream_t st) {
     const int d = m->d, H = m->H;
-    cudaError_t e = gemm(false, true, B, H, d, x, d, m->W1(), d, a1, H, m->b1(), 1, 0.f, st);
-    if (e == cudaSuccess) e = gemm(false, true, B, H, H, a1, H, m->W2(), H, a2, H, m->b2(), 1, 0.f, st);
-    if (e == cudaSuccess) e = gemm(false, true, B, 2 * d, H, a2, H, m->W3(), H, out, 2 * d, m->b3(), 0, 0.f, st);
+    standardise_kernel<<<(unsigned)(((size_t)B * d + 255) / 256), 256, 0, st>>>(B, d, theta, m->mean, m->in_scale, x);
+    Gemm g1 = product(false, true, B, H, d, x, d, m->W1(), d, a1, H);
+    g1.bias = m->b1();
+    g1.relu = 1;
+    Gemm g2 = product(false, true, B, H, H, a1, H, m->W2(), H, a2, H);
+    g2.bias = m->b2();
+    g2.relu = 1;
+    Gemm g3 = product(false, true, B, 2 * d, H, a2, H, m->W3(), H, out, 2 * d);
+    g3.bias = m->b3();
+    cudaError_t e = gemm(g1, st);
+    if (e == cudaSuccess) e = gemm(g2, st);
+    if (e == cudaSuccess) e = gemm(g3, st);
     return e;
 }
 
-// forward of B standardised rows (m->x) into m->out; activations kept for backward
-static cudaError_t forward(hmm_mlp *m, int B, cudaStream_t st) { return forward_ext(m, B, m->x, m->a1, m->a2, m->out, st); }
-
-// gradients of the loss wrt every parameter from dout (m->grads, same layout)
+// gradients of the loss wrt every parameter from dout (m->grads, same layout);
+// A > 0 iff Z > 0 for the kept activations
 static cudaError_t backward(hmm_mlp *m, int B, cudaStream_t st) {
     const int d = m->d, H = m->H;
     float *g = m->grads;
     float *gW1 = g, *gb1 = gW1 + (size_t)H * d, *gW2 = gb1 + H, *gb2 = gW2 + (size_t)H * H, *gW3 = gb2 + H,
           *gb3 = gW3 + (size_t)2 * d * H;
-    // layer 3: dW3 = dout^T a2, db3 = colsum dout, d2 = dout W3 (then relu')
-    cudaError_t e = gemm(true, false, 2 * d, H, B, m->dout, 2 * d, m->a2, H, gW3, H, nullptr, 0, 0.f, st);
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(2 * d + 127) / 128, 128, 0, st>>>(B, 2 * d, m->dout, gb3);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = gemm(false, false, B, H, 2 * d, m->dout, 2 * d, m->W3(), H, m->d2, H, nullptr, 0, 0.f, st);
-    if (e == cudaSuccess) {
-        relu_back_kernel<<<256, 256, 0, st>>>((size_t)B * H, m->a2, m->d2);
-        e = gemm(true, false, H, H, B, m->d2, H, m->a1, H, gW2, H, nullptr, 0, 0.f, st);
-    }
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(H + 127) / 128, 128, 0, st>>>(B, H, m->d2, gb2);
-        e = gemm(false, false, B, H, H, m->d2, H, m->W2(), H, m->d1, H, nullptr, 0, 0.f, st);
-    }
-    if (e == cudaSuccess) {
-        relu_back_kernel<<<256, 256, 0, st>>>((size_t)B * H, m->a1, m->d1);
-        e = gemm(true, false, H, d, B, m->d1, H, m->x, d, gW1, d, nullptr, 0, 0.f, st);
-    }
-    if (e == cudaSuccess) {
-        colsum_kernel<<<(H + 127) / 128, 128, 0, st>>>(B, H, m->d1, gb1);
-        e = cudaGetLastError();
-    }
+    // layer 3: dW3 = dout^T a2, db3 = column sums of dout, and d2 = dout W3 where a2 > 0
+    Gemm w3 = product(true, false, 2 * d, H, B, m->dout, 2 * d, m->a2, H, gW3, H);
+    w3.colsum = gb3;
+    Gemm d2 = product(false, false, B, H, 2 * d, m->dout, 2 * d, m->W3(), H, m->d2, H);
+    d2.mask = m->a2;
+    Gemm w2 = product(true, false, H, H, B, m->d2, H, m->a1, H, gW2, H);
+    w2.colsum = gb2;
+    Gemm d1 = product(false, false, B, H, H, m->d2, H, m->W2(), H, m->d1, H);
+    d1.mask = m->a1;
+    Gemm w1 = product(true, false, H, d, B, m->d1, H, m->x, d, gW1, d);
+    w1.colsum = gb1;
+    cudaError_t e = gemm2(w3, d2, st);
+    if (e == cudaSuccess) e = gemm2(w2, d1, st);
+    if (e == cudaSuccess) e = gemm(w1, st);
     return e;
 }
 
 static int loss_and_grad(hmm_mlp *m, int B, const float *theta, const float *y, double *loss_dev, cudaStream_t st) {
     int rc = ensure_batch(m, B);
     if (rc) return rc;
-    standardise_kernel<<<256, 256, 0, st>>>(B, m->d, theta, m->mean, m->in_scale, m->x);
-    cudaError_t e = forward(m, B, st);
+    cudaError_t e = forward_ext(m, B, theta, m->x, m->a1, m->a2, m->out, st);
     if (e == cudaSuccess) {
         loss_grad_kernel<<<B, 128, 0, st>>>(B, m->d, theta, y, m->scale, m->out, m->dout, m->rowloss);
         mean_kernel<<<1, 256, 0, st>>>(B, m->rowloss, loss_dev);
@@ -389,10 +474,7 @@ int hmm_mlp_forward(hmm_mlp *m, int32_t B, const float *theta, float *out_dev, v
     cudaStream_t st = (cudaStream_t)stream;
     int rc = ensure_batch(m, B);
     if (rc) return rc;
-    standardise_kernel<<<256, 256, 0, st>>>(B, m->d, theta, m->mean, m->in_scale, m->x);
-    cudaError_t e = forward(m, B, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out_dev, m->out, sizeof(float) * B * 2 * m->d, cudaMemcpyDeviceToDevice, st);
+    const cudaError_t e = forward_ext(m, B, theta, m->x, m->a1, m->a2, out_dev, st);
     return e == cudaSuccess ? HMM_OK : HMM_ECUDA;
 }
 
@@ -459,8 +541,7 @@ cudaError_t mlp_state_io(hmm_mlp *m, float *host, float *lam, float *drift, bool
 // network outputs for B states into out (B x 2d) through caller-owned buffers
 // x [B][d], a1 and a2 [B][H] (their addresses stay fixed under a CUDA graph)
 int mlp_eval(hmm_mlp *m, int B, const float *theta, float *x, float *a1, float *a2, float *out, cudaStream_t st) {
-    standardise_kernel<<<256, 256, 0, st>>>(B, m->d, theta, m->mean, m->in_scale, x);
-    return forward_ext(m, B, x, a1, a2, out, st) == cudaSuccess ? HMM_OK : HMM_ECUDA;
+    return forward_ext(m, B, theta, x, a1, a2, out, st) == cudaSuccess ? HMM_OK : HMM_ECUDA;
 }
 
 }  // namespace hmm
