@@ -861,9 +861,12 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         launches = 0;
         prof_mark(c, HMM_PHASE_PREP, s);
         cudaError_t r = cudaMemsetAsync(obs_bad, 0, 2 * sizeof(int), s);
-        if (r == cudaSuccess) { r = launch_prep(n_prop, K, lay, prec, opts.init_mode, pi, P, p, mu, cov, cblock, prop_bad, c->d_status, sp, s); ++launches; }
-        prof_mark(c, HMM_PHASE_PACK, s);
-        if (r == cudaSuccess && T_total > 0) { r = launch_pack(n_seg, pl.d_offsets, pl.d_pbase, T_total, xy, tremor, packed, head, obs_bad, c->d_status, s); ++launches; }
+        if (r == cudaSuccess) {
+            r = launch_prep_pack(n_prop, K, lay, prec, pi, P, p, mu, cov, cblock, prop_bad, sp, n_seg, pl.d_offsets,
+                                 pl.d_pbase, T_total, xy, tremor, packed, head, obs_bad, c->d_status, s);
+            ++launches;
+        }
+        prof_mark(c, HMM_PHASE_PACK, s);  // (in the same launch)
         prof_mark(c, HMM_PHASE_CHUNK, s);
         if (r == cudaSuccess && sp.n > 0) {
             if (pl.strand_tensor) r = launch_strand_mma(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);

@@ -188,14 +188,11 @@ __device__ __forceinline__ float log2_emission(const float *__restrict__ em, int
 
 ConstLayout make_layout(int K, int precision);
 
-cudaError_t launch_prep(int n_prop, int K, const ConstLayout &lay, int precision, int init_mode,
-                        const float *pi, const float *P, const float *p, const float *mu,
-                        const float *cov, float *cblock, int *prop_bad, unsigned *status,
-                        const StrandPtrs &sp, cudaStream_t st);
-
-cudaError_t launch_pack(int n_seg, const int64_t *d_offsets, const int64_t *d_pbase,
-                        int64_t T_total, const float *xy, const uint8_t *tremor, float2 *packed,
-                        float2 *head, int *obs_bad, unsigned *status, cudaStream_t st);
+cudaError_t launch_prep_pack(int n_prop, int K, const ConstLayout &lay, int precision, const float *pi,
+                             const float *P, const float *p, const float *mu, const float *cov, float *cblock,
+                             int *prop_bad, const StrandPtrs &sp, int n_seg, const int64_t *d_offsets,
+                             const int64_t *d_pbase, int64_t T_total, const float *xy, const uint8_t *tremor,
+                             float2 *packed, float2 *head, int *obs_bad, unsigned *status, cudaStream_t st);
 
 cudaError_t launch_chunk_simt(int n_prop, int n_chunks, int L, int renorm, const ConstLayout &lay,
                               const float *cblock, const ChunkDesc *chunks, const float2 *packed,

@@ -202,10 +202,9 @@ extern "C" int hmm_loglik_noalloc(const hmm_params *prm, const hmm_obs *obs, dou
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = launch_prep(1, K, lay, HMM_PREC_FP32_SIMT, 0, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov,
-                        cblock, prop_bad, status, StrandPtrs{}, st);
-    if (e == cudaSuccess && T > 0)
-        e = launch_pack(1, offs, pbase, T, obs->xy, obs->tremor, packed, head, obs_bad, status, st);
+        e = launch_prep_pack(1, K, lay, HMM_PREC_FP32_SIMT, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, cblock,
+                             prop_bad, StrandPtrs{}, 1, offs, pbase, T, obs->xy, obs->tremor, packed, head, obs_bad,
+                             status, st);
     if (e == cudaSuccess && C > 0)
         e = launch_chunk_simt(1, C, NA_L, 4, lay, cblock, chunks, packed, lv.A[0], (int32_t *)lv.e[0], status, nullptr, st);
     int gbase = 0;

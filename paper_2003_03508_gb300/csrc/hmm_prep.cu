@@ -1,7 +1,7 @@
 // Parameter preparation and observation packing.
 //
 // prep (one CTA per proposal): checks a parameter set and turns it into the
-// constants the chunk kernels read -- the emission coefficients of Eq.
+// constants the later kernels read -- the emission coefficients of Eq.
 // "emission-matrix" in the log2 domain, P padded to KP x KP, and the
 // tensor-core operand images of P.
 //
@@ -55,12 +55,15 @@ __device__ __forceinline__ int kmajor_offset(int n, int k, int KP, int elems16) 
 
 constexpr int PREP_THREADS = 256;
 
-__global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout lay, int precision, const float *__restrict__ pi,
-                            const float *__restrict__ P, const float *__restrict__ p,
-                            const float *__restrict__ mu, const float *__restrict__ cov,
-                            float *__restrict__ cblock, int *__restrict__ prop_bad,
-                            unsigned *__restrict__ status, StrandPtrs sp) {
-    const int q = blockIdx.x;
+// One proposal's constants, by one CTA. FP64 is two lanes per cycle and SM here,
+// so the chain of a state's logarithms and square roots is spread over four
+// threads (14 us for a lone proposal when one thread took them in turn).
+__device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &lay, int precision,
+                                              const float *__restrict__ pi, const float *__restrict__ P,
+                                              const float *__restrict__ p, const float *__restrict__ mu,
+                                              const float *__restrict__ cov, float *__restrict__ cblock,
+                                              int *__restrict__ prop_bad, unsigned *__restrict__ status,
+                                              const StrandPtrs &sp) {
     const int KP = lay.KP;
     pi += (size_t)q * K;
     P += (size_t)q * K * K;
@@ -68,32 +71,70 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout l
     mu += (size_t)q * 2 * K;
     cov += (size_t)q * 3 * K;
     float *cb = cblock + (size_t)q * lay.stride;
-    __shared__ int bad, small;
-    __shared__ float centre[2];
-    if (threadIdx.x == 0) bad = small = 0;
-    if (threadIdx.x < 32) {
+    float *em = cb + lay.off_emis;
+    __shared__ float s_ctr[80], s_cno[80], s_centre[2];
+    const int lane = threadIdx.x & 31;
+    bool bad = false, small = false;
+
+    // per-state emission constants (log2 domain), padded states emit nothing
+    const double LOG2E = 1.4426950408889634074;
+    const double LOG2_2PI = 2.6514961294723187980;
+    const int job = threadIdx.x >> 6;
+    float cx = 0.0f, cy = 0.0f;
+    if (job == 3) {
         // the states' centre: the strands take coordinates from it
-        float sx = 0.0f, sy = 0.0f;
-        for (int k = threadIdx.x; k < K; k += 32) {
-            sx += mu[2 * k] / (float)K;
-            sy += mu[2 * k + 1] / (float)K;
+        for (int k = lane; k < K; k += 32) {
+            cx += mu[2 * k] / (float)K;
+            cy += mu[2 * k + 1] / (float)K;
         }
         for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+            cx += __shfl_xor_sync(0xffffffffu, cx, o);
+            cy += __shfl_xor_sync(0xffffffffu, cy, o);
         }
-        if (threadIdx.x == 0) {
-            centre[0] = sx;
-            centre[1] = sy;
+        if (threadIdx.x == 192) {
+            s_centre[0] = cx;
+            s_centre[1] = cy;
         }
     }
-    __syncthreads();
-
+    for (int k = threadIdx.x & 63; k < KP; k += 64) {
+        const bool in = k < K;
+        const double pk = in ? p[k] : 0.0;
+        const double sxx = in ? cov[3 * k] : 1.0, sxy = in ? cov[3 * k + 1] : 0.0, syy = in ? cov[3 * k + 2] : 1.0;
+        const double det = sxx * syy - sxy * sxy;
+        const float mx = in ? mu[2 * k] : 0.0f, my = in ? mu[2 * k + 1] : 0.0f;
+        const bool ok = isfinite(pk) && pk >= 0.0 && pk <= 1.0 && isfinite(sxx) && isfinite(sxy) && isfinite(syy) &&
+                        sxx > 0.0 && syy > 0.0 && det > 0.0 && isfinite(mx) && isfinite(my);
+        if (!ok) bad = true;
+        const bool use = in && ok;
+        if (job == 0) {
+            em[EM_MUX * KP + k] = use ? mx : 0.0f;
+            em[EM_MUY * KP + k] = use ? my : 0.0f;
+            em[EM_QA * KP + k] = use ? (float)(-0.5 * LOG2E * syy / det) : 0.0f;
+            em[EM_QB * KP + k] = use ? (float)(LOG2E * sxy / det) : 0.0f;
+            em[EM_QC * KP + k] = use ? (float)(-0.5 * LOG2E * sxx / det) : 0.0f;
+        } else if (job == 1) {
+            const float v = use ? (float)(0.5 * log2(pk * pk / det) - LOG2_2PI) : -INFINITY;
+            em[EM_CTR * KP + k] = v;
+            s_ctr[k] = v;
+        } else if (job == 2) {
+            const float v = use ? (float)log2(1.0 - pk) : -INFINITY;
+            em[EM_CNO * KP + k] = v;
+            s_cno[k] = v;
+        } else {
+            // the quadratic form as two squares (Cholesky factor of the precision matrix)
+            const double ux = use ? sqrt(0.5 * LOG2E * syy / det) : 0.0, wy = use ? sqrt(0.5 * LOG2E / syy) : 0.0;
+            const double uy = use ? -ux * sxy / syy : 0.0, dx = (double)mx - cx, dy = (double)my - cy;
+            em[EM_UX * KP + k] = (float)ux;
+            em[EM_UY * KP + k] = (float)uy;
+            em[EM_U0 * KP + k] = use ? (float)-(ux * dx + uy * dy) : 0.0f;
+            em[EM_WY * KP + k] = (float)wy;
+            em[EM_W0 * KP + k] = use ? (float)(-wy * dy) : 0.0f;
+        }
+    }
     // rows of P and pi: non-negative, finite, summing to 1 within 1e-5 (a warp
     // per row; row K is pi)
-    for (int i = threadIdx.x >> 5; i <= K; i += blockDim.x >> 5) {
+    for (int i = threadIdx.x >> 5; i <= K; i += PREP_THREADS / 32) {
         const float *row = i < K ? P + i * K : pi;
-        const int lane = threadIdx.x & 31;
         double s = 0.0;
         bool ok = true, tiny = false;
         for (int j = lane; j < K; j += 32) {
@@ -103,58 +144,11 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout l
             s += v;
         }
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (!ok || (lane == 0 && !(fabs(s - 1.0) <= 1e-5))) bad = 1;
-        if (i < K && tiny) small = 1;
-    }
-    // per-state emission constants (log2 domain), padded states emit nothing
-    const double LOG2E = 1.4426950408889634074;
-    const double LOG2_2PI = 2.6514961294723187980;
-    for (int k = threadIdx.x; k < KP; k += blockDim.x) {
-        float mx = 0.f, my = 0.f, qa = 0.f, qb = 0.f, qc = 0.f;
-        float ctr = -INFINITY, cno = -INFINITY;
-        double ux = 0.0, uy = 0.0, u0 = 0.0, wy = 0.0, w0 = 0.0;
-        if (k < K) {
-            double pk = p[k];
-            double sxx = cov[3 * k], sxy = cov[3 * k + 1], syy = cov[3 * k + 2];
-            double det = sxx * syy - sxy * sxy;
-            bool ok = isfinite(pk) && pk >= 0.0 && pk <= 1.0 && isfinite(sxx) && isfinite(sxy) &&
-                      isfinite(syy) && sxx > 0.0 && syy > 0.0 && det > 0.0 &&
-                      isfinite(mu[2 * k]) && isfinite(mu[2 * k + 1]);
-            if (!ok) {
-                bad = 1;
-            } else {
-                mx = mu[2 * k];
-                my = mu[2 * k + 1];
-                qa = (float)(-0.5 * LOG2E * syy / det);
-                qb = (float)(LOG2E * sxy / det);
-                qc = (float)(-0.5 * LOG2E * sxx / det);
-                ctr = (float)(log2(pk) - LOG2_2PI - 0.5 * log2(det));
-                cno = (float)log2(1.0 - pk);
-                // the quadratic form as two squares (Cholesky factor of the precision matrix)
-                ux = sqrt(0.5 * LOG2E * syy / det);
-                uy = -ux * sxy / syy;
-                wy = sqrt(0.5 * LOG2E / syy);
-                const double cx = (double)mx - centre[0], cy = (double)my - centre[1];
-                u0 = -(ux * cx + uy * cy);
-                w0 = -wy * cy;
-            }
-        }
-        float *em = cb + lay.off_emis;
-        em[EM_MUX * KP + k] = mx;
-        em[EM_MUY * KP + k] = my;
-        em[EM_QA * KP + k] = qa;
-        em[EM_QB * KP + k] = qb;
-        em[EM_QC * KP + k] = qc;
-        em[EM_CTR * KP + k] = ctr;
-        em[EM_CNO * KP + k] = cno;
-        em[EM_UX * KP + k] = (float)ux;
-        em[EM_UY * KP + k] = (float)uy;
-        em[EM_U0 * KP + k] = (float)u0;
-        em[EM_WY * KP + k] = (float)wy;
-        em[EM_W0 * KP + k] = (float)w0;
+        bad = bad || !ok || !(fabs(s - 1.0) <= 1e-5);
+        small = small || (i < K && tiny);
     }
     // P padded to KP x KP (FP32, row-major) and the tensor-core images
-    for (int idx = threadIdx.x; idx < KP * KP; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < KP * KP; idx += PREP_THREADS) {
         int i = idx / KP, j = idx % KP;
         float v = (i < K && j < K) ? P[i * K + j] : 0.0f;
         cb[lay.off_p32 + idx] = v;
@@ -172,26 +166,26 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout l
             img[KP * KP + kmajor_offset(j, i, KP, 8)] = lo;
         }
     }
-    __syncthreads();
+    bad = __syncthreads_or(bad);
+    small = __syncthreads_or(small);
     if (threadIdx.x < 32) {
         // EM_OFF: the emissions' largest constants, rounded up to whole numbers
-        float *em = cb + lay.off_emis;
         float mt = -INFINITY, mn = -INFINITY;
-        for (int k = threadIdx.x; k < K; k += 32) {
-            mt = fmaxf(mt, em[EM_CTR * KP + k]);
-            mn = fmaxf(mn, em[EM_CNO * KP + k]);
+        for (int k = lane; k < K; k += 32) {
+            mt = fmaxf(mt, s_ctr[k]);
+            mn = fmaxf(mn, s_cno[k]);
         }
         for (int o = 16; o > 0; o >>= 1) {
             mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
             mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
         }
-        if (threadIdx.x == 0) {
+        if (lane == 0) {
             mt = isfinite(mt) ? ceilf(mt) : 0.0f;
             mn = isfinite(mn) ? ceilf(mn) : 0.0f;
             em[EM_OFF * KP] = mt;
             em[EM_OFF * KP + 1] = mn;
-            em[EM_OFF * KP + 2] = centre[0];
-            em[EM_OFF * KP + 3] = centre[1];
+            em[EM_OFF * KP + 2] = s_centre[0];
+            em[EM_OFF * KP + 3] = s_centre[1];
             prop_bad[q] = bad;
             if (bad) atomicOr(status, ST_EINVAL);
             if (sp.route) {
@@ -208,24 +202,13 @@ __global__ void __launch_bounds__(PREP_THREADS) prep_kernel(int K, ConstLayout l
     }
 }
 
-cudaError_t launch_prep(int n_prop, int K, const ConstLayout &lay, int precision, int init_mode,
-                        const float *pi, const float *P, const float *p, const float *mu,
-                        const float *cov, float *cblock, int *prop_bad, unsigned *status,
-                        const StrandPtrs &sp, cudaStream_t st) {
-    (void)init_mode;
-    prep_kernel<<<n_prop, PREP_THREADS, 0, st>>>(K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad,
-                                        status, sp);
-    return cudaGetLastError();
-}
-
 // One thread per observation; the segment is found by binary search.
-__global__ void pack_kernel(int n_seg, const int64_t *__restrict__ offs,
-                            const int64_t *__restrict__ pbase, int64_t T_total,
-                            const float2 *__restrict__ xy, const uint8_t *__restrict__ tremor,
-                            float2 *__restrict__ packed, float2 *__restrict__ head,
-                            int *__restrict__ obs_bad, unsigned *__restrict__ status) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T_total;
-         t += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void pack_observations(int block, int blocks, int n_seg, const int64_t *__restrict__ offs,
+                                                  const int64_t *__restrict__ pbase, int64_t T_total,
+                                                  const float2 *__restrict__ xy, const uint8_t *__restrict__ tremor,
+                                                  float2 *__restrict__ packed, float2 *__restrict__ head,
+                                                  int *__restrict__ obs_bad, unsigned *__restrict__ status) {
+    for (int64_t t = block * (int64_t)PREP_THREADS + threadIdx.x; t < T_total; t += (int64_t)blocks * PREP_THREADS) {
         int lo = 0, hi = n_seg - 1;  // last s with offs[s] <= t
         while (lo < hi) {
             int mid = (lo + hi + 1) >> 1;
@@ -246,15 +229,33 @@ __global__ void pack_kernel(int n_seg, const int64_t *__restrict__ offs,
     }
 }
 
-cudaError_t launch_pack(int n_seg, const int64_t *d_offsets, const int64_t *d_pbase,
-                        int64_t T_total, const float *xy, const uint8_t *tremor, float2 *packed,
-                        float2 *head, int *obs_bad, unsigned *status, cudaStream_t st) {
-    if (T_total == 0) return cudaSuccess;
-    int64_t blocks = (T_total + 255) / 256;
+// Both in one launch: the first n_prop CTAs take a proposal each, the rest the
+// observations.
+__global__ void __launch_bounds__(PREP_THREADS)
+prep_pack_kernel(int n_prop, int K, ConstLayout lay, int precision, const float *__restrict__ pi,
+                 const float *__restrict__ P, const float *__restrict__ p, const float *__restrict__ mu,
+                 const float *__restrict__ cov, float *__restrict__ cblock, int *__restrict__ prop_bad,
+                 StrandPtrs sp, int n_seg, const int64_t *__restrict__ offs, const int64_t *__restrict__ pbase,
+                 int64_t T_total, const float2 *__restrict__ xy, const uint8_t *__restrict__ tremor,
+                 float2 *__restrict__ packed, float2 *__restrict__ head, int *__restrict__ obs_bad,
+                 unsigned *__restrict__ status) {
+    if ((int)blockIdx.x < n_prop)
+        prep_proposal(blockIdx.x, K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad, status, sp);
+    else
+        pack_observations(blockIdx.x - n_prop, gridDim.x - n_prop, n_seg, offs, pbase, T_total, xy, tremor, packed,
+                          head, obs_bad, status);
+}
+
+cudaError_t launch_prep_pack(int n_prop, int K, const ConstLayout &lay, int precision, const float *pi,
+                             const float *P, const float *p, const float *mu, const float *cov, float *cblock,
+                             int *prop_bad, const StrandPtrs &sp, int n_seg, const int64_t *d_offsets,
+                             const int64_t *d_pbase, int64_t T_total, const float *xy, const uint8_t *tremor,
+                             float2 *packed, float2 *head, int *obs_bad, unsigned *status, cudaStream_t st) {
+    int64_t blocks = (T_total + PREP_THREADS - 1) / PREP_THREADS;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    pack_kernel<<<(int)blocks, 256, 0, st>>>(n_seg, d_offsets, d_pbase, T_total,
-                                             reinterpret_cast<const float2 *>(xy), tremor, packed,
-                                             head, obs_bad, status);
+    prep_pack_kernel<<<(unsigned)(n_prop + blocks), PREP_THREADS, 0, st>>>(
+        n_prop, K, lay, precision, pi, P, p, mu, cov, cblock, prop_bad, sp, n_seg, d_offsets, d_pbase, T_total,
+        reinterpret_cast<const float2 *>(xy), tremor, packed, head, obs_bad, status);
     return cudaGetLastError();
 }
 

@@ -123,32 +123,49 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
         float keep[NS];
 #pragma unroll
         for (int u = 0; u < NS; ++u) keep[u] = v[u];
+        // two steps at a time: the recursion first, then both rows' sums, whose
+        // shuffles would otherwise stand between the steps
 #pragma unroll
-        for (int j = 3; j >= 0; --j) {
-            const int64_t i = 4 * w + j;
-            float f[NS], y[NS], al[NS], s = 0.0f;
+        for (int j2 = 2; j2 >= 0; j2 -= 2) {
+            float f[2][NS], y[2][NS], al[2][NS], s[2] = {0.0f, 0.0f};
 #pragma unroll
-            for (int u = 0; u < NS; ++u) al[u] = 0.0f;
-            if (own_steps && valid == 4) S.fetch(sm.alpha + i * KP, al);
+            for (int h = 1; h >= 0; --h) {
+                const int j = j2 + h;
 #pragma unroll
-            for (int u = 0; u < NS / 2; ++u) ec[u].eval(ox[j], oy[j], !isnan(ox[j]), f[2 * u], f[2 * u + 1]);
+                for (int u = 0; u < NS / 2; ++u) ec[u].eval(ox[j], oy[j], !isnan(ox[j]), f[h][2 * u], f[h][2 * u + 1]);
 #pragma unroll
-            for (int u = 0; u < NS; ++u) f[u] = ex2(f[u]) * v[u];
-            S.mul(f, y);
+                for (int u = 0; u < NS; ++u) f[h][u] = ex2(f[h][u]) * v[u];
+                S.mul(f[h], y[h]);
 #pragma unroll
-            for (int u = 0; u < NS; ++u) s = fmaf(al[u], y[u], s);
-            s = S.sum_all(s);
-            if (own_steps && valid == 4) {
-                const float r = rcp(s);
-                put_gamma(i, al, y, r);
-                if (sm.u) {
+                for (int u = 0; u < NS; ++u) v[u] = y[h][u];
+            }
+            if (!__any_sync(FULL, own_steps && valid == 4)) continue;  // all of the warp's strands are warming up
 #pragma unroll
-                    for (int u = 0; u < NS; ++u) f[u] *= r;
-                    S.store(sm.u + i * KP, f);
-                }
+            for (int h = 1; h >= 0; --h) {
+#pragma unroll
+                for (int u = 0; u < NS; ++u) al[h][u] = 0.0f;
+                if (own_steps && valid == 4) S.fetch(sm.alpha + (4 * w + j2 + h) * KP, al[h]);
+#pragma unroll
+                for (int u = 0; u < NS; ++u) s[h] = fmaf(al[h][u], y[h][u], s[h]);
             }
 #pragma unroll
-            for (int u = 0; u < NS; ++u) v[u] = y[u];
+            for (int o = 1; o < C::G; o <<= 1) {
+                s[0] += __shfl_xor_sync(FULL, s[0], o);
+                s[1] += __shfl_xor_sync(FULL, s[1], o);
+            }
+            if (own_steps && valid == 4) {
+#pragma unroll
+                for (int h = 1; h >= 0; --h) {
+                    const int64_t i = 4 * w + j2 + h;
+                    const float r = rcp(s[h]);
+                    put_gamma(i, al[h], y[h], r);
+                    if (sm.u) {
+#pragma unroll
+                        for (int u = 0; u < NS; ++u) f[h][u] *= r;
+                        S.store(sm.u + i * KP, f[h]);
+                    }
+                }
+            }
         }
         const float m = S.max_all(S.max_own(v));
         const bool fine = valid == 4 && m >= STRAND_SHRINK_KEEP && m <= STRAND_GROW;

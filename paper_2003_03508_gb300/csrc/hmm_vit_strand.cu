@@ -359,6 +359,8 @@ vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__res
 }
 
 // every piece's map: leaving state -> the state before its first step
+// (NC lanes' worth of states: a row is one byte a lane, or two)
+template <int NC>
 __global__ void __launch_bounds__(128)
 vit_map_kernel(int K, int KP, StrandPtrs sp, VitPtrs vp) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -369,14 +371,20 @@ vit_map_kernel(int K, int KP, StrandPtrs sp, VitPtrs vp) {
     int s0 = lane, s1 = lane + 32;
 #pragma unroll 8
     for (int t = d.len - 1; t >= 0; --t) {
-        const int r0 = lane < KP ? bp[(size_t)t * KP + lane] : 0, r1 = lane + 32 < KP ? bp[(size_t)t * KP + lane + 32] : 0;
-        const int a0 = __shfl_sync(FULL, r0, s0 & 31), a1 = __shfl_sync(FULL, r1, s0 & 31);
-        const int b0 = __shfl_sync(FULL, r0, s1 & 31), b1 = __shfl_sync(FULL, r1, s1 & 31);
-        s0 = s0 < 32 ? a0 : a1;
-        s1 = s1 < 32 ? b0 : b1;
+        const int r0 = lane < KP ? bp[(size_t)t * KP + lane] : 0;
+        const int a0 = __shfl_sync(FULL, r0, s0 & 31);
+        if (NC == 1) {
+            s0 = a0;
+        } else {
+            const int r1 = lane + 32 < KP ? bp[(size_t)t * KP + lane + 32] : 0;
+            const int a1 = __shfl_sync(FULL, r1, s0 & 31);
+            const int b0 = __shfl_sync(FULL, r0, s1 & 31), b1 = __shfl_sync(FULL, r1, s1 & 31);
+            s0 = s0 < 32 ? a0 : a1;
+            s1 = s1 < 32 ? b0 : b1;
+        }
     }
     if (lane < KP) vp.map[(size_t)c * KP + lane] = (uint8_t)s0;
-    if (lane + 32 < KP) vp.map[(size_t)c * KP + lane + 32] = (uint8_t)s1;
+    if (NC > 1 && lane + 32 < KP) vp.map[(size_t)c * KP + lane + 32] = (uint8_t)s1;
 }
 
 // One CTA: each warp composes the maps of a run of pieces, the runs are walked
@@ -425,6 +433,7 @@ vit_compose_kernel(int K, int KP, StrandPtrs sp, VitPtrs vp) {
 
 // A piece's states from its last one, and their part of the path's score: the
 // transitions into and the emissions of its observations (and of the first).
+template <int NC>
 __global__ void __launch_bounds__(128)
 vit_trace_kernel(int K, int KP, int init_mode, const float *__restrict__ pi, const float *__restrict__ P,
                  const float2 *__restrict__ head, const float2 *__restrict__ packed, StrandPtrs sp, VitPtrs vp,
@@ -448,9 +457,13 @@ vit_trace_kernel(int K, int KP, int init_mode, const float *__restrict__ pi, con
         int to = 0, from = 0;
 #pragma unroll 8
         for (int t = t1 - 1; t >= t0; --t) {
-            const int r0 = lane < KP ? bp[(size_t)t * KP + lane] : 0, r1 = lane + 32 < KP ? bp[(size_t)t * KP + lane + 32] : 0;
-            const int a0 = __shfl_sync(FULL, r0, s & 31), a1 = __shfl_sync(FULL, r1, s & 31);
-            const int before = s < 32 ? a0 : a1;
+            const int r0 = lane < KP ? bp[(size_t)t * KP + lane] : 0;
+            int before = __shfl_sync(FULL, r0, s & 31);
+            if (NC > 1) {
+                const int r1 = lane + 32 < KP ? bp[(size_t)t * KP + lane + 32] : 0;
+                const int a1 = __shfl_sync(FULL, r1, s & 31);
+                before = s < 32 ? before : a1;
+            }
             if (lane == t - t0) {
                 to = s;
                 from = before;
@@ -521,9 +534,11 @@ cudaError_t launch_vit_strands(int K, int KP, int init_mode, const ConstLayout &
     auto rejoin = KP <= 32 ? vit_rejoin_kernel<1> : vit_rejoin_kernel<2>;
     rejoin<<<ctas, 128, 0, st>>>(K, KP, false, lay, cb, packed, sp, vp);
     rejoin<<<ctas, 128, 0, st>>>(K, KP, true, lay, cb, packed, sp, vp);
-    vit_map_kernel<<<ctas, 128, 0, st>>>(K, KP, sp, vp);
+    if (KP <= 32) vit_map_kernel<1><<<ctas, 128, 0, st>>>(K, KP, sp, vp);
+    else vit_map_kernel<2><<<ctas, 128, 0, st>>>(K, KP, sp, vp);
     vit_compose_kernel<<<1, VC, 0, st>>>(K, KP, sp, vp);
-    vit_trace_kernel<<<ctas, 128, 0, st>>>(K, KP, init_mode, pi, P, head, packed, sp, vp, path);
+    auto trace = KP <= 32 ? vit_trace_kernel<1> : vit_trace_kernel<2>;
+    trace<<<ctas, 128, 0, st>>>(K, KP, init_mode, pi, P, head, packed, sp, vp, path);
     vit_score_kernel<<<1, 256, 0, st>>>(sp.n, vp, score);
     return cudaGetLastError();
 }
