@@ -4,28 +4,28 @@ Workload (one "step"): n_prop = 256 parameter proposals, each a random-walk
 perturbation of one generating parameter set, evaluated on one synthetic
 tremor-shaped sequence of T = 2^20 observations with K = 32 hidden states --
 one call of hmm_loglik_batched, i.e. every stage of the likelihood path
-(parameter constants, observation packing, chunk products, product tree,
-FP64 combine). Inputs are resident in HBM when the timed region starts; the
+(parameter constants and observation packing, strands and their join, chunk
+products and tree for what these leave, FP64 combine). Inputs are resident in HBM when the timed region starts; the
 L2 is flushed (a 256 MiB write) between timed steps, outside the events.
 Before the warm-up the chunk length is tuned for this shape by the library's
 autotuner (hmm_autotune_batched, untimed); the timed calls use the stored
 length (chunk_len = 0).
 
 Also reported on the same line:
-  plain_gpu     the same metric with the FP32-SIMT chunk products (same
-                workload, all proposals);
-  tf32_split    the same metric with TF32 chunk products whose P is carried
-                as hi + lo (two MMAs): FP32-like accuracy on the tensor cores;
+  plain_gpu     the same metric in FP32 on the CUDA cores (same workload, all
+                proposals);
+  tf32_split    the same metric with TF32 operands whose P is carried as hi +
+                lo (two MMAs): FP32-like accuracy on the tensor cores;
   e2e           the same metric through hmm_loglik_batched_host (pinned host
                 buffers, host->device inputs and device->host results inside
                 the timed region);
-  roofline      the chunk-product kernel against its peak;
+  roofline      the strands (2 K^2 flops a proposal and step; their join is in
+                the time) against the precision's peak;
   cpu_baseline  the FP64 CPU oracle on a bounded sample, on the host cores;
-  runlen        the run-length shortcut (FP32, not in the paper) on a
+  runlen        the run-length option (FP32, not in the paper) on a
                 sparse-tremor workload of the same size (tremor probabilities
                 0.002-0.05, long no-tremor runs) beside the tensor-core path on
-                the same data; its arithmetic depends on the data, so it is
-                reported apart from the roofline;
+                the same data;
   mcmc          effective samples per second of the log posterior and of
                 label-invariant summaries: the random-walk sampler, the learned
                 (MLP) proposal trained on the random walk's own history, and
@@ -355,7 +355,7 @@ def main():
     stream = torch.cuda.current_stream()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     steps_per_eval = int(offs[-1]) - (len(offs) - 1)
-    flops_per_eval = 2.0 * args.K ** 3 * steps_per_eval
+    flops_per_eval = 2.0 * args.K ** 2 * steps_per_eval  # one vector-matrix product a step
 
     def step():
         ctx.hmm_loglik_batched(*dev, offs, xy, fl, opts=opts, out=out)
@@ -402,22 +402,12 @@ def main():
     value = job_rate(args.n_prop * args.steps, world, total_ms)
     status = ctx.hmm_status()
 
-    # roofline of the chunk-product kernel (its phase is one launch per step)
+    # roofline of the strands (their phase also holds the join)
     chunk_ms = prof["chunk"] / max(1, ncalls)
     bound, peak, peak_src = roofline_peak(args.precision, peaks())
     achieved = flops_per_eval * args.n_prop / (chunk_ms / 1e3) / 1e12
-    traffic = None
-    tpath = os.path.join(ROOT, "profiles", "chunk_traffic.json")
-    if os.path.exists(tpath):
-        from paper_2003_03508_gb300 import build as _b
-        with open(tpath) as f:
-            tr = json.load(f)
-        key = f"{args.precision}:K{args.K}:T{args.T}:P{args.n_prop}:L{L}"
-        ent = tr.get(key)
-        if ent and ent.get("kernel_digest") == _b.kernel_digest("hmm_chunk_tc.cu", "hmm_chunk_simt.cu", "hmm_tc_common.cuh"):
-            traffic = ent["bytes_per_launch"]
     roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak, "traffic": traffic, "kernel": "hmm chunk products",
+            "frac": achieved / peak, "traffic": None, "kernel": "hmm strands",
             "peak_source": peak_src, "kernel_ms": chunk_ms,
             "phase_share": {k: v / max(1e-9, sum(prof.values())) for k, v in prof.items()}}
 
@@ -438,7 +428,7 @@ def main():
         result["autotune"] = tuned
 
     def timed_variant(precision, reps=2):
-        """The same workload and proposals with other chunk products (untimed
+        """The same workload and proposals in another precision (untimed
         warm-up call, then `reps` event-timed calls, L2 flushed before each)."""
         vo = api.make_opts(precision=precision)
         vout = torch.empty(args.n_prop, dtype=torch.float64, device="cuda")
@@ -458,7 +448,7 @@ def main():
         return {"value": job_rate(args.n_prop, world, ms), "unit": UNIT, "precision": precision,
                 "n_prop": args.n_prop, "ms_per_step": ms, "chunk_len": ctx.last_chunk_len}, vout
 
-    # plain GPU (FP32-SIMT chunk products) on the same workload and proposals
+    # plain GPU (FP32 on the CUDA cores) on the same workload and proposals
     variant_out = {}
     if not args.no_plain and args.precision != "fp32":
         result["plain_gpu"], pout = timed_variant("fp32")
@@ -470,7 +460,7 @@ def main():
         result["tf32_split"], sout = timed_variant("tf32_split")
         variant_out["tf32_split"] = sout.cpu().numpy()
 
-    # run-length shortcut on the sparse-tremor workload of the same size
+    # run-length option on the sparse-tremor workload of the same size
     if not args.no_runlen:
         result["runlen"] = runlen_leg(args, api, synth, ctx, stream, flush, world, rank)
 

@@ -19,6 +19,10 @@
  *   evaluated in parallel, the matrices M_t = P D_t are multiplied as a chain
  *   split into chunks, the chunk products are combined, and log L (not L) is
  *   returned, with scale coefficients keeping every partial product in range.
+ *   Where the chain forgets its start (the vectors that neighbouring pieces
+ *   reach are checked to be proportional, entry by entry) each piece carries one
+ *   forward vector in place of a K x K product; other proposals take the chunk
+ *   products. Both give log L to the stated precision.
  *
  * Conventions for every entry point:
  *   - Every function returns an int status: HMM_OK (0) or one of HMM_E*.
@@ -57,11 +61,11 @@ extern "C" {
 #define HMM_ETIMEOUT 5     /* a bounded device wait expired (kernel returned early) */
 #define HMM_EUNSUPPORTED 6 /* option not available for this K / device */
 
-/* ---- arithmetic of the chunk products (Step 3) ---- */
+/* ---- arithmetic of the vector and chunk products (Step 3) ---- */
 #define HMM_PREC_FP32_SIMT 0  /* FP32 FFMA on the CUDA cores ("plain GPU") */
-#define HMM_PREC_TF32 1       /* tcgen05 tensor cores, TF32 operands, FP32 accumulation */
-#define HMM_PREC_BF16 2       /* tcgen05 tensor cores, BF16 running product, P as BF16 hi+lo */
-#define HMM_PREC_TF32_SPLIT 3 /* tcgen05 TF32 with P as TF32 hi+lo (two MMAs) */
+#define HMM_PREC_TF32 1       /* tensor cores, TF32 operands, FP32 accumulation */
+#define HMM_PREC_BF16 2       /* tensor cores, P as BF16 hi+lo; vectors as BF16 hi+lo, chunk products BF16 */
+#define HMM_PREC_TF32_SPLIT 3 /* TF32 with P as TF32 hi+lo (two MMAs) */
 
 /* ---- where pi enters ---- */
 #define HMM_INIT_EMIT_FIRST 0       /* L = pi^T D_1 P D_2 ... (pi = law of the first state) */
@@ -90,17 +94,19 @@ typedef struct {
     int32_t precision;    /* HMM_PREC_*                                           */
     int32_t init_mode;    /* HMM_INIT_*                                           */
     int32_t chunk_len;    /* steps per chunk product (multiple of 64); 0 = tuned or cost model (below) */
-    int32_t renorm_every; /* per-row power-of-two renormalisation interval; 0 = 4 */
+    int32_t renorm_every; /* chunk products: per-row power-of-two renormalisation interval; 0 = 4 */
     int32_t recheck_fp32; /* samplers only (see hmm_sampler_create); ignored here  */
     int32_t runlen_min;   /* run-length shortcut, FP32-SIMT only; 0 = off (below)  */
     int32_t reserved[2];  /* must be 0                                             */
 } hmm_opts;
 
 /*
- * Run-length shortcut (opts->runlen_min = n_min >= 1). Every step without a
+ * Run-length shortcut (opts->runlen_min = n_min >= 1), for data in which
+ * tremors are rare. The forward vectors then start further before their pieces;
+ * the chunk products of what these leave use that every step without a
  * tremor has the same matrix M_0 = P diag(1 - p_k) (Eq. "emission-matrix"),
- * so a run of n of them inside a chunk contributes M_0^n. With the shortcut
- * on, the library first builds, per proposal, M_0^(2^b) for b = 0 ..
+ * so a run of n of them inside a chunk contributes M_0^n: the
+ * library builds, per proposal, M_0^(2^b) for b = 0 ..
  * floor(log2(chunk length)) by repeated squaring (each row a float row plus
  * its own power-of-two exponent), and every run of at least n_min
  * no-tremor steps is applied as the product of the powers of its length's
@@ -136,11 +142,11 @@ int hmm_status(hmm_ctx *ctx, void *stream);
  * (the forward-backward algorithm; Rabiner, Proc. IEEE 1989, Section III-A).
  * gamma (device, T x K floats, row-major) receives
  * gamma[t][k] = P(s_t = k | o_0 .. o_{T-1}); *loglik (device double)
- * receives log L. Computed on the chunk structure of hmm_loglik, with the
- * same options (opts->precision chooses the chunk products): two scans over
- * the chunk products give the forward vector entering and the backward
- * vector leaving every chunk, then every chunk recomputes its steps in FP32
- * from both, normalising each vector every step. T >= 1. A zero likelihood
+ * receives log L. Forward and backward vectors are carried
+ * over pieces of the sequence in FP32, as in hmm_loglik; where they do not
+ * apply, two scans over the chunk products (of opts->precision) give the
+ * forward vector entering and the backward vector leaving every chunk, and
+ * every chunk recomputes its steps in FP32 from both. T >= 1. A zero likelihood
  * gives NaN rows.
  */
 int hmm_posterior(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *obs, const hmm_opts *opts,
@@ -148,11 +154,12 @@ int hmm_posterior(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *obs, co
 
 /*
  * The most probable hidden path of one sequence (Viterbi; Rabiner 1989,
- * Section III-B) on the chunk structure: every chunk's max-plus product
- * (best log2 score from each entering to each leaving state, CUDA cores),
- * a scan over chunk boundaries in FP64 with back-pointers, then every chunk
- * re-runs its recursion from its entering state and traces the path back
- * from its leaving state. path (device, T int32) receives the states;
+ * Section III-B). Every piece of the sequence carries one max-plus vector (best
+ * log2 score of each state, CUDA cores) with back-pointers, checked against its
+ * neighbour's as in hmm_loglik, and the pieces are traced back by their composed
+ * maps; sequences whose paths do not coalesce take every chunk's max-plus
+ * product, a scan over chunk boundaries in FP64 with back-pointers, and a re-run
+ * of every chunk between its states. path (device, T int32) receives the states;
  * *score (device double) log p(path, o) (natural log, -inf if every path has
  * probability zero); *loglik (device double) log L. Ties go to the smallest
  * state; paths whose scores differ only by FP32 rounding may differ from an
@@ -163,7 +170,7 @@ int hmm_viterbi(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *obs, cons
 
 /*
  * Expected sufficient statistics of the hidden chain (the E-step of EM,
- * Baum-Welch; Rabiner 1989, Section III-C), from the same chunked forward-
+ * Baum-Welch; Rabiner 1989, Section III-C), from the same forward-
  * backward pass as hmm_posterior, into `stats` (device, K*K + 8*K doubles):
  *   N[i][j] = sum_{t>=1} P(s_{t-1}=i, s_t=j | o)  (K*K, row-major)
  *   G0[k] = P(s_0 = k | o); Gs[k] = sum_t gamma_t(k);
@@ -171,8 +178,8 @@ int hmm_viterbi(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *obs, cons
  *   Sx, Sy, Sxx, Sxy, Syy [k] = the same sums weighted by x, y, x^2, xy, y^2
  * (K each, in this order after N). With the Fisher identity they give the
  * gradient of log L with respect to every parameter (for gradient-based
- * samplers), and an EM update. Chunk partial sums are added in chunk order
- * in FP64 (deterministic). *loglik (device) receives log L. T >= 2.
+ * samplers), and an EM update. Partial sums over blocks of steps are added
+ * in a fixed order in FP64 (deterministic). *loglik (device) receives log L. T >= 2.
  */
 int hmm_expected_stats(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *obs, const hmm_opts *opts,
                        double *stats, double *loglik, void *stream);
@@ -183,7 +190,7 @@ int hmm_expected_stats(hmm_ctx *ctx, const hmm_params *params, const hmm_obs *ob
  * posterior expectation of the gradient of the complete-data log likelihood
  * of Section 2 (hidden path, transitions P, emissions of Eq.
  * "emission-matrix"), formed in FP64 on the device from the statistics of
- * hmm_expected_stats (same options, same chunked forward-backward pass).
+ * hmm_expected_stats (same options, same forward-backward pass).
  * grad (device, K*K + 7*K doubles) receives, in the order of hmm_params,
  *   d/dpi [K], d/dP [K*K] (row-major), d/dp_tremor [K], d/dmu [K*2],
  *   d/dcov [K*3] (sxx, sxy, syy; sxy enters both off-diagonal entries),
@@ -284,8 +291,9 @@ int hmm_last_call_graph(const hmm_ctx *ctx);
 /* ---- chunk-length tuning of the batched schedule ----
  *
  * Section "The likelihood algorithm" splits the matrix chain into chunks
- * without fixing their length. The chunk length L sets the schedule of
- * hmm_loglik_batched: how many chunk products (work items of the persistent
+ * without fixing their length. The chunk length L sets the schedule of the
+ * chunk products of hmm_loglik_batched (the pieces of the forward vectors have
+ * a rule of their own): how many chunk products (work items of the persistent
  * chunk kernels) there are, how many waves of them the GPU runs, and the size
  * of the product tree. The tile shapes are fixed by the hardware mapping
  * (M = 128 rows of tensor memory, N = the padded state count), so L is the
@@ -368,9 +376,9 @@ int hmm_tune_save(const char *path);
 int hmm_tune_load(const char *path);
 
 /* ---- per-phase device timing (benchmarks) ---- */
-#define HMM_PHASE_PREP 0   /* parameter checks and constants          */
-#define HMM_PHASE_PACK 1   /* observation packing                      */
-#define HMM_PHASE_CHUNK 2  /* chunk products (Section "Step 3")        */
+#define HMM_PHASE_PREP 0   /* parameter checks and constants, observation packing */
+#define HMM_PHASE_PACK 1   /* (packing runs in the launch before: about 0) */
+#define HMM_PHASE_CHUNK 2  /* vectors and their join, chunk products (Section "Step 3") */
 #define HMM_PHASE_TREE 3   /* combining the chunk products             */
 #define HMM_PHASE_FINAL 4  /* head vector, FP64 log L, segment sum     */
 #define HMM_PHASE_COUNT 5
