@@ -238,7 +238,7 @@ template <int NC, bool BACK>
 __global__ void __launch_bounds__(128)
 rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__restrict__ cb,
                  const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm) {
-    __shared__ float2 sag[4][32 * NC];
+    __shared__ __align__(16) float2 sag[4][32 * NC];
     constexpr float tol = 3.0517578125e-5f;  // 2^-15, as in the likelihood's join
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
@@ -283,66 +283,103 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
 #pragma unroll
             for (int j = 0; j < 32; ++j) pc[NC == 1 ? j : 0] = j < K && lane < K ? (BACK ? P[lane * KPl + j] : P[j * KPl + lane]) : 0.0f;
         }
+        // emissions relative to the whole offsets, as the strands have them; a
+        // step that shrinks too far is made again with exact scaling
+        const float offt = em[EM_OFF * KPl], offn = em[EM_OFF * KPl + 1];
+        float ec[NC][7];  // in registers: the rows written below could alias them
+#pragma unroll
+        for (int n = 0; n < NC; ++n) {
+            const int k = lane + 32 * n;
+#pragma unroll
+            for (int r = 0; r < 7; ++r) ec[n][r] = k < K ? em[r * KPl + k] : r >= EM_CTR ? -INFINITY : 0.0f;
+            ec[n][EM_CTR] -= offt;
+            ec[n][EM_CNO] -= offn;
+        }
+        float2 ob = make_float2(0.0f, 0.0f);  // 32 steps' observations, one a lane
         for (int &s = rows; s < least || (s & 3) || !met(); ++s) {
             if (s >= d.len) return 0;
             const int64_t i = BACK ? d.pstart + d.len - 1 - s : d.pstart + s;
-            const float2 o = packed[i];
-            const bool tr = !isnan(o.x);
-            float f[NC], wa[NC], mx = -INFINITY;
+            if ((s & 31) == 0) {
+                const int64_t x = BACK ? i - lane : i + lane;
+                if (BACK ? x >= d.pstart : x < d.pstart + d.len) ob = packed[x];
+                if (BACK && x >= d.pstart) {
+                    // alpha's rows of these steps, ahead of their turn
+                    for (int k = 0; k < KP; k += 32) asm volatile("prefetch.global.L1 [%0];" ::"l"(sm.alpha + x * KP + k));
+                }
+            }
+            const float ox = __shfl_sync(FULL, ob.x, s & 31), oy = __shfl_sync(FULL, ob.y, s & 31);
+            const bool tr = !isnan(ox);
+            float l[NC], f[NC], wa[NC], ka[NC], kg[NC], al[NC], ma, mg;
 #pragma unroll
             for (int n = 0; n < NC; ++n) {
                 const int k = lane + 32 * n;
-                f[n] = k < K ? log2_emission(em, KPl, k, o.x, o.y, tr) : -INFINITY;
-                mx = fmaxf(mx, f[n]);
+                al[n] = BACK && k < K ? sm.alpha[i * KP + k] : 0.0f;  // early: used after the step
+                const float dx = ox - ec[n][EM_MUX], dy = oy - ec[n][EM_MUY];
+                l[n] = fmaf(fmaf(ec[n][EM_QA], dx, ec[n][EM_QB] * dy), dx, fmaf(ec[n][EM_QC] * dy, dy, ec[n][EM_CTR]));
+                l[n] = tr ? l[n] : ec[n][EM_CNO];
+                f[n] = ex2(l[n]);
+                ka[n] = a[n];
+                kg[n] = g[n];
             }
-            mx = all_max(mx);
-            if (!(mx >= -(float)EXP_LIMIT)) return -1;
-            const float fm = floorf(mx);
+            for (int attempt = 0;; ++attempt) {
 #pragma unroll
-            for (int n = 0; n < NC; ++n) {
-                f[n] = ex2(f[n] - fm);
-                wa[n] = BACK ? a[n] * f[n] : a[n];
-                sag[warp][lane + 32 * n] = make_float2(wa[n], BACK ? g[n] * f[n] : g[n]);
-                a[n] = g[n] = 0.0f;
-            }
-            __syncwarp();
-            if (NC == 1) {
-                f32x2 t[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float p = pc[NC == 1 ? j : 0];
-                    t[j & 3] = fma2(*reinterpret_cast<const f32x2 *>(&sag[warp][j]), pack2(p, p), t[j & 3]);
+                for (int n = 0; n < NC; ++n) {
+                    wa[n] = BACK ? ka[n] * f[n] : ka[n];
+                    sag[warp][lane + 32 * n] = make_float2(wa[n], BACK ? kg[n] * f[n] : kg[n]);
+                    a[n] = g[n] = 0.0f;
                 }
-                unpack2(add2(add2(t[0], t[1]), add2(t[2], t[3])), a[0], g[0]);
-            } else {
-#pragma unroll 8
-                for (int j = 0; j < 32 * NC; ++j) {
-                    const float2 x = sag[warp][j];
+                __syncwarp();
+                if (NC == 1) {
+                    f32x2 t[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-                    for (int n = 0; n < NC; ++n) {
-                        const int k = lane + 32 * n;
-                        const float p = k < K && j < K ? (BACK ? P[k * KPl + j] : P[j * KPl + k]) : 0.0f;
-                        a[n] = fmaf(x.x, p, a[n]);
-                        g[n] = fmaf(x.y, p, g[n]);
+                    for (int j = 0; j < 32; j += 2) {
+                        const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sag[warp][j]);
+                        const float p0 = pc[NC == 1 ? j : 0], p1 = pc[NC == 1 ? j + 1 : 0];
+                        t[j & 2] = fma2(x.x, pack2(p0, p0), t[j & 2]);
+                        t[(j & 2) + 1] = fma2(x.y, pack2(p1, p1), t[(j & 2) + 1]);
+                    }
+                    unpack2(add2(add2(t[0], t[1]), add2(t[2], t[3])), a[0], g[0]);
+                } else {
+#pragma unroll 8
+                    for (int j = 0; j < 32 * NC; ++j) {
+                        const float2 x = sag[warp][j];
+#pragma unroll
+                        for (int n = 0; n < NC; ++n) {
+                            const int k = lane + 32 * n;
+                            const float p = k < K && j < K ? (BACK ? P[k * KPl + j] : P[j * KPl + k]) : 0.0f;
+                            a[n] = fmaf(x.x, p, a[n]);
+                            g[n] = fmaf(x.y, p, g[n]);
+                        }
                     }
                 }
-            }
-            __syncwarp();
-            float ma = 0.0f, mg = 0.0f;
+                __syncwarp();
+                ma = mg = 0.0f;
 #pragma unroll
-            for (int n = 0; n < NC; ++n) {
-                if (!BACK) {
-                    a[n] *= f[n];
-                    g[n] *= f[n];
+                for (int n = 0; n < NC; ++n) {
+                    if (!BACK) {
+                        a[n] *= f[n];
+                        g[n] *= f[n];
+                    }
+                    ma = fmaxf(ma, a[n]);
+                    mg = fmaxf(mg, g[n]);
                 }
-                ma = fmaxf(ma, a[n]);
-                mg = fmaxf(mg, g[n]);
+                ma = all_max(ma);
+                mg = all_max(mg);
+                if (ma >= STRAND_SHRINK_KEEP && mg >= STRAND_SHRINK_KEEP && ma <= STRAND_GROW && mg <= STRAND_GROW) break;
+                if (attempt) {
+                    if (ma >= STRAND_SHRINK && mg >= STRAND_SHRINK && ma <= STRAND_GROW && mg <= STRAND_GROW) break;
+                    return -1;
+                }
+                float mx = l[0];
+#pragma unroll
+                for (int n = 1; n < NC; ++n) mx = fmaxf(mx, l[n]);
+                mx = all_max(mx);
+                if (!(mx + (tr ? offt : offn) >= -(float)EXP_LIMIT)) return -1;
+#pragma unroll
+                for (int n = 0; n < NC; ++n) f[n] = ex2(l[n] - floorf(mx));
             }
-            ma = all_max(ma);
-            mg = all_max(mg);
-            if (!(ma >= STRAND_SHRINK && mg >= STRAND_SHRINK && ma <= STRAND_GROW && mg <= STRAND_GROW)) return -1;
             const float fa = pow2f(-float_exponent(ma)), fg = pow2f(-float_exponent(mg));
-            float z = 0.0f, al[NC];
+            float z = 0.0f;
 #pragma unroll
             for (int n = 0; n < NC; ++n) {
                 const int k = lane + 32 * n;
@@ -350,14 +387,13 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
                 g[n] *= fg;
                 wa[n] *= fa;
                 if (BACK) {
-                    al[n] = k < K ? sm.alpha[i * KP + k] : 0.0f;
                     z = fmaf(al[n], a[n], z);
                 } else if (k < KP) {
                     sm.alpha[(i + 1) * KP + k] = a[n];
                 }
             }
             if (BACK) {
-                const float r = 1.0f / all_sum(z);
+                const float r = rcp(all_sum(z));
 #pragma unroll
                 for (int n = 0; n < NC; ++n) {
                     const int k = lane + 32 * n;
@@ -545,10 +581,10 @@ __global__ void stats_sum_kernel(int K, int n_parts, const double *__restrict__ 
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) stats[K * K + k] = g0[k];
 }
 
-template <int KP>
+template <int KP, int H>
 cudaError_t back_t(int K, int64_t steps, const ConstLayout &lay, const float *cb, const float2 *packed,
                    const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st) {
-    using C = SimtTile<KP>;
+    using C = SimtTile<KP, H>;
     const int warps = (sp.n + C::PER_WARP - 1) / C::PER_WARP;
     strand_back_kernel<C><<<(warps + STRAND_WPC - 1) / STRAND_WPC, 32 * STRAND_WPC, 0, st>>>(K, steps, sm.warm, lay, cb,
                                                                                            packed, sp, sm);
@@ -581,18 +617,19 @@ cudaError_t launch_smooth(int K, int KP, int64_t steps, const ConstLayout &lay, 
                           const float2 *packed, const StrandPtrs &sp, const SmoothPtrs &sm, cudaStream_t st) {
     cudaError_t e = join_t<false>(K, KP, lay, cblock, packed, sp, sm, st);
     if (e != cudaSuccess) return e;
-#define HMM_SMOOTH_CASE(KPV)                                                       \
+#define HMM_SMOOTH_CASE(KPV, HV)                                                   \
     case KPV:                                                                      \
-        e = back_t<KPV>(K, steps, lay, cblock, packed, sp, sm, st);                \
+        e = strand_rows(KPV, sp.n) == 2 ? back_t<KPV, HV>(K, steps, lay, cblock, packed, sp, sm, st) \
+                                        : back_t<KPV, HV == 2 && KPV < 64 ? 1 : HV>(K, steps, lay, cblock, packed, sp, sm, st); \
         if (e == cudaSuccess) e = join_t<true>(K, KP, lay, cblock, packed, sp, sm, st); \
         if (e == cudaSuccess && sm.stats) e = stats_t<KPV>(K, steps, lay, cblock, head, packed, sp, sm, st); \
         return e;
     switch (KP) {
-        HMM_SMOOTH_CASE(4)
-        HMM_SMOOTH_CASE(8)
-        HMM_SMOOTH_CASE(16)
-        HMM_SMOOTH_CASE(32)
-        HMM_SMOOTH_CASE(64)
+        HMM_SMOOTH_CASE(4, 1)
+        HMM_SMOOTH_CASE(8, 1)
+        HMM_SMOOTH_CASE(16, 2)
+        HMM_SMOOTH_CASE(32, 2)
+        HMM_SMOOTH_CASE(64, 2)
         default: return cudaErrorInvalidValue;
     }
 #undef HMM_SMOOTH_CASE

@@ -200,12 +200,18 @@ template <int KP>
 cudaError_t launch_t(int n_prop, int K, int init_mode, const ConstLayout &lay, bool round_tf32, const float *cblock,
                      const float *pi, const float2 *head, const float2 *packed, const StrandPtrs &sp, float *alpha,
                      cudaStream_t st) {
+    auto go = [&](auto kern, int per_warp) {
+        const long long warps = (long long)n_prop * ((sp.n + per_warp - 1) / per_warp);
+        kern<<<(unsigned)((warps + STRAND_WPC - 1) / STRAND_WPC), 32 * STRAND_WPC, 0, st>>>(
+            n_prop, K, init_mode, lay, round_tf32, cblock, pi, head, packed, sp, alpha);
+        return cudaGetLastError();
+    };
     using C = SimtTile<KP>;
-    const long long warps = (long long)n_prop * ((sp.n + C::PER_WARP - 1) / C::PER_WARP);
-    auto kern = alpha ? strand_simt_kernel<C, true> : strand_simt_kernel<C, false>;
-    kern<<<(unsigned)((warps + STRAND_WPC - 1) / STRAND_WPC), 32 * STRAND_WPC, 0, st>>>(
-        n_prop, K, init_mode, lay, round_tf32, cblock, pi, head, packed, sp, alpha);
-    return cudaGetLastError();
+    constexpr bool two = KP == 16 || KP == 32;
+    using C2 = SimtTile<KP, two ? 2 : C::H>;
+    if (two && (long long)n_prop * sp.n < (1 << 20) && strand_rows(KP, n_prop * sp.n) == 2)
+        return alpha ? go(strand_simt_kernel<C2, true>, C2::PER_WARP) : go(strand_simt_kernel<C2, false>, C2::PER_WARP);
+    return alpha ? go(strand_simt_kernel<C, true>, C::PER_WARP) : go(strand_simt_kernel<C, false>, C::PER_WARP);
 }
 
 }  // namespace

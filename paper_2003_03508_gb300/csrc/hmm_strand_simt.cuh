@@ -13,12 +13,15 @@ constexpr int STRAND_WPC = 4;  // warps per CTA
 // it is responsible for (KP / H of their rows) in registers, as pairs over the
 // row index, so a step reads the vector from shared memory as 16-byte
 // broadcasts (one load feeds 16 FMAs) and nothing else: one step of KP = 32 is
-// 64 packed FMAs and 8 loads per thread, and a warp carries four strands. For
-// KP = 64 two half-warps take half of the rows each and swap two partial sums.
-template <int KP_>
+// 64 packed FMAs and 8 loads per thread, and a warp carries four strands. With
+// H = 2 twice the threads take half of the rows each and swap two partial sums:
+// for KP = 64, whose columns do not fit one thread otherwise, and for sequences
+// with too few strands to give every scheduler a warp, where a step's latency is
+// what counts (strand_rows).
+template <int KP_, int H_ = (KP_ > 32 ? 2 : 1)>
 struct SimtTile {
     static constexpr int KP = KP_;
-    static constexpr int H = KP > 32 ? 2 : 1;    // row split
+    static constexpr int H = H_;                 // row split
     static constexpr int CG = KP / 4;            // column groups
     static constexpr int G = CG * H;             // threads per strand
     static constexpr int NI = KP / H;            // rows per thread
@@ -28,8 +31,15 @@ struct SimtTile {
     // one strand's vector in shared memory, padded so that the broadcasts of
     // different strands (and of the two row halves) fall on different banks
     static constexpr int STRIDE = KP + 4 * H;
-    static __device__ __forceinline__ int at(int i) { return H == 1 ? i : i + 4 * (i / 32); }
+    static __device__ __forceinline__ int at(int i) { return H == 1 ? i : i + 4 * (i / NI); }
 };
+
+// Row split for n strands in all: two while one row block would leave schedulers
+// without a warp (4 on each of 152 SMs). Posterior K=25, T=105,000: forward 53 ->
+// 43 us, backward 98 -> 81; Viterbi's strands 148 -> 98.
+inline int strand_rows(int KP, int n) {
+    return KP == 64 ? 2 : (KP == 32 && n <= 4 * 608) || (KP == 16 && n <= 8 * 608) ? 2 : 1;
+}
 
 template <class C>
 struct SimtStrand {
@@ -106,8 +116,8 @@ struct SimtStrand {
             for (int u = 0; u < NS; ++u) y[u] = s[u];
         } else {
             // the other half's rows: swap the two sums each half does not own
-            const float t0 = __shfl_xor_sync(0xffffffffu, h ? s[0] : s[2], 16);
-            const float t1 = __shfl_xor_sync(0xffffffffu, h ? s[1] : s[3], 16);
+            const float t0 = __shfl_xor_sync(0xffffffffu, h ? s[0] : s[2], C::CG);
+            const float t1 = __shfl_xor_sync(0xffffffffu, h ? s[1] : s[3], C::CG);
             y[0] = (h ? s[2] : s[0]) + t0;
             y[1] = (h ? s[3] : s[1]) + t1;
         }

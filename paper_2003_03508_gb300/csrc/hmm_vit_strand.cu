@@ -195,8 +195,8 @@ vit_strand_kernel(int K, int init_mode, ConstLayout lay, const float *__restrict
             // the other half's rows: the first half wins ties (smaller indices)
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const float ob = __shfl_xor_sync(FULL, h ? best[u] : best[2 + u], 16);
-                const int oa = __shfl_xor_sync(FULL, h ? arg[u] : arg[2 + u], 16);
+                const float ob = __shfl_xor_sync(FULL, h ? best[u] : best[2 + u], C::CG);
+                const int oa = __shfl_xor_sync(FULL, h ? arg[u] : arg[2 + u], C::CG);
                 const float mb = h ? best[2 + u] : best[u];
                 const int ma = h ? arg[2 + u] : arg[u];
                 const bool take = h ? ob >= mb : ob > mb;
@@ -503,10 +503,10 @@ __global__ void __launch_bounds__(256) vit_score_kernel(int n, VitPtrs vp, doubl
     if (threadIdx.x == 0) *score = red[0];
 }
 
-template <int KP>
+template <int KP, int H>
 cudaError_t vit_t(int K, int init_mode, const ConstLayout &lay, const float *cb, const float *pi, const float2 *head,
                   const float2 *packed, const StrandPtrs &sp, const VitPtrs &vp, cudaStream_t st) {
-    using C = SimtTile<KP>;
+    using C = SimtTile<KP, H>;
     const int warps = (sp.n + C::PER_WARP - 1) / C::PER_WARP;
     vit_strand_kernel<C><<<(warps + STRAND_WPC - 1) / STRAND_WPC, 32 * STRAND_WPC, 0, st>>>(K, init_mode, lay, cb, pi,
                                                                                           head, packed, sp, vp);
@@ -522,11 +522,17 @@ cudaError_t launch_vit_strands(int K, int KP, int init_mode, const ConstLayout &
     vit_table_kernel<<<(KP * KP + 127) / 128, 128, 0, st>>>(K, KP, P, p, mu, cov, vp);
     cudaError_t e = cudaSuccess;
     switch (KP) {
-        case 4: e = vit_t<4>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
-        case 8: e = vit_t<8>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
-        case 16: e = vit_t<16>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
-        case 32: e = vit_t<32>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
-        case 64: e = vit_t<64>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
+        case 4: e = vit_t<4, 1>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
+        case 8: e = vit_t<8, 1>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
+        case 16:
+            e = strand_rows(KP, sp.n) == 2 ? vit_t<16, 2>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st)
+                                           : vit_t<16, 1>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st);
+            break;
+        case 32:
+            e = strand_rows(KP, sp.n) == 2 ? vit_t<32, 2>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st)
+                                           : vit_t<32, 1>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st);
+            break;
+        case 64: e = vit_t<64, 2>(K, init_mode, lay, cb, pi, head, packed, sp, vp, st); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
