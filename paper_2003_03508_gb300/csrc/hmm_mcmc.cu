@@ -126,28 +126,44 @@ __device__ double block_sum(double v, double *red) {
 __device__ double transform(int K, const double *th, const Prior &pr, float *pi, float *P, float *p, float *mu,
                             float *cov, double *red) {
     double part = 0.0;
-    // rows of P, and pi as row K (state 0 its reference): a warp per row, one
-    // exponential an entry and lane (a thread per row took K of them in turn:
-    // 61 us for 512 chains of K = 16)
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i <= K; i += TPB / 32) {
+    // Rows of P, and pi as row K (state 0 its reference): a group of lanes per
+    // row, two or four rows a warp where they fit, and one exponential an entry.
+    // FP64 runs at two lanes per cycle and SM here, so its instructions are what
+    // this costs: 512 chains of K = 16 took 61 us with two exponentials an entry,
+    // a thread or a warp per row alike.
+    const int width = K <= 8 ? 8 : K <= 16 ? 16 : 32;
+    const int lane = threadIdx.x % width;
+    const unsigned lanes = (width == 32 ? 0xffffffffu : (1u << width) - 1u) << ((threadIdx.x & 31) / width * width);
+    for (int i = threadIdx.x / width; i <= K; i += TPB / width) {
         const double *z = th + (size_t)i * (K - 1);
         const int ref = i < K ? i : 0;
         const double alpha = i < K ? pr.alpha_P : pr.alpha_pi;
-        auto logit = [&](int j) { return j == ref ? 0.0 : z[j < ref ? j : j - 1]; };
-        double mx = 0.0;
-        for (int j = lane; j < K; j += 32) mx = fmax(mx, logit(j));
-        for (int s = 16; s > 0; s >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-        double s = 0.0;
-        for (int j = lane; j < K; j += 32) s += exp(logit(j) - mx);
-        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        const double lse = mx + log(s);
-        float *out = i < K ? P + (size_t)i * K : pi;
-        for (int j = lane; j < K; j += 32) {
-            const double zz = logit(j);
-            out[j] = (float)exp(zz - lse);
-            part += alpha * (zz - lse);
+        double zz[3], e[3], mx = 0.0, s = 0.0, zs = 0.0;  // this lane's entries (K <= 80)
+        int n = 0;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int j = lane + u * width;
+            if (j < K) {
+                zz[u] = j == ref ? 0.0 : z[j < ref ? j : j - 1];
+                mx = fmax(mx, zz[u]);
+                zs += zz[u];
+                ++n;
+            }
         }
+        for (int d = width / 2; d > 0; d >>= 1) mx = fmax(mx, __shfl_xor_sync(lanes, mx, d));
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (lane + u * width < K) {
+                e[u] = exp(zz[u] - mx);
+                s += e[u];
+            }
+        for (int d = width / 2; d > 0; d >>= 1) s += __shfl_xor_sync(lanes, s, d);
+        const double inv = 1.0 / s, lse = mx + log(s);
+        float *out = i < K ? P + (size_t)i * K : pi;
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (lane + u * width < K) out[lane + u * width] = (float)(e[u] * inv);
+        part += alpha * (zs - n * lse);
     }
     int o = K * (K - 1);
     o += K - 1;
@@ -156,9 +172,9 @@ __device__ double transform(int K, const double *th, const Prior &pr, float *pi,
         const double w = th[o + k];
         const double m = (k < K / 2) ? pr.p_mean_lo : pr.p_mean_hi;
         const double a = m * m / pr.p_var, b = m / pr.p_var;
-        const double pk = 1.0 / (1.0 + exp(-w));
+        const double t = exp(-w), pk = 1.0 / (1.0 + t), lt = log1p(t);
         p[k] = (float)pk;
-        part += a * (-log1p(exp(-w))) - b * pk + (-log1p(exp(w)));
+        part += -a * lt - b * pk - (w + lt);  // log1p(e^w) = w + log1p(e^-w)
         // mean: uniform on the box
         const double x = th[o + K + 2 * k], y = th[o + K + 2 * k + 1];
         mu[2 * k] = (float)x;
@@ -172,9 +188,9 @@ __device__ double transform(int K, const double *th, const Prior &pr, float *pi,
         cov[3 * k] = (float)sxx;
         cov[3 * k + 1] = (float)sxy;
         cov[3 * k + 2] = (float)syy;
-        const double det = sxx * syy - sxy * sxy;
-        part += -0.5 * (pr.iw_df + 3.0) * log(det) - 0.5 * (sxx + syy) / det;
-        part += log(4.0) + log1p(-rho * rho) + 3.0 * u + 3.0 * v;
+        const double det = sxx * syy - sxy * sxy, lr = log1p(-rho * rho);
+        part += -0.5 * (pr.iw_df + 3.0) * (2.0 * u + 2.0 * v + lr) - 0.5 * (sxx + syy) / det;
+        part += 1.3862943611198906188 + lr + 3.0 * u + 3.0 * v;  // log 4
     }
     return block_sum(part, red);
 }

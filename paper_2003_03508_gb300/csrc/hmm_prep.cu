@@ -109,9 +109,10 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
         if (job == 0) {
             em[EM_MUX * KP + k] = use ? mx : 0.0f;
             em[EM_MUY * KP + k] = use ? my : 0.0f;
-            em[EM_QA * KP + k] = use ? (float)(-0.5 * LOG2E * syy / det) : 0.0f;
-            em[EM_QB * KP + k] = use ? (float)(LOG2E * sxy / det) : 0.0f;
-            em[EM_QC * KP + k] = use ? (float)(-0.5 * LOG2E * sxx / det) : 0.0f;
+            const double inv = LOG2E / det;
+            em[EM_QA * KP + k] = use ? (float)(-0.5 * syy * inv) : 0.0f;
+            em[EM_QB * KP + k] = use ? (float)(sxy * inv) : 0.0f;
+            em[EM_QC * KP + k] = use ? (float)(-0.5 * sxx * inv) : 0.0f;
         } else if (job == 1) {
             const float v = use ? (float)(0.5 * log2(pk * pk / det) - LOG2_2PI) : -INFINITY;
             em[EM_CTR * KP + k] = v;
@@ -193,7 +194,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
                 const bool fits = !small && fabsf(mt) <= 1000.0f && fabsf(mn) <= 1000.0f;
                 sp.route[q] = bad ? ROUTE_BAD : ROUTE_STRANDS;
                 sp.jumps[q] = 0;
-                if (!bad && !fits) {
+                if (bad ? sp.bad_too : !fits) {
                     sp.route[q] = ROUTE_CHUNKS;
                     sp.todo[1 + atomicAdd(&sp.todo[0], 1)] = q;
                 }
