@@ -417,6 +417,7 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     }
     // every row of a posterior is used: pieces and warm-ups long enough that the
     // vectors have met before a piece ends
+    // (the few that have not run on one warp a piece, at a third of a strand's step)
     if (pl.smooth) L = std::max(L, 128);
     pl.strand_warm = pl.smooth ? 128 : strand_warm(pl.K, L, sparse, pl.strand_tensor);
     for (int s = 0; s < pl.n_seg; ++s) {
@@ -816,9 +817,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     float2 *packed = wp.packed;
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
-    // strands first; `todo` lists what is left to the chunk products (null: everything)
-    const StrandPtrs sp = wp.sp;
-    const int *todo = sp.todo;
+    StrandPtrs sp = wp.sp;
+    sp.bad_too = mode == Mode::SMOOTH;
     SmoothPtrs sm;
     float *fvec = nullptr, *bvec = nullptr;
     double *scan_part = nullptr, *scan_g0 = nullptr;
@@ -844,6 +844,12 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             return cv.off;
         };
         rc = ensure(c, c->fb, carve(nullptr) + 256);
+        if (rc == HMM_ENOMEM && sp.n) {
+            // no room for two more rows a step: scans over the chunk products
+            sp = StrandPtrs{};
+            sm = SmoothPtrs{};
+            rc = ensure(c, c->fb, carve(nullptr) + 256);
+        }
         if (rc) return rc;
         carve(c->fb.p);
         sm.warm = pl.strand_warm;
@@ -854,6 +860,9 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             sm.part = sm.g0 = nullptr;
         }
     }
+
+    // what the strands leave to the chunk products (null: everything)
+    const int *todo = sp.todo;
 
     // ---- launches ----
     // The whole sequence, on stream `s` (the caller's, or the capture stream).
@@ -922,7 +931,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             (uint64_t)(uintptr_t)cov, (uint64_t)(uintptr_t)xy, (uint64_t)(uintptr_t)tremor, (uint64_t)(uintptr_t)out,
             (uint64_t)(uintptr_t)c->work.p, c->plan_version, (uint64_t)n_prop, (uint64_t)K, (uint64_t)n_seg,
             (uint64_t)prec, (uint64_t)opts.init_mode, (uint64_t)renorm, (uint64_t)min_run, (uint64_t)L,
-            (uint64_t)T_total, (uint64_t)mode,
+            (uint64_t)T_total, (uint64_t)mode, (uint64_t)(todo != nullptr),
             (uint64_t)(uintptr_t)c->fb.p, (uint64_t)(uintptr_t)(out2 ? out2->gamma : nullptr),
             (uint64_t)(uintptr_t)(out2 ? out2->stats : nullptr)};
         if (c->call_exec && c->call_key == key) {
@@ -1092,7 +1101,8 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     if (rc) return rc;
     const Plan &pl = c->plan;
     const int K = prm->K, KP = pl.lay.KP;
-    const size_t C = std::max(1, pl.n_chunks), n = pl.strand_kp ? pl.strands.size() : 0, kp = (size_t)pl.strand_kp;
+    const size_t C = std::max(1, pl.n_chunks), kp = (size_t)pl.strand_kp;
+    size_t n = pl.strand_kp ? pl.strands.size() : 0;
     WorkPtrs wp;
     carve_work(c->work.p, 1, 1, pl.lay, pl, &wp);
     VitPtrs vp;
@@ -1124,6 +1134,12 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
         return cv.off;
     };
     rc = ensure(c, c->fb, carve(nullptr) + 1024);
+    if (rc == HMM_ENOMEM && n) {
+        // no room for the strands' back-pointers beside the chunks'
+        n = 0;
+        vp = VitPtrs{};
+        rc = ensure(c, c->fb, carve(nullptr) + 1024);
+    }
     if (rc) return rc;
     carve(c->fb.p);
     cudaError_t e = cudaSuccess;

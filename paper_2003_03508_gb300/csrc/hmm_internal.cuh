@@ -96,6 +96,7 @@ struct StrandPtrs {
     int *jumps = nullptr;      // [n_prop] some piece's jump is not itself
     int *route = nullptr;      // [n_prop]
     int *todo = nullptr;       // [1 + n_prop]
+    bool bad_too = false;      // invalid parameters take the chunk products as well (they fill every output)
 };
 
 // The posterior of one sequence by strands (hmm_smooth.cu). Row t belongs to
