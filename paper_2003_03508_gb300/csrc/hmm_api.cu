@@ -311,7 +311,7 @@ static bool tune_entry_valid(const TuneEntry &e) {
 // What a warp holds and costs, per kernel and padded state count: strands per
 // warp, warps an SM runs at once, whether warps come in fours of one proposal,
 // and cycles of one step when the warp runs alone on its scheduler (latency)
-// and when others fill it (issue).
+// and when others fill it (issue), as measured at T = 2^17 to 2^20.
 struct StrandCost {
     int per_warp, warps_per_sm, fours, latency, issue;
     bool tensor = false;

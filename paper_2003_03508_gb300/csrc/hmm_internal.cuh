@@ -3,7 +3,7 @@
 // Data layout in HBM (per call, carved out of one context-owned workspace):
 //   cblock  [n_prop][cstride] f32  per-proposal constants written by the prep
 //                                  kernel: emission coefficients (log2 domain,
-//                                  8 x KP SoA), P padded to KP x KP in FP32,
+//                                  EM_ALL x KP SoA), P padded to KP x KP in FP32,
 //                                  and the tensor-core operand images of P.
 //   packed  [n_packed] float2      chain observations x_1..x_{T-1} of every
 //                                  segment, each segment starting on a
@@ -13,6 +13,9 @@
 //   A0/e0   [n_prop][n_chunks]     chunk products (KP x KP f32) and per-row
 //                                  int32 power-of-two exponents.
 //   A_l/e_l levels of the product tree (int64 exponents).
+//   strands                        StrandPtrs: two vectors, exponent and scale per
+//                                  strand and proposal, the routes and the list
+//                                  of proposals left to the chunk products.
 //   qtab/qexp [n_prop][nb] run-length shortcut table (KP x KP f32 and KP int32
 //                                  row exponents per power), only when it is on.
 #pragma once

@@ -7,9 +7,11 @@
 // over are taken from it (jump); after JOIN_MOST steps the proposal is sent to
 // the chunk products.
 //
-// Nearly every piece meets at once (the warm-up covers the usual distance), so
-// the kernel reads 2 KP floats a piece; the rest are a few hundred steps of
-// one warp each, bound by the latency of a step.
+// Most pieces meet at once (the warm-up covers the usual distance), so the
+// kernel reads 2 KP floats a piece; the rest are up to some hundred steps of one
+// warp each, bound by the latency of a step: 0.2 us with P's column in registers
+// (K <= 32), four steps between two looks and two renormalisations (0.3 us with a
+// look at every step), about 1 us where P comes from the cache.
 #include "hmm_strand.cuh"
 
 namespace hmm {

@@ -17,8 +17,18 @@
 // the four products, which costs half as much again as one TF32 product.
 // Accumulation is FP32, and everything between two products stays FP32.
 //
-// P's fragments and the emission constants are in registers up to KP = 32 and
-// in shared memory above, where two row blocks a warp (MT = 2) halve the loads.
+// P's fragments are in registers up to KP = 32 and in shared memory above, where
+// two row blocks a warp (MT = 2) halve the loads; the emission constants are in
+// registers up to KP = 32 as well, but for BF16 at 32, whose hi and lo words need
+// the room (5.9 against 7.4 ms at T = 2^20, 256 proposals).
+//
+// What bounds it: MMAs, packed FMAs and selects share the register ports and do
+// not overlap (4 MMAs of 32 cycles and 16 packed FMAs of 36 take 68), so a step
+// of a warp costs their sum: at KP = 32 TF32 about 300 cycles for 16 strands,
+// 128 of them MMAs. K=32, T=2^20, 256 proposals: 4.35 ms TF32, 6.5 ms TF32_SPLIT,
+// 5.9 ms BF16; 13.5 ms on the CUDA cores, 60.5 ms by chunk products. Two warps a
+// scheduler without spills (4.37 ms) beat three with (4.81) and four (6.64); two
+// row blocks a warp at KP = 32 took 6.8 ms.
 #include <cuda_bf16.h>
 
 #include "hmm_strand.cuh"
