@@ -73,10 +73,12 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
 #pragma unroll
     for (int u = 0; u < NS; ++u) v[u] = own + u < K ? 1.0f : 0.0f;
 
-    // gamma's row t of the strand's own states from alpha's row and y
+    // gamma's row t of the strand's own states from alpha's row and y. gamma is
+    // the caller's: any float address, so 16-byte stores only where it allows them
+    const bool wide = (K & 3) == 0 && ((uintptr_t)sm.gamma & 15) == 0;
     auto put_gamma = [&](int64_t t, const float (&al)[NS], const float (&y)[NS], float r) {
         float *g = sm.gamma + t * K + own;
-        if ((K & 3) == 0 && NS == 4) {
+        if (wide && NS == 4) {
             if (own < K) *reinterpret_cast<float4 *>(g) = make_float4(al[0] * y[0] * r, al[1] * y[1] * r, al[NS - 2] * y[NS - 2] * r, al[NS - 1] * y[NS - 1] * r);
         } else {
 #pragma unroll
