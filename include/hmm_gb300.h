@@ -101,6 +101,17 @@ typedef struct {
 } hmm_opts;
 
 /*
+ * Vectors or chunk products. hmm_set_strands(ctx, 0) makes every later call of
+ * this context take the chunk products for everything (1, the default: vectors
+ * where they apply); with it their accuracy and speed can be looked at on any
+ * input. hmm_last_chunk_proposals writes how many proposals of the context's
+ * last call took the chunk products (for the one-sequence calls 0 or 1; for
+ * hmm_viterbi, whether its path did). It synchronises the stream.
+ */
+int hmm_set_strands(hmm_ctx *ctx, int on);
+int hmm_last_chunk_proposals(hmm_ctx *ctx, int32_t *n, void *stream);
+
+/*
  * Run-length shortcut (opts->runlen_min = n_min >= 1), for data in which
  * tremors are rare. The forward vectors then start further before their pieces;
  * the chunk products of what these leave use that every step without a

@@ -102,6 +102,8 @@ SIGNATURES = {
                                                _VP, _VP, _VP, ctypes.POINTER(hmm_opts), _VP, _VP]),
     "hmm_last_launch_count": (ctypes.c_int, [_VP]),
     "hmm_last_chunk_len": (ctypes.c_int, [_VP]),
+    "hmm_set_strands": (ctypes.c_int, [_VP, ctypes.c_int]),
+    "hmm_last_chunk_proposals": (ctypes.c_int, [_VP, ctypes.POINTER(_I32), _VP]),
     "hmm_set_call_graphs": (ctypes.c_int, [_VP, ctypes.c_int]),
     "hmm_last_call_graph": (ctypes.c_int, [_VP]),
     "hmm_default_chunk_len": (ctypes.c_int32, [_I32, _I32, _I32, ctypes.c_int64, _I32]),
@@ -239,6 +241,17 @@ class Context:
     @property
     def last_chunk_len(self) -> int:
         return int(self.lib.hmm_last_chunk_len(self.h))
+
+    def set_strands(self, on: bool = True):
+        """Carry one vector per piece where that applies (default), or take the
+        chunk products for everything."""
+        self._check(self.lib.hmm_set_strands(self.h, int(bool(on))))
+
+    def last_chunk_proposals(self, stream=None) -> int:
+        """How many proposals of the last call took the chunk products (synchronises)."""
+        n = _I32()
+        self._check(self.lib.hmm_last_chunk_proposals(self.h, ctypes.byref(n), _stream_ptr(stream)))
+        return int(n.value)
 
     def set_call_graphs(self, on: bool = True):
         """Capture and replay the batched call as a CUDA graph (default on)."""

@@ -75,6 +75,10 @@ struct hmm_ctx {
     int last_launches = 0;
     int last_L = 0;
     int n_sms = 0;
+    bool strands_on = true;
+    // who took chunk products in the last call: *last_todo proposals (device), or last_props where it is null
+    const int *last_todo = nullptr;
+    int last_props = 0;
     // phase timing
     bool prof_on = false;
     bool prof_pending = false;
@@ -629,6 +633,23 @@ int hmm_last_launch_count(const hmm_ctx *c) { return c ? c->last_launches : -1; 
 
 int hmm_last_chunk_len(const hmm_ctx *c) { return c ? c->last_L : -1; }
 
+int hmm_set_strands(hmm_ctx *c, int on) {
+    if (!c) return HMM_EINVAL;
+    c->strands_on = on != 0;
+    return HMM_OK;
+}
+
+int hmm_last_chunk_proposals(hmm_ctx *c, int32_t *n, void *stream) {
+    if (!c || !n) return HMM_EINVAL;
+    *n = c->last_props;
+    if (!c->last_todo) return HMM_OK;
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t e = cudaSetDevice(c->device);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(n, c->last_todo, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? HMM_OK : cuda_fail(c, e, "hmm_last_chunk_proposals");
+}
+
 int hmm_set_call_graphs(hmm_ctx *c, int on) {
     if (!c) return HMM_EINVAL;
     c->graphs_on = on != 0;
@@ -742,6 +763,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
                           const hmm_opts *opts_in, double *out, Mode mode, const SmoothOut *out2, void *stream) {
     if (!c) return HMM_EINVAL;
     c->last_launches = 0;
+    c->last_todo = nullptr;
+    c->last_props = 0;
     hmm_opts opts;
     if (opts_in) opts = *opts_in; else hmm_opts_default(&opts);
     if (K < 1 || K > 80) return fail(c, HMM_EINVAL, "K=%d outside 1..80", K);
@@ -820,7 +843,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     float2 *packed = wp.packed;
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
-    StrandPtrs sp = wp.sp;
+    StrandPtrs sp = c->strands_on ? wp.sp : StrandPtrs{};
     sp.bad_too = mode == Mode::SMOOTH;
     SmoothPtrs sm;
     float *fvec = nullptr, *bvec = nullptr;
@@ -866,6 +889,8 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
 
     // what the strands leave to the chunk products (null: everything)
     const int *todo = sp.todo;
+    c->last_todo = todo;
+    c->last_props = pl.n_chunks > 0 ? n_prop : 0;
 
     // ---- launches ----
     // The whole sequence, on stream `s` (the caller's, or the capture stream).
@@ -1105,7 +1130,7 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     const Plan &pl = c->plan;
     const int K = prm->K, KP = pl.lay.KP;
     const size_t C = std::max(1, pl.n_chunks), kp = (size_t)pl.strand_kp;
-    size_t n = pl.strand_kp ? pl.strands.size() : 0;
+    size_t n = pl.strand_kp && c->strands_on ? pl.strands.size() : 0;
     WorkPtrs wp;
     carve_work(c->work.p, 1, 1, pl.lay, pl, &wp);
     VitPtrs vp;
@@ -1155,6 +1180,7 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
         e = launch_viterbi(K, o.init_mode, pl.n_chunks, pl.L, pl.lay, pl.d_chunks, prm->pi, prm->P, wp.cblock, wp.head,
                            wp.packed, V, voff, ptr, bstate, bp, path, score, vp.chunks, (cudaStream_t)stream);
     c->last_launches += pl.n_chunks > 0 ? 3 : 2;
+    c->last_todo = vp.chunks;
     if (e != cudaSuccess) return cuda_fail(c, e, "viterbi launch");
     return HMM_OK;
 }
