@@ -425,7 +425,11 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
         return;
     }
     // one warp per piece: those unmet whose neighbour behind had met (its end is
-    // the true vector) go on, up to the next such piece
+    // the true vector) go on, up to the next such piece. Where the true vector
+    // meets the strand of a piece that is itself noted as unmet (against the
+    // untrue end of the one behind), the next piece's own run did set out from the
+    // truth; if that run ended unmet too, no warp of its own takes it on (its
+    // neighbour behind is noted), so this one goes on from what it ended with.
     const int x0 = blockIdx.x * 4 + warp;  // in the recursion's direction
     if (x0 >= sp.n) return;
     auto piece = [&](int x) { return BACK ? sp.n - 1 - x : x; };
@@ -438,6 +442,11 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
         // (all the rows that the piece's own run wrote, from a vector that was not the true one)
         how = starts(x) || spent > ROWS_MOST ? -1 : run(piece(x), sm.unmet[piece(x)] >> 1);
         spent += sp.desc[piece(x)].len;
+        if (how == 1 && x + 1 < sp.n && (sm.unmet[piece(x)] & 1) && (sm.unmet[piece(x + 1)] & 1)) {
+            ++x;
+            fetch(sm.carry + (size_t)piece(x) * KP, a);
+            how = 0;
+        }
     }
     if (how < 0 && lane == 0) send_to_chunks(sp, 0);
 }

@@ -349,6 +349,11 @@ vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__res
     for (int x = c0 + 1; x < sp.n && how == 0; ++x) {
         how = starts(x) || spent > VIT_MOST ? -1 : run(x, vp.unmet[x] >> 1);
         spent += sp.desc[x].len;
+        if (how == 1 && x + 1 < sp.n && (vp.unmet[x] & 1) && (vp.unmet[x + 1] & 1)) {
+            ++x;
+            fetch(vp.carry + (size_t)x * KP, a);
+            how = 0;
+        }
     }
     if (how < 0 && lane == 0) *vp.chunks = 1;
     if (how == 0) {  // to the sequence's end: this is its last vector
