@@ -206,7 +206,7 @@ cudaError_t launch_chunk_simt(int n_prop, int n_chunks, int L, int renorm, const
 // padded state count (0: K too large).
 int strand_simt_kp(int K);
 int strand_simt_per_warp(int KP);
-cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay,
                                const float *cblock, const float *pi, const float2 *head, const float2 *packed,
                                const StrandPtrs &sp, float *alpha, cudaStream_t st);
 cudaError_t launch_smooth(int K, int KP, int64_t steps, const ConstLayout &lay, const float *cblock, const float2 *head,

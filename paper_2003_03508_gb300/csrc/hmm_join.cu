@@ -290,7 +290,7 @@ cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int p
     // more. The rest runs on in FP32 to JOIN_TOL (K=80 BF16, 32 proposals:
     // 1000 us when every boundary had to).
     const float tol = !tensor ? JOIN_TOL : precision == HMM_PREC_BF16 ? 2.44140625e-4f : 3.90625e-3f;
-    const bool rt = precision == HMM_PREC_TF32;  // P as the strands have it
+    const bool rt = tensor && precision == HMM_PREC_TF32;  // P as the strands have it
     const long long warps = (long long)n_prop * sp.n;
     const unsigned grid = (unsigned)((warps + JOIN_WARPS - 1) / JOIN_WARPS);
     if (KP <= 32) join_kernel<1><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);

@@ -50,7 +50,7 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
 
     SimtStrand<C> S;
     S.init(sv[warp], lane);
-    S.load(cb + lay.off_p32, KPl, true, false);
+    S.load(cb + lay.off_p32, KPl, true);
     const int own = S.own;
     StrandBase base;
     base.load(em, KPl);

@@ -1,8 +1,10 @@
-// Strands on the CUDA cores (FP32): HMM_PREC_FP32_SIMT, and the other precisions
-// where the batch has too few strands for the tensor cores' rows (with P rounded
-// to TF32 for HMM_PREC_TF32). See hmm_strand.cuh for the method and
-// hmm_strand_simt.cuh for the layout. For the posterior of one sequence the
-// vector of every step is kept as well (hmm_smooth.cu).
+// Strands on the CUDA cores: FP32 whatever the call's precision, for
+// HMM_PREC_FP32_SIMT, for the other precisions where the batch has too few
+// strands for the tensor cores' rows, and for the posterior of one sequence,
+// which keeps the vector of every step (hmm_smooth.cu; its backward vectors are
+// FP32 too, so P is never rounded here: forward vectors on a P rounded to TF32
+// put gamma off by up to 2.6e-3). See hmm_strand.cuh for the method and
+// hmm_strand_simt.cuh for the layout.
 //
 // What bounds it: the FMA pipe's register ports. One step of a warp at KP = 32
 // is 64 packed FMAs of 2.2 cycles (the vector's pair repeats over four columns;
@@ -19,7 +21,7 @@ constexpr unsigned FULL = 0xffffffffu;
 // KEEP: alpha [steps + 1][KP] receives the (scaled) vector of every step
 template <class C, bool KEEP>
 __global__ void __launch_bounds__(32 * STRAND_WPC, C::MIN_CTAS)
-strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round_tf32, const float *__restrict__ cblock,
+strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const float *__restrict__ cblock,
                    const float *__restrict__ pi_all, const float2 *__restrict__ head,
                    const float2 *__restrict__ packed, StrandPtrs sp, float *__restrict__ alpha) {
     constexpr int KP = C::KP, G = C::G, NS = C::NS;
@@ -40,7 +42,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
 
     SimtStrand<C> S;
     S.init(sv[warp], lane);
-    S.load(cb + lay.off_p32, KPl, false, round_tf32);
+    S.load(cb + lay.off_p32, KPl, false);
     const int own = S.own;
     StrandBase base;
     base.load(em, KPl);
@@ -197,13 +199,13 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, bool round
 }
 
 template <int KP>
-cudaError_t launch_t(int n_prop, int K, int init_mode, const ConstLayout &lay, bool round_tf32, const float *cblock,
+cudaError_t launch_t(int n_prop, int K, int init_mode, const ConstLayout &lay, const float *cblock,
                      const float *pi, const float2 *head, const float2 *packed, const StrandPtrs &sp, float *alpha,
                      cudaStream_t st) {
     auto go = [&](auto kern, int per_warp) {
         const long long warps = (long long)n_prop * ((sp.n + per_warp - 1) / per_warp);
         kern<<<(unsigned)((warps + STRAND_WPC - 1) / STRAND_WPC), 32 * STRAND_WPC, 0, st>>>(
-            n_prop, K, init_mode, lay, round_tf32, cblock, pi, head, packed, sp, alpha);
+            n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha);
         return cudaGetLastError();
     };
     using C = SimtTile<KP>;
@@ -218,17 +220,16 @@ cudaError_t launch_t(int n_prop, int K, int init_mode, const ConstLayout &lay, b
 
 int strand_simt_kp(int K) { return K <= 4 ? 4 : K <= 8 ? 8 : K <= 16 ? 16 : K <= 32 ? 32 : K <= 64 ? 64 : 0; }
 
-cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+cudaError_t launch_strand_simt(int n_prop, int K, int init_mode, const ConstLayout &lay,
                                const float *cblock, const float *pi, const float2 *head, const float2 *packed,
                                const StrandPtrs &sp, float *alpha, cudaStream_t st) {
     if (sp.n == 0) return cudaSuccess;
-    const bool rt = precision == HMM_PREC_TF32;
     switch (strand_simt_kp(K)) {
-        case 4: return launch_t<4>(n_prop, K, init_mode, lay, rt, cblock, pi, head, packed, sp, alpha, st);
-        case 8: return launch_t<8>(n_prop, K, init_mode, lay, rt, cblock, pi, head, packed, sp, alpha, st);
-        case 16: return launch_t<16>(n_prop, K, init_mode, lay, rt, cblock, pi, head, packed, sp, alpha, st);
-        case 32: return launch_t<32>(n_prop, K, init_mode, lay, rt, cblock, pi, head, packed, sp, alpha, st);
-        case 64: return launch_t<64>(n_prop, K, init_mode, lay, rt, cblock, pi, head, packed, sp, alpha, st);
+        case 4: return launch_t<4>(n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha, st);
+        case 8: return launch_t<8>(n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha, st);
+        case 16: return launch_t<16>(n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha, st);
+        case 32: return launch_t<32>(n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha, st);
+        case 64: return launch_t<64>(n_prop, K, init_mode, lay, cblock, pi, head, packed, sp, alpha, st);
         default: return cudaErrorInvalidValue;
     }
 }

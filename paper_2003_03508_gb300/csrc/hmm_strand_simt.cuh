@@ -58,7 +58,7 @@ struct SimtStrand {
         buf = 0;
     }
     // the matrix: P (row vector times P), or with `transposed` P^T (P times a column vector)
-    __device__ __forceinline__ void load(const float *__restrict__ P, int KPl, bool transposed, bool round_tf32) {
+    __device__ __forceinline__ void load(const float *__restrict__ P, int KPl, bool transposed) {
 #pragma unroll
         for (int i = 0; i < C::NI / 2; ++i)
 #pragma unroll
@@ -68,11 +68,6 @@ struct SimtStrand {
                 for (int u = 0; u < 2; ++u) {
                     const int r = h * C::NI + 2 * i + u, k = 4 * cg + c;
                     v[u] = r < KPl && k < KPl ? P[transposed ? k * KPl + r : r * KPl + k] : 0.0f;
-                    if (round_tf32) {
-                        uint32_t b;
-                        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(v[u]));
-                        v[u] = __uint_as_float(b);
-                    }
                 }
                 p[c][i] = pack2(v[0], v[1]);
             }
