@@ -220,6 +220,7 @@ strand_mma_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const float
             emis(n).eval(o.x - base.cx, o.y - base.cy, tr, l[n][0], l[n][1]);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
+                l[n][u] -= lost;  // no product, nothing truncated (3.5e-4 a segment otherwise)
                 const int k2 = 8 * n + 2 * tig + u;
                 float w = 0.0f;
                 if (k2 < K) {
