@@ -909,7 +909,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             if (pl.strand_tensor) r = launch_strand_mma(n_prop, K, opts.init_mode, lay, prec, cblock, pi, head, packed, sp, s);
             else r = launch_strand_simt(n_prop, K, opts.init_mode, lay, cblock, pi, head, packed, sp, sm.alpha, s);
             if (r == cudaSuccess) r = launch_join(n_prop, K, pl.strand_kp, lay, prec, pl.strand_tensor, cblock, packed, sp, s);
-            launches += 2;
+            launches += pl.strand_tensor && KP > 32 ? 3 : 2;
             if (r == cudaSuccess && sm.alpha) {
                 r = launch_smooth(K, pl.strand_kp, steps_total, lay, cblock, head, packed, sp, sm, s);
                 launches += 5 + (sm.stats ? 2 : 0);

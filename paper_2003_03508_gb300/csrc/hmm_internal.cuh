@@ -45,11 +45,12 @@ enum {
     EM_CNO = 6,  // log2 (1 - p)
     EM_ROWS = 8,
     // the strands' form of the same density (hmm_strand.cuh)
-    EM_OFF = 8,  // [0], [1]: whole numbers next above the row maxima of EM_CTR and EM_CNO; [2], [3]: centre of the states
-    EM_UX = 9,   // u = ux x + uy y + u0, w = wy y + w0, x and y from the centre: log2 density = ctr - u^2 - w^2
+    EM_OFF = 8,  // [0], [1]: whole numbers next above the row maxima of EM_CTR and EM_CNO; with 16 states and more
+                 // [2], [3]: the states' centre, [4]: 1 where the affine forms serve (hmm_strand.cuh), else 0
+    EM_UX = 9,   // u = ux dx + uy dy, w = wy dy, from the mean: log2 density = ctr - u^2 - w^2
     EM_UY = 10,
-    EM_U0 = 11,
-    EM_WY = 12,
+    EM_WY = 11,
+    EM_U0 = 12,  // u = ux x + uy y + u0, w = wy y + w0, from the centre
     EM_W0 = 13,
     EM_ALL = 14,
 };
@@ -219,6 +220,13 @@ int strand_mma_per_warp(int KP);
 cudaError_t launch_strand_mma(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
                               const float *cblock, const float *pi, const float2 *head, const float2 *packed,
                               const StrandPtrs &sp, cudaStream_t st);
+// beyond 32 states: the proposals whose emissions take the affine forms, and the others
+cudaError_t launch_strand_mma_near(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+                                   const float *cblock, const float *pi, const float2 *head, const float2 *packed,
+                                   const StrandPtrs &sp, cudaStream_t st);
+cudaError_t launch_strand_mma_far(int n_prop, int K, int init_mode, const ConstLayout &lay, int precision,
+                                  const float *cblock, const float *pi, const float2 *head, const float2 *packed,
+                                  const StrandPtrs &sp, cudaStream_t st);
 cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int precision, bool tensor, const float *cblock,
                         const float2 *packed, const StrandPtrs &sp, cudaStream_t st);
 

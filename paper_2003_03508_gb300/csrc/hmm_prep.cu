@@ -74,7 +74,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
     float *em = cb + lay.off_emis;
     __shared__ float s_ctr[80], s_cno[80], s_centre[2];
     const int lane = threadIdx.x & 31;
-    bool bad = false, small = false;
+    bool bad = false, small = false, far = false;
 
     // per-state emission constants (log2 domain), padded states emit nothing
     const double LOG2E = 1.4426950408889634074;
@@ -82,7 +82,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
     const int job = threadIdx.x >> 6;
     float cx = 0.0f, cy = 0.0f;
     if (job == 3) {
-        // the states' centre: the strands take coordinates from it
+        // the states' centre: the affine forms take coordinates from it
         for (int k = lane; k < K; k += 32) {
             cx += mu[2 * k] / (float)K;
             cy += mu[2 * k + 1] / (float)K;
@@ -127,9 +127,10 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
             const double uy = use ? -ux * sxy / syy : 0.0, dx = (double)mx - cx, dy = (double)my - cy;
             em[EM_UX * KP + k] = (float)ux;
             em[EM_UY * KP + k] = (float)uy;
-            em[EM_U0 * KP + k] = use ? (float)-(ux * dx + uy * dy) : 0.0f;
             em[EM_WY * KP + k] = (float)wy;
+            em[EM_U0 * KP + k] = use ? (float)-(ux * dx + uy * dy) : 0.0f;
             em[EM_W0 * KP + k] = use ? (float)(-wy * dy) : 0.0f;
+            far = far || (use && !(fabs(ux * dx) + fabs(uy * dy) <= EMIS_NEAR && fabs(wy * dy) <= EMIS_NEAR));
         }
     }
     // rows of P and pi: non-negative, finite, summing to 1 within 1e-5 (a warp
@@ -169,6 +170,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
     }
     bad = __syncthreads_or(bad);
     small = __syncthreads_or(small);
+    far = __syncthreads_or(far);
     if (threadIdx.x < 32) {
         // EM_OFF: the emissions' largest constants, rounded up to whole numbers
         float mt = -INFINITY, mn = -INFINITY;
@@ -185,8 +187,11 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
             mn = isfinite(mn) ? ceilf(mn) : 0.0f;
             em[EM_OFF * KP] = mt;
             em[EM_OFF * KP + 1] = mn;
-            em[EM_OFF * KP + 2] = s_centre[0];
-            em[EM_OFF * KP + 3] = s_centre[1];
+            if (KP >= 16) {
+                em[EM_OFF * KP + 2] = s_centre[0];
+                em[EM_OFF * KP + 3] = s_centre[1];
+                em[EM_OFF * KP + 4] = far ? 0.0f : 1.0f;
+            }
             prop_bad[q] = bad;
             if (bad) atomicOr(status, ST_EINVAL);
             if (sp.route) {

@@ -107,8 +107,8 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
     for (int it = 0; it < nwin; ++it) {
         const int64_t w = wtop - it;
         const bool act = it < mine;
-        const float ox[4] = {na.x - base.cx, na.z - base.cx, nb.x - base.cx, nb.z - base.cx};
-        const float oy[4] = {na.y - base.cy, na.w - base.cy, nb.y - base.cy, nb.w - base.cy};
+        const float ox[4] = {na.x, na.z, nb.x, nb.z};
+        const float oy[4] = {na.y, na.w, nb.y, nb.w};
         if (it + 1 < mine) {
             na = obs[2 * (w - 1)];
             nb = obs[2 * (w - 1) + 1];

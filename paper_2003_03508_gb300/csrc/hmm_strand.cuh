@@ -71,60 +71,78 @@ __device__ __forceinline__ float ex2(float x) {
 }
 
 // What all states of a proposal share: the whole offsets of the factors, taken
-// out of ctr and cno so that every factor is at most 1, and the centre that the
-// strands' coordinates are taken from.
+// out of ctr and cno so that every factor is at most 1.
 struct StrandBase {
-    float offt, offn, cx, cy;
+    float offt, offn;
 
     __device__ __forceinline__ void load(const float *__restrict__ em, int KPl) {
         offt = em[EM_OFF * KPl];
         offn = em[EM_OFF * KPl + 1];
-        cx = em[EM_OFF * KPl + 2];
-        cy = em[EM_OFF * KPl + 3];
     }
     __device__ __forceinline__ float off(bool tremor) const { return tremor ? offt : offn; }
 };
 
-// Emission constants of two states. The density's exponent is taken as two
-// squares of affine forms of the centred location, five packed operations a
-// pair where differences from the mean and their products take seven; the FMA
-// pipe is what the strands run on. Its rounding is that of the location itself
-// (float32, at most 2^-24 of the states' spread): 1e-5 in log2 at three
-// deviations of a state 1/60 of the box wide, without bias over a chain.
-struct Emis2 {
-    f32x2 ux, uy, u0, wy, w0, nctr;  // nctr = -(ctr - offset)
+// Emission constants of two states. The density's exponent is two squares of
+// linear forms of the difference from the mean, seven packed operations a pair.
+// AFFINE: five, as affine forms of the location from the states' centre, which
+// lose the bits that the mean's distance has over the state's width (s = |u0|,
+// |w0|: 2^-23 s |u| of a log2 factor). FP32 never takes them: they
+// cost the CUDA cores nothing (log L, host and run-length calls within 1.5%), and
+// at 25 states 0.2 km wide log L was 1.5e-6 off with them, 1.7e-7 without. The
+// tensor cores' strands do where s is at most EMIS_NEAR for every state (the
+// synthetic recipe stays below 40): 2e-5 of a factor at three deviations, a tenth
+// of the rounding of a TF32 operand; K=32, T=2^20, 256 proposals 4.35 ms with
+// them, 4.57 without.
+constexpr float EMIS_NEAR = 64.0f;
+
+template <bool AFFINE>
+struct EmisPair {
+    f32x2 p, q, ux, uy, wy, nctr;  // p, q: minus the mean (AFFINE: u0, w0); nctr = -(ctr - offset)
     float cno0, cno1;
 
     __device__ __forceinline__ void load(const float *__restrict__ em, int KPl, int k0, float offt, float offn) {
+        constexpr int rows[5] = {AFFINE ? EM_U0 : EM_MUX, AFFINE ? EM_W0 : EM_MUY, EM_UX, EM_UY, EM_WY};
         float v[2][7];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int k = k0 + u;
             const bool in = k < KPl;
 #pragma unroll
-            for (int r = 0; r < 5; ++r) v[u][r] = in ? em[(EM_UX + r) * KPl + k] : 0.0f;
+            for (int r = 0; r < 5; ++r) {
+                v[u][r] = in ? em[rows[r] * KPl + k] : 0.0f;
+                if (!AFFINE && r < 2) v[u][r] = -v[u][r];
+            }
             v[u][5] = in ? offt - em[EM_CTR * KPl + k] : INFINITY;
             v[u][6] = in ? em[EM_CNO * KPl + k] - offn : -INFINITY;
         }
-        ux = pack2(v[0][0], v[1][0]);
-        uy = pack2(v[0][1], v[1][1]);
-        u0 = pack2(v[0][2], v[1][2]);
-        wy = pack2(v[0][3], v[1][3]);
-        w0 = pack2(v[0][4], v[1][4]);
+        p = pack2(v[0][0], v[1][0]);
+        q = pack2(v[0][1], v[1][1]);
+        ux = pack2(v[0][2], v[1][2]);
+        uy = pack2(v[0][3], v[1][3]);
+        wy = pack2(v[0][4], v[1][4]);
         nctr = pack2(v[0][5], v[1][5]);
         cno0 = v[0][6];
         cno1 = v[1][6];
     }
-    // log2 emission factors of the centred observation (x, y)
+    // log2 emission factors of the observation (x, y) (AFFINE: from the centre)
     __device__ __forceinline__ void eval(float x, float y, bool tremor, float &l0, float &l1) const {
         const f32x2 xx = pack2(x, x), yy = pack2(y, y);
-        const f32x2 u = fma2(ux, xx, fma2(uy, yy, u0)), w = fma2(wy, yy, w0);
+        f32x2 u, w;
+        if (AFFINE) {
+            u = fma2(ux, xx, fma2(uy, yy, p));
+            w = fma2(wy, yy, q);
+        } else {
+            const f32x2 dx = add2(xx, p), dy = add2(yy, q);
+            u = fma2(ux, dx, mul2(uy, dy));
+            w = mul2(wy, dy);
+        }
         float n0, n1;
         unpack2(fma2(w, w, fma2(u, u, nctr)), n0, n1);
         l0 = tremor ? -n0 : cno0;
         l1 = tremor ? -n1 : cno1;
     }
 };
+using Emis2 = EmisPair<false>;
 
 // Marks proposal q for the chunk products (once).
 __device__ __forceinline__ void send_to_chunks(const StrandPtrs &sp, int q) {

@@ -71,7 +71,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
         const bool tr = !isnan(o.x);
         float l[NS], m = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < NS / 2; ++u) ec[u].eval(o.x - base.cx, o.y - base.cy, tr, l[2 * u], l[2 * u + 1]);
+        for (int u = 0; u < NS / 2; ++u) ec[u].eval(o.x, o.y, tr, l[2 * u], l[2 * u + 1]);
 #pragma unroll
         for (int u = 0; u < NS; ++u) {
             const int s = own + u;
@@ -107,7 +107,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
         nb = obs[1];
     }
     for (int w = 0; w < nwin; ++w) {
-        float ox[4] = {na.x, na.z, nb.x, nb.z}, oy[4] = {na.y, na.w, nb.y, nb.w};
+        const float ox[4] = {na.x, na.z, nb.x, nb.z}, oy[4] = {na.y, na.w, nb.y, nb.w};
         if (4 * (w + 1) < total) {
             na = obs[2 * (w + 1)];
             nb = obs[2 * (w + 1) + 1];
@@ -116,11 +116,6 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
         int step_e = 0;
 #pragma unroll
         for (int u = 0; u < NS; ++u) keep[u] = v[u];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            ox[j] -= base.cx;
-            oy[j] -= base.cy;
-        }
         const int left = total - 4 * w;  // steps of this strand still to do
         const bool own_steps = KEEP && left >= 4 && 4 * w >= d.warm;
 #pragma unroll
