@@ -52,7 +52,9 @@ enum {
     EM_WY = 11,
     EM_U0 = 12,  // u = ux x + uy y + u0, w = wy y + w0, from the centre
     EM_W0 = 13,
-    EM_ALL = 14,
+    EM_SC = 14,  // the strands' offset [0] - log2 constant of a tremor
+    EM_QF = 15,  // and their factor of a step without one: (1 - p) 2^-offset [1]
+    EM_ALL = 16,
 };
 
 // a step whose best state has log2-emission below -EXP_LIMIT is not representable

@@ -73,6 +73,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
     float *cb = cblock + (size_t)q * lay.stride;
     float *em = cb + lay.off_emis;
     __shared__ float s_ctr[80], s_cno[80], s_centre[2];
+    __shared__ double s_ctr64[80];
     const int lane = threadIdx.x & 31;
     bool bad = false, small = false, far = false;
 
@@ -114,9 +115,11 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
             em[EM_QB * KP + k] = use ? (float)(sxy * inv) : 0.0f;
             em[EM_QC * KP + k] = use ? (float)(-0.5 * sxx * inv) : 0.0f;
         } else if (job == 1) {
-            const float v = use ? (float)(0.5 * log2(pk * pk / det) - LOG2_2PI) : -INFINITY;
+            const double v64 = use ? 0.5 * log2(pk * pk / det) - LOG2_2PI : -INFINITY;
+            const float v = (float)v64;
             em[EM_CTR * KP + k] = v;
             s_ctr[k] = v;
+            s_ctr64[k] = v64;
         } else if (job == 2) {
             const float v = use ? (float)log2(1.0 - pk) : -INFINITY;
             em[EM_CNO * KP + k] = v;
@@ -182,9 +185,19 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
             mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
             mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
         }
+        mt = isfinite(mt) ? ceilf(mt) : 0.0f;
+        mn = isfinite(mn) ? ceilf(mn) : 0.0f;
+        // The strands' constants, rounded once from 64 bits. EX2_BIAS: what
+        // ex2.approx loses in the mean, for arguments below 0 as all are here
+        // (-5.0e-8 of its value, measured), spread over the states by the rounding.
+        // The quiet steps' factor is no exponential at all: that loss, the same at
+        // every quiet step, was most of log L's error (rare tremors: 6.0e-8 of it).
+        constexpr double EX2_BIAS = 7.2e-8;
+        for (int k = lane; k < KP; k += 32) {
+            em[EM_SC * KP + k] = (float)((double)mt - s_ctr64[k] - EX2_BIAS);
+            em[EM_QF * KP + k] = s_cno[k] > -INFINITY ? (float)((1.0 - (double)p[k]) * (double)pow2f(-(int)mn)) : 0.0f;
+        }
         if (lane == 0) {
-            mt = isfinite(mt) ? ceilf(mt) : 0.0f;
-            mn = isfinite(mn) ? ceilf(mn) : 0.0f;
             em[EM_OFF * KP] = mt;
             em[EM_OFF * KP + 1] = mn;
             if (KP >= 16) {

@@ -56,7 +56,7 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
     base.load(em, KPl);
     Emis2 ec[NS / 2];
 #pragma unroll
-    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u, base.offt, base.offn);
+    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u);
 
     const int k = wid * C::PER_WARP + S.slot;
     const int sid = k < sp.n ? k : -1;
@@ -134,9 +134,9 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
             for (int h = 1; h >= 0; --h) {
                 const int j = j2 + h;
 #pragma unroll
-                for (int u = 0; u < NS / 2; ++u) ec[u].eval(ox[j], oy[j], !isnan(ox[j]), f[h][2 * u], f[h][2 * u + 1]);
+                for (int u = 0; u < NS / 2; ++u) ec[u].factors(ox[j], oy[j], !isnan(ox[j]), 0.0f, f[h][2 * u], f[h][2 * u + 1]);
 #pragma unroll
-                for (int u = 0; u < NS; ++u) f[h][u] = ex2(f[h][u]) * v[u];
+                for (int u = 0; u < NS; ++u) f[h][u] *= v[u];
                 S.mul(f[h], y[h]);
 #pragma unroll
                 for (int u = 0; u < NS; ++u) v[u] = y[h][u];
@@ -186,12 +186,14 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
                 for (int u = 0; u < NS; ++u) al[u] = 0.0f;
                 if (todo && own_steps) S.fetch(sm.alpha + i * KP, al);
 #pragma unroll
-                for (int u = 0; u < NS / 2; ++u) ec[u].eval(x, yy, !isnan(x), l[2 * u], l[2 * u + 1]);
+                for (int u = 0; u < NS / 2; ++u) ec[u].sizes(x, yy, !isnan(x), l[2 * u], l[2 * u + 1]);
                 float mx = S.max_all(S.max_own(l));
                 const bool emits = mx + base.off(!isnan(x)) >= -(float)EXP_LIMIT;
                 const float fm = emits ? floorf(mx) : 0.0f;
 #pragma unroll
-                for (int u = 0; u < NS; ++u) l[u] = ex2(l[u] - fm) * v[u];
+                for (int u = 0; u < NS / 2; ++u) ec[u].factors(x, yy, !isnan(x), fm, l[2 * u], l[2 * u + 1]);
+#pragma unroll
+                for (int u = 0; u < NS; ++u) l[u] *= v[u];
                 S.mul(l, y);
                 mx = S.max_all(S.max_own(y));
                 const bool can = emits && mx >= STRAND_SHRINK && mx <= STRAND_GROW;

@@ -97,10 +97,11 @@ constexpr float EMIS_NEAR = 64.0f;
 
 template <bool AFFINE>
 struct EmisPair {
-    f32x2 p, q, ux, uy, wy, nctr;  // p, q: minus the mean (AFFINE: u0, w0); nctr = -(ctr - offset)
-    float cno0, cno1;
+    f32x2 p, q, ux, uy, wy, nctr;  // p, q: minus the mean (AFFINE: u0, w0); nctr: offset - constant
+    float quiet0, quiet1;          // factors of a step without a tremor
 
-    __device__ __forceinline__ void load(const float *__restrict__ em, int KPl, int k0, float offt, float offn) {
+    // `up`: log2 of what every factor is made larger by
+    __device__ __forceinline__ void load(const float *__restrict__ em, int KPl, int k0, float up = 0.0f) {
         constexpr int rows[5] = {AFFINE ? EM_U0 : EM_MUX, AFFINE ? EM_W0 : EM_MUY, EM_UX, EM_UY, EM_WY};
         float v[2][7];
 #pragma unroll
@@ -112,8 +113,9 @@ struct EmisPair {
                 v[u][r] = in ? em[rows[r] * KPl + k] : 0.0f;
                 if (!AFFINE && r < 2) v[u][r] = -v[u][r];
             }
-            v[u][5] = in ? offt - em[EM_CTR * KPl + k] : INFINITY;
-            v[u][6] = in ? em[EM_CNO * KPl + k] - offn : -INFINITY;
+            v[u][5] = in ? em[EM_SC * KPl + k] - up : INFINITY;
+            v[u][6] = in ? em[EM_QF * KPl + k] : 0.0f;
+            if (up != 0.0f) v[u][6] *= exp2f(up);
         }
         p = pack2(v[0][0], v[1][0]);
         q = pack2(v[0][1], v[1][1]);
@@ -121,11 +123,11 @@ struct EmisPair {
         uy = pack2(v[0][3], v[1][3]);
         wy = pack2(v[0][4], v[1][4]);
         nctr = pack2(v[0][5], v[1][5]);
-        cno0 = v[0][6];
-        cno1 = v[1][6];
+        quiet0 = v[0][6];
+        quiet1 = v[1][6];
     }
-    // log2 emission factors of the observation (x, y) (AFFINE: from the centre)
-    __device__ __forceinline__ void eval(float x, float y, bool tremor, float &l0, float &l1) const {
+    // log2 factors of a tremor at (x, y) (AFFINE: from the centre)
+    __device__ __forceinline__ void density(float x, float y, float &l0, float &l1) const {
         const f32x2 xx = pack2(x, x), yy = pack2(y, y);
         f32x2 u, w;
         if (AFFINE) {
@@ -138,8 +140,23 @@ struct EmisPair {
         }
         float n0, n1;
         unpack2(fma2(w, w, fma2(u, u, nctr)), n0, n1);
-        l0 = tremor ? -n0 : cno0;
-        l1 = tremor ? -n1 : cno1;
+        l0 = -n0;
+        l1 = -n1;
+    }
+    // emission factors of an observation, a tremor's relative to 2^fm
+    __device__ __forceinline__ void factors(float x, float y, bool tremor, float fm, float &f0, float &f1) const {
+        density(x, y, f0, f1);
+        f0 = tremor ? ex2(f0 - fm) : quiet0;
+        f1 = tremor ? ex2(f1 - fm) : quiet1;
+    }
+    // What fm is taken from: log2 factors of a tremor; without one 0 for every
+    // state that emits (their factors are in (2^-25, 1], the largest above 1/2).
+    __device__ __forceinline__ void sizes(float x, float y, bool tremor, float &l0, float &l1) const {
+        density(x, y, l0, l1);
+        if (!tremor) {
+            l0 = quiet0 > 0.0f ? 0.0f : -INFINITY;
+            l1 = quiet1 > 0.0f ? 0.0f : -INFINITY;
+        }
     }
 };
 using Emis2 = EmisPair<false>;

@@ -131,7 +131,7 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
     base.load(em, KPl);
     const float cx = NEAR ? em[EM_OFF * KPl + 2] : 0.0f, cy = NEAR ? em[EM_OFF * KPl + 3] : 0.0f;
     // the factors' offsets; TF32 operands lose TRUNC_LOG2 a step
-    const float lost = C::MODE == M_TF32 ? TRUNC_LOG2 : 0.0f, et = base.offt - lost, en = base.offn - lost;
+    const float lost = C::MODE == M_TF32 ? TRUNC_LOG2 : 0.0f;
 
     uint32_t breg[C::REGS ? NS : 1][C::REGS ? NT : 1][NB];
     EmisPair<NEAR> ereg[C::EREG ? NT : 1];
@@ -141,11 +141,11 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
     auto fill_emission = [&](int first, int step) {
         for (int i = first; i < NT * 4; i += step) {
             EmisPair<NEAR> e;
-            e.load(em, KPl, 8 * (i / 4) + 2 * (i % 4), et, en);
+            e.load(em, KPl, 8 * (i / 4) + 2 * (i % 4), lost);
             // pairs (u, u + 1) of a lane side by side: 16-byte loads
             f32x2 *d = sE + (i / 4) * 32 + (i % 4) * 2;
             d[0] = e.p; d[1] = e.q; d[8] = e.ux; d[9] = e.uy; d[16] = e.wy; d[17] = e.nctr;
-            d[24] = pack2(e.cno0, e.cno1);
+            d[24] = pack2(e.quiet0, e.quiet1);
         }
     };
     if (C::REGS) {
@@ -156,7 +156,7 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
             for (int n = 0; n < (C::REGS ? NT : 1); ++n) b_fragment<C>(P, KPl, s, n, lane, breg[s][n]);
         if (C::EREG) {
 #pragma unroll
-            for (int n = 0; n < (C::EREG ? NT : 1); ++n) ereg[n].load(em, KPl, 8 * n + 2 * tig, et, en);
+            for (int n = 0; n < (C::EREG ? NT : 1); ++n) ereg[n].load(em, KPl, 8 * n + 2 * tig, lost);
         } else {
             fill_emission(lane, 32);
             __syncwarp();
@@ -181,7 +181,7 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
         const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(d), b = *reinterpret_cast<const ulonglong2 *>(d + 8),
                          c = *reinterpret_cast<const ulonglong2 *>(d + 16);
         e.p = a.x; e.q = a.y; e.ux = b.x; e.uy = b.y; e.wy = c.x; e.nctr = c.y;
-        unpack2(d[24], e.cno0, e.cno1);
+        unpack2(d[24], e.quiet0, e.quiet1);
         return e;
     };
     const int ct = (int)base.offt, cn = (int)base.offn;
@@ -205,13 +205,13 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
         const bool at_head = (d.flags & SD_HEAD) != 0;
         const float2 o = head[d.seg];
         const bool tr = !isnan(o.x);
+        const float hx = NEAR ? o.x - cx : o.x, hy = NEAR ? o.y - cy : o.y;
         float l[NT][2], m = -INFINITY;
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
-            emis(n).eval(NEAR ? o.x - cx : o.x, NEAR ? o.y - cy : o.y, tr, l[n][0], l[n][1]);
+            emis(n).sizes(hx, hy, tr, l[n][0], l[n][1]);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                l[n][u] -= lost;  // no product, nothing truncated (3.5e-4 a segment otherwise)
                 const int k2 = 8 * n + 2 * tig + u;
                 float w = 0.0f;
                 if (k2 < K) {
@@ -233,14 +233,18 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
         const float fm = emits ? floorf(m) : 0.0f;
         if (at_head && !emits) bad |= 1u << r;
         if (at_head && emits) e32[r] = (int)fm + (tr ? ct : cn);
+        // no product here, nothing truncated: `lost` comes off again (3.5e-4 a segment otherwise)
+        const float kept = C::MODE == M_TF32 ? exp2f(-lost) : 1.0f;
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
+        for (int n = 0; n < NT; ++n) {
+            emis(n).factors(hx, hy, tr, fm, l[n][0], l[n][1]);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 float &x = v[r / 2][n][2 * (r & 1) + u];
-                if (at_head && emits) x = x > 0.0f ? x * ex2(l[n][u] - fm) : 0.0f;
+                if (at_head && emits) x = x > 0.0f ? x * (l[n][u] * kept) : 0.0f;
                 else x = 8 * n + 2 * tig + u < K ? 1.0f : 0.0f;
             }
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nwin = max(nwin, __shfl_xor_sync(FULL, nwin, o));
@@ -356,10 +360,10 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
                 const EmisPair<NEAR> e = emis(n);
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {
-                    float l0, l1;
-                    e.eval(o[r].x, o[r].y, !isnan(o[r].x), l0, l1);
-                    v[r / 2][n][2 * (r & 1)] = acc[r / 2][2 * (r & 1)] * ex2(l0);
-                    v[r / 2][n][2 * (r & 1) + 1] = acc[r / 2][2 * (r & 1) + 1] * ex2(l1);
+                    float f0, f1;
+                    e.factors(o[r].x, o[r].y, !isnan(o[r].x), 0.0f, f0, f1);
+                    v[r / 2][n][2 * (r & 1)] = acc[r / 2][2 * (r & 1)] * f0;
+                    v[r / 2][n][2 * (r & 1) + 1] = acc[r / 2][2 * (r & 1) + 1] * f1;
                 }
             });
         }
@@ -402,7 +406,7 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
 #pragma unroll
                     for (int r = 0; r < NR; ++r) {
                         float l0, l1;
-                        e.eval(o[r].x, o[r].y, !isnan(o[r].x), l0, l1);
+                        e.sizes(o[r].x, o[r].y, !isnan(o[r].x), l0, l1);
                         mx[r] = fmaxf(mx[r], fmaxf(l0, l1));
                     }
                 }
@@ -420,10 +424,10 @@ carry_strands(int q, int wq, int wpp, int K, int init_mode, const ConstLayout &l
                     const EmisPair<NEAR> e = emis(n);
 #pragma unroll
                     for (int r = 0; r < NR; ++r) {
-                        float l0, l1;
-                        e.eval(o[r].x, o[r].y, !isnan(o[r].x), l0, l1);
-                        z[r / 2][n][2 * (r & 1)] = acc[r / 2][2 * (r & 1)] * ex2(l0 - fm[r]);
-                        z[r / 2][n][2 * (r & 1) + 1] = acc[r / 2][2 * (r & 1) + 1] * ex2(l1 - fm[r]);
+                        float f0, f1;
+                        e.factors(o[r].x, o[r].y, !isnan(o[r].x), fm[r], f0, f1);
+                        z[r / 2][n][2 * (r & 1)] = acc[r / 2][2 * (r & 1)] * f0;
+                        z[r / 2][n][2 * (r & 1) + 1] = acc[r / 2][2 * (r & 1) + 1] * f1;
                     }
                 });
 #pragma unroll

@@ -49,7 +49,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
     const int ct = (int)base.offt, cn = (int)base.offn;
     Emis2 ec[NS / 2];
 #pragma unroll
-    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u, base.offt, base.offn);
+    for (int u = 0; u < NS / 2; ++u) ec[u].load(em, KPl, own + 2 * u);
 
     const int k = (int)(wid % wpp) * C::PER_WARP + S.slot;
     const int sid = k < sp.n ? sp.order[k] : -1;
@@ -71,7 +71,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
         const bool tr = !isnan(o.x);
         float l[NS], m = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < NS / 2; ++u) ec[u].eval(o.x, o.y, tr, l[2 * u], l[2 * u + 1]);
+        for (int u = 0; u < NS / 2; ++u) ec[u].sizes(o.x, o.y, tr, l[2 * u], l[2 * u + 1]);
 #pragma unroll
         for (int u = 0; u < NS; ++u) {
             const int s = own + u;
@@ -94,8 +94,10 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
         if (at_head && emits) e32 = (int)fm + (tr ? ct : cn);
         bad = at_head && !emits;
 #pragma unroll
+        for (int u = 0; u < NS / 2; ++u) ec[u].factors(o.x, o.y, tr, fm, l[2 * u], l[2 * u + 1]);
+#pragma unroll
         for (int u = 0; u < NS; ++u) {
-            if (at_head && emits) v[u] = v[u] > 0.0f ? v[u] * ex2(l[u] - fm) : 0.0f;
+            if (at_head && emits) v[u] = v[u] > 0.0f ? v[u] * l[u] : 0.0f;
             else v[u] = own + u < K ? 1.0f : 0.0f;
         }
         if (KEEP && (d.flags & SD_FIRST) && sid >= 0) S.store(alpha, v);
@@ -124,9 +126,7 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
             const bool tr = !isnan(ox[j]);
             step_e += tr ? ct : cn;
 #pragma unroll
-            for (int u = 0; u < NS / 2; ++u) ec[u].eval(ox[j], oy[j], tr, f[2 * u], f[2 * u + 1]);
-#pragma unroll
-            for (int u = 0; u < NS; ++u) f[u] = ex2(f[u]);
+            for (int u = 0; u < NS / 2; ++u) ec[u].factors(ox[j], oy[j], tr, 0.0f, f[2 * u], f[2 * u + 1]);
             S.mul(v, y);
 #pragma unroll
             for (int u = 0; u < NS; ++u) v[u] = y[u] * f[u];
@@ -152,12 +152,14 @@ strand_simt_kernel(int n_prop, int K, int init_mode, ConstLayout lay, const floa
                 const float yy = j == 0 ? oy[0] : j == 1 ? oy[1] : j == 2 ? oy[2] : oy[3];
                 const bool tr = !isnan(x);
 #pragma unroll
-                for (int u = 0; u < NS / 2; ++u) ec[u].eval(x, yy, tr, l[2 * u], l[2 * u + 1]);
+                for (int u = 0; u < NS / 2; ++u) ec[u].sizes(x, yy, tr, l[2 * u], l[2 * u + 1]);
                 mx = S.max_all(S.max_own(l));
                 const bool emits = mx + base.off(tr) >= -(float)EXP_LIMIT;
                 const float fm = emits ? floorf(mx) : 0.0f;
 #pragma unroll
-                for (int u = 0; u < NS; ++u) z[u] = y[u] * ex2(l[u] - fm);
+                for (int u = 0; u < NS / 2; ++u) ec[u].factors(x, yy, tr, fm, l[2 * u], l[2 * u + 1]);
+#pragma unroll
+                for (int u = 0; u < NS; ++u) z[u] = y[u] * l[u];
                 mx = S.max_all(S.max_own(z));
                 const bool can = emits && mx >= STRAND_SHRINK && mx <= STRAND_GROW;
                 const bool mine = redo && j < left;
