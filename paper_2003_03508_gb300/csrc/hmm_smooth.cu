@@ -243,7 +243,12 @@ __global__ void __launch_bounds__(128)
 rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__restrict__ cb,
                  const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm) {
     __shared__ __align__(16) float2 sag[4][32 * NC];
-    constexpr float tol = 3.0517578125e-5f;  // 2^-15, as in the likelihood's join
+    // Every row is a result, so vectors have met where they differ by little more
+    // than FP32's rounding: with rare tremors 2^-19.8 of an entry at the median and
+    // 2^-18.7 at most of the time for K = 16, 2^-18.8 and 2^-17.8 for K = 32, 2^-17.9
+    // and 2^-16.8 for K = 64 (a float32 replay). With 2^-15, which the likelihood's
+    // join takes, gamma was up to 1.3e-5 off (K = 16), 5.4e-6 now.
+    const float tol = KP <= 16 ? 3.814697265625e-6f : KP <= 32 ? 7.62939453125e-6f : 1.52587890625e-5f;  // 2^-18, -17, -16
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
     const float *em = cb + lay.off_emis, *P = cb + lay.off_p32;
