@@ -459,11 +459,24 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
 }
 
 // ---- E-step statistics ----
-constexpr int SX_THREADS = 256, SX_BLOCK = 64;
+constexpr int SX_THREADS = 256, SX_BLOCK = 64, SX_GROUP = 8, SX_FLUSH = 64;
+
+// hi + lo += x, what the addition drops kept in lo (Knuth's two-sum)
+__device__ __forceinline__ void add_kept(float &hi, float &lo, float x) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
+}
 
 // One CTA per range of steps: sum of alpha_i (x) u_i times P, and the gamma
-// moments about the states' means, FP32 within a block of 64 steps and FP64
-// across blocks; the CTAs' sums are added in order by a later kernel.
+// moments about the states' means. Sums as in 64 bits: every term rounded to
+// FP32, groups of SX_GROUP products in FP32 (a quiet stretch adds nearly the same
+// term again and again, whose rounding would repeat), what their additions drop
+// kept beside them for up to SX_FLUSH blocks of 64 steps, FP64 across those. FP64
+// additions and conversions run at two a cycle and SM here: eleven sums a thread
+// and block were most of this kernel (EM step, K=12,
+// T=200,003: 216 us in all with one addition each, 252 with two, 209 with none). The CTAs'
+// sums are added in order by a later kernel.
 template <int KP>
 __global__ void __launch_bounds__(SX_THREADS)
 stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__restrict__ cb,
@@ -472,6 +485,7 @@ stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__
     constexpr int CQ = KP / 4;                                        // column quads
     constexpr int NR = KP * CQ <= SX_THREADS ? 1 : KP * CQ / SX_THREADS;  // rows of N per thread
     constexpr int SL = KP * CQ <= SX_THREADS ? SX_THREADS / (KP * CQ) : 1;  // step slices of N
+    constexpr int GROUP = SX_BLOCK / SL < SX_GROUP ? SX_BLOCK / SL : SX_GROUP;  // products of one slice in FP32
     constexpr int MS = SX_THREADS / KP;                               // step slices of the moments
     __shared__ __align__(16) float sA[SX_BLOCK][KP], sU[SX_BLOCK][KP];
     __shared__ float2 sO[SX_BLOCK];
@@ -488,18 +502,34 @@ stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__
     const float mx = mk < K ? em[EM_MUX * lay.KP + mk] : 0.0f, my = mk < K ? em[EM_MUY * lay.KP + mk] : 0.0f;
     double mom[7] = {};
     // gamma rows: i + 1 for each of this CTA's steps i, and row 0 for the first CTA
-    auto add = [&](float (&s)[7], float g, float2 o) {
-        s[0] += g;
+    auto add = [&](float (&s)[7], float (&l)[7], float g, float2 o) {
+        add_kept(s[0], l[0], g);
         if (!isnan(o.x)) {
             const float dx = o.x - mx, dy = o.y - my;
-            s[1] += g;
-            s[2] = fmaf(g, dx, s[2]);
-            s[3] = fmaf(g, dy, s[3]);
-            s[4] = fmaf(g * dx, dx, s[4]);
-            s[5] = fmaf(g * dx, dy, s[5]);
-            s[6] = fmaf(g * dy, dy, s[6]);
+            add_kept(s[1], l[1], g);
+            add_kept(s[2], l[2], g * dx);
+            add_kept(s[3], l[3], g * dy);
+            add_kept(s[4], l[4], g * dx * dx);
+            add_kept(s[5], l[5], g * dx * dy);
+            add_kept(s[6], l[6], g * dy * dy);
         }
     };
+    float hi[NR][4] = {}, lo[NR][4] = {}, m[7] = {}, ml[7] = {};
+    auto flush = [&]() {
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                acc[r][c] += (double)hi[r][c] + (double)lo[r][c];
+                hi[r][c] = lo[r][c] = 0.0f;
+            }
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+            mom[c] += (double)m[c] + (double)ml[c];
+            m[c] = ml[c] = 0.0f;
+        }
+    };
+    int done = 0;
     for (int64_t b = i0; b < i1; b += SX_BLOCK) {
         const int n = (int)min((int64_t)SX_BLOCK, i1 - b);
         __syncthreads();
@@ -511,39 +541,38 @@ stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__
         }
         for (int x = tid; x < n; x += SX_THREADS) sO[x] = packed[b + x];
         __syncthreads();
-        float t[NR][4] = {};
         if (sl < SL) {
-            for (int s = sl; s < SX_BLOCK; s += SL) {
-                const float4 u = *reinterpret_cast<const float4 *>(&sU[s][4 * cq]);
+            for (int s0 = sl; s0 < SX_BLOCK; s0 += SL * GROUP) {
+                float t[NR][4] = {};
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const float al = sA[s][row + r * (KP / NR)];
-                    t[r][0] = fmaf(al, u.x, t[r][0]);
-                    t[r][1] = fmaf(al, u.y, t[r][1]);
-                    t[r][2] = fmaf(al, u.z, t[r][2]);
-                    t[r][3] = fmaf(al, u.w, t[r][3]);
+                for (int g = 0; g < GROUP; ++g) {
+                    const int s = s0 + g * SL;
+                    const float4 u = *reinterpret_cast<const float4 *>(&sU[s][4 * cq]);
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        const float al = sA[s][row + r * (KP / NR)];
+                        t[r][0] = fmaf(al, u.x, t[r][0]);
+                        t[r][1] = fmaf(al, u.y, t[r][1]);
+                        t[r][2] = fmaf(al, u.z, t[r][2]);
+                        t[r][3] = fmaf(al, u.w, t[r][3]);
+                    }
                 }
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) add_kept(hi[r][c], lo[r][c], t[r][c]);
             }
-#pragma unroll
-            for (int r = 0; r < NR; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] += t[r][c];
         }
-        if (msl < MS && mk < K) {
-            float m[7] = {};
-            for (int s = msl; s < n; s += MS) add(m, sm.gamma[(b + s + 1) * K + mk], sO[s]);
-#pragma unroll
-            for (int c = 0; c < 7; ++c) mom[c] += m[c];
-        }
+        if (msl < MS && mk < K)
+            for (int s = msl; s < n; s += MS) add(m, ml, sm.gamma[(b + s + 1) * K + mk], sO[s]);
+        if (++done % SX_FLUSH == 0) flush();
     }
     if (blockIdx.x == 0 && msl == 0 && mk < K) {
-        float m[7] = {};
         const float g = sm.gamma[mk];
-        add(m, g, head[0]);
-#pragma unroll
-        for (int c = 0; c < 7; ++c) mom[c] += m[c];
+        add(m, ml, g, head[0]);
         g0[mk] = g;
     }
+    flush();
     // the slices together, in order
     const float *P = cb + lay.off_p32;
 #pragma unroll
