@@ -25,9 +25,11 @@ namespace hmm {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-// differences between met vectors are rounding, 1e-6 a step; those of vectors
-// that have not met are as large as the scores
-constexpr float VIT_TOL = 1e-3f;
+// Vectors whose paths have coalesced differ by rounding alone, which renormalising
+// at the same steps makes alike: 0 nearly always, 2e-6 at most in a float32 replay
+// (K = 4 to 64, scores to -3000). Those that have not may differ by any amount,
+// and a difference passed over is a path given up for a worse one.
+constexpr float VIT_TOL = 7.62939453125e-6f;  // 2^-17
 constexpr int64_t VIT_MOST = 16384;  // steps that a rejoin may run on
 
 // log2 P in FP32 for the recursion, and what the path's score takes in FP64:
