@@ -65,18 +65,22 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
         a[c] = k < K ? sp.ve[(idx - 1) * KP + k] : 0.0f;
         g[c] = k < K ? sp.vs[idx * KP + k] : 0.0f;
     }
+    // in every entry; never where one is not a number (fmin and fmax pass those over) or none is large enough
     auto met = [&](float tol) {
         float lo = INFINITY, hi = 0.0f;
+        bool numbers = true;
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+        for (int c = 0; c < NC; ++c) {
+            numbers = numbers && a[c] == a[c] && g[c] == g[c];
             if (a[c] > STRAND_TINY || g[c] > STRAND_TINY) {
                 const float r = a[c] / g[c];
                 lo = fminf(lo, r);
                 hi = fmaxf(hi, r);
             }
+        }
         lo = warp_min(lo);
         hi = warp_max(hi);
-        return hi <= lo * (1.0f + tol);  // false for NaN
+        return __all_sync(FULL, numbers) && hi > 0.0f && hi < INFINITY && hi <= lo * (1.0f + tol);
     };
     int ea = 0, eg = 0;  // exponents gathered while running on: a's from this piece's start, g's from piece `at`'s
     long long xa = 0, xg = 0;  // their sums

@@ -266,14 +266,18 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
     };
     auto met = [&]() {
         float lo = INFINITY, hi = 0.0f;
+        bool numbers = true;  // fmin and fmax pass over what is not
 #pragma unroll
-        for (int n = 0; n < NC; ++n)
+        for (int n = 0; n < NC; ++n) {
+            numbers = numbers && a[n] == a[n] && g[n] == g[n];
             if (a[n] > STRAND_TINY || g[n] > STRAND_TINY) {
                 const float r = a[n] / g[n];
                 lo = fminf(lo, r);
                 hi = fmaxf(hi, r);
             }
-        return all_max(hi) <= -all_max(-lo) * (1.0f + tol);
+        }
+        hi = all_max(hi);
+        return __all_sync(FULL, numbers) && hi > 0.0f && hi < INFINITY && hi <= -all_max(-lo) * (1.0f + tol);
     };
     auto fetch = [&](const float *row, float (&x)[NC]) {
 #pragma unroll

@@ -261,7 +261,7 @@ vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__res
             }
         hi = all_max(hi);
         lo = -all_max(-lo);
-        return hi - lo <= VIT_TOL;  // false for infinities
+        return hi >= lo && hi - lo <= VIT_TOL;  // false for infinities, and where no entry was compared
     };
     auto fetch = [&](const float *r, float (&x)[NC]) {
 #pragma unroll
