@@ -11,7 +11,10 @@
 // kernel reads 2 KP floats a piece; the rest are up to some hundred steps of one
 // warp each, bound by the latency of a step: 0.2 us with P's column in registers
 // (K <= 32), four steps between two looks and two renormalisations (0.3 us with a
-// look at every step), about 1 us where P comes from the cache.
+// look at every step). Beyond 32 states a CTA's four pieces are of one proposal
+// and share its P in shared memory, loaded where one of them has not met: @@ us a
+// step, 3.4 where every step fetched it through the cache (K = 48, 16 proposals,
+// T = 5000: 0.475 ms for the call, which chunk products make in 0.44; @@ now).
 #include "hmm_strand.cuh"
 
 namespace hmm {
@@ -45,25 +48,34 @@ __global__ void __launch_bounds__(32 * JOIN_WARPS)
 join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float tol0, const float *__restrict__ cblock,
             const float2 *__restrict__ packed, StrandPtrs sp) {
     __shared__ __align__(16) float2 sag[JOIN_WARPS][32 * NC];
+    extern __shared__ float sP[];  // NC > 1: P, rows of 32 NC floats
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long id = (long long)blockIdx.x * JOIN_WARPS + warp;
-    const int q = (int)(id / sp.n), s = (int)(id % sp.n);
-    if (q >= n_prop || __shfl_sync(FULL, sp.route[q], 0) != ROUTE_STRANDS) return;
-    StrandDesc d = sp.desc[s];
+    int q, s;
+    if (NC == 1) {
+        const long long id = (long long)blockIdx.x * JOIN_WARPS + warp;
+        q = (int)(id / sp.n);
+        s = (int)(id % sp.n);
+        if (q >= n_prop) return;
+    } else {  // CTAs of one proposal
+        const int cpp = (sp.n + JOIN_WARPS - 1) / JOIN_WARPS;
+        q = blockIdx.x / cpp;
+        s = (blockIdx.x % cpp) * JOIN_WARPS + warp;
+    }
+    // (another warp may change the route meanwhile: what this one does does not hang on when it looks)
+    const bool mine = s < sp.n && __shfl_sync(FULL, sp.route[q], 0) == ROUTE_STRANDS;
+    StrandDesc d = sp.desc[mine ? s : 0];
     const size_t idx = (size_t)q * sp.n + s;
-    if (d.flags & SD_FIRST) {
-        if (lane == 0) {
-            sp.logr[idx] = 0.0;
-            sp.jump[idx] = s;
-        }
-        return;
+    const bool first = (d.flags & SD_FIRST) != 0, joins = mine && !first;
+    if (mine && first && lane == 0) {
+        sp.logr[idx] = 0.0;
+        sp.jump[idx] = s;
     }
     float a[NC], g[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const int k = lane + 32 * c;
-        a[c] = k < K ? sp.ve[(idx - 1) * KP + k] : 0.0f;
-        g[c] = k < K ? sp.vs[idx * KP + k] : 0.0f;
+        a[c] = joins && k < K ? sp.ve[(idx - 1) * KP + k] : 0.0f;
+        g[c] = joins && k < K ? sp.vs[idx * KP + k] : 0.0f;
     }
     // in every entry; never where one is not a number (fmin and fmax pass those over) or none is large enough
     auto met = [&](float tol) {
@@ -88,19 +100,24 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
     int at = s;
     bool over = false;  // the segment ended before the vectors met
     bool ok = met(tol0);
+    const float *cb = cblock + (size_t)q * lay.stride;
+    const int KPl = lay.KP;
+    auto load_p = [&](int i, int k) {
+        float v = i < KPl && k < KPl ? cb[lay.off_p32 + i * KPl + k] : 0.0f;
+        if (round_tf32) {
+            uint32_t r;
+            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
+            v = __uint_as_float(r);
+        }
+        return v;
+    };
+    if (NC > 1 && __syncthreads_or(joins && !ok)) {
+        for (int x = threadIdx.x; x < KP * 32 * NC; x += 32 * JOIN_WARPS) sP[x] = load_p(x / (32 * NC), x % (32 * NC));
+        __syncthreads();
+    }
+    if (!joins) return;
     if (!ok) {
-        const float *cb = cblock + (size_t)q * lay.stride;
         const float *em = cb + lay.off_emis;
-        const int KPl = lay.KP;
-        auto load_p = [&](int i, int k) {
-            float v = i < KPl && k < KPl ? cb[lay.off_p32 + i * KPl + k] : 0.0f;
-            if (round_tf32) {
-                uint32_t r;
-                asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
-                v = __uint_as_float(r);
-            }
-            return v;
-        };
         f32x2 pc[NC == 1 ? 32 : 1];  // this lane's column of P, each entry twice
         if (NC == 1) {
 #pragma unroll
@@ -143,11 +160,11 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                 }
             } else {
 #pragma unroll 4
-                for (int i = 0; i < 32 * NC; i += 2) {
+                for (int i = 0; i < KP; i += 2) {
                     const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sag[warp][i]);
 #pragma unroll
                     for (int n = 0; n < NC; ++n) {
-                        const float v = load_p(i, lane + 32 * n), w = load_p(i + 1, lane + 32 * n);
+                        const float v = sP[i * 32 * NC + lane + 32 * n], w = sP[(i + 1) * 32 * NC + lane + 32 * n];
                         acc[n][0] = fma2(x.x, pack2(v, v), acc[n][0]);
                         acc[n][1] = fma2(x.y, pack2(w, w), acc[n][1]);
                     }
@@ -296,10 +313,12 @@ cudaError_t launch_join(int n_prop, int K, int KP, const ConstLayout &lay, int p
     const float tol = !tensor ? JOIN_TOL : precision == HMM_PREC_BF16 ? 2.44140625e-4f : 3.90625e-3f;
     const bool rt = tensor && precision == HMM_PREC_TF32;  // P as the strands have it
     const long long warps = (long long)n_prop * sp.n;
-    const unsigned grid = (unsigned)((warps + JOIN_WARPS - 1) / JOIN_WARPS);
-    if (KP <= 32) join_kernel<1><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
-    else if (KP <= 64) join_kernel<2><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
-    else join_kernel<3><<<grid, 32 * JOIN_WARPS, 0, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
+    const int nc = KP <= 32 ? 1 : KP <= 64 ? 2 : 3;
+    const unsigned grid = (unsigned)(nc == 1 ? (warps + JOIN_WARPS - 1) / JOIN_WARPS
+                                             : (long long)n_prop * ((sp.n + JOIN_WARPS - 1) / JOIN_WARPS));
+    const size_t smem = nc == 1 ? 0 : sizeof(float) * KP * 32 * nc;  // at most 30 KB
+    auto kern = nc == 1 ? join_kernel<1> : nc == 2 ? join_kernel<2> : join_kernel<3>;
+    kern<<<grid, 32 * JOIN_WARPS, smem, st>>>(n_prop, K, KP, lay, rt, tol, cblock, packed, sp);
     return cudaGetLastError();
 }
 

@@ -243,6 +243,9 @@ __global__ void __launch_bounds__(128)
 rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__restrict__ cb,
                  const float2 *__restrict__ packed, StrandPtrs sp, SmoothPtrs sm) {
     __shared__ __align__(16) float2 sag[4][32 * NC];
+    // NC > 1: P, or its transpose, where the step reads it (rows of 64 floats);
+    // through the cache a step took some 1.1 us
+    __shared__ float sP[NC == 1 ? 1 : 32 * NC][NC == 1 ? 1 : 32 * NC];
     // Every row is a result, so vectors have met where they differ by little more
     // than FP32's rounding: with rare tremors 2^-19.8 of an entry at the median and
     // 2^-18.7 at most of the time for K = 16, 2^-18.8 and 2^-17.8 for K = 32, 2^-17.9
@@ -250,9 +253,17 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
     // join takes, gamma was up to 1.3e-5 off (K = 16), 5.4e-6 now.
     const float tol = KP <= 16 ? 3.814697265625e-6f : KP <= 32 ? 7.62939453125e-6f : 1.52587890625e-5f;  // 2^-18, -17, -16
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
+    if (NC == 1 && __shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
     const float *em = cb + lay.off_emis, *P = cb + lay.off_p32;
     const int KPl = lay.KP;
+    if (NC > 1) {
+        for (int x = threadIdx.x; x < 32 * NC * 32 * NC; x += 128) {
+            const int i = x / (32 * NC), k = x % (32 * NC);
+            sP[NC == 1 ? 0 : BACK ? k : i][NC == 1 ? 0 : BACK ? i : k] = i < K && k < K ? P[i * KPl + k] : 0.0f;
+        }
+        __syncthreads();
+        if (__shfl_sync(FULL, sp.route[0], 0) != ROUTE_STRANDS) return;
+    }
     float a[NC], g[NC];
     auto all_max = [&](float v) {
 #pragma unroll
@@ -354,12 +365,11 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
                     unpack2(add2(add2(t[0], t[1]), add2(t[2], t[3])), a[0], g[0]);
                 } else {
 #pragma unroll 8
-                    for (int j = 0; j < 32 * NC; ++j) {
+                    for (int j = 0; j < K; ++j) {
                         const float2 x = sag[warp][j];
 #pragma unroll
                         for (int n = 0; n < NC; ++n) {
-                            const int k = lane + 32 * n;
-                            const float p = k < K && j < K ? (BACK ? P[k * KPl + j] : P[j * KPl + k]) : 0.0f;
+                            const float p = sP[NC == 1 ? 0 : j][NC == 1 ? 0 : lane + 32 * n];
                             a[n] = fmaf(x.x, p, a[n]);
                             g[n] = fmaf(x.y, p, g[n]);
                         }

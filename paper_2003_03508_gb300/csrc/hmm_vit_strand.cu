@@ -238,8 +238,14 @@ __global__ void __launch_bounds__(128)
 vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__restrict__ cb,
                   const float2 *__restrict__ packed, StrandPtrs sp, VitPtrs vp) {
     __shared__ float sag[4][2][32 * NC];
+    __shared__ float slp[32 * NC][32 * NC];  // log2 P
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c0 = blockIdx.x * 4 + warp;
+    for (int x = threadIdx.x; x < 32 * NC * 32 * NC; x += 128) {
+        const int i = x / (32 * NC), k = x % (32 * NC);
+        slp[i][k] = i < K && k < K ? vp.lp[i * KP + k] : -INFINITY;
+    }
+    __syncthreads();
     if (c0 >= sp.n || __shfl_sync(FULL, *vp.chunks, 0)) return;
     const float *em = cb + lay.off_emis;
     const float offt = em[EM_OFF * lay.KP], offn = em[EM_OFF * lay.KP + 1];
@@ -294,7 +300,7 @@ vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__res
                 const float xa = sag[warp][0][j], xg = sag[warp][1][j];
 #pragma unroll
                 for (int n = 0; n < NC; ++n) {
-                    const float p = lane + 32 * n < K ? vp.lp[j * KP + lane + 32 * n] : -INFINITY;
+                    const float p = slp[j][lane + 32 * n];
                     const float w = xa + p;
                     if (w > a[n]) {
                         a[n] = w;
