@@ -47,6 +47,7 @@ struct Plan {
     int strand_kp = 0;                      // 0: this shape runs on chunk products alone
     bool strand_tensor = false;             // strands on the tensor cores
     int strand_warm = 0;
+    int join_most = 0, join_budget = 0, rows_most = 0, path_most = 0;  // strand_limits
     std::vector<StrandDesc> strands;
     std::vector<int32_t> strand_order;      // longest first
     // device copies (inside plan_buf)
@@ -389,6 +390,36 @@ static int choose_strand_len(const StrandCost &c, int K, int n_prop, const std::
     return (int)best_L;
 }
 
+// How far the joins may run on before the chunk products are the quicker way.
+// Vectors of a chain that does not mix never meet, and what was spent on them is
+// lost: the joins of a likelihood get half of the time that the chunk products of
+// the call would take, those of a posterior or path about a third of the scans' for
+// each kind (all of them ran to 2048 or 16384 steps before: K=80 BF16, 32
+// proposals 43 ms for 5.3, 10 now; a path of K=25, T=105,000 12.7 ms for 4.0, 5.4 now).
+// Tremor data needs 250 steps at most, which every join may have. Times in us,
+// measured at T = 10^4 to 2^17: chunk products a start (their tree) and a time a
+// proposal-step by padded count; a join's step 0.2, 1 and 1.2 alone (up to 32, 64, 80
+// states; 0.55 since), 0.15, 0.65 and 1.1 ns where the GPU is full of them; a scan's posterior
+// and path by T and K; a row's step 0.1 (0.2 beyond 32 states), a path's 0.1 + 0.0175 K
+// (1.5).
+static void strand_limits(Plan &pl, int64_t steps) {
+    const int kp = pl.lay.KP;
+    const double root = std::sqrt((double)steps), scan = 4.5 * root * (1.0 + pl.K / 32.0);
+    const double path = 4.0 * root * (1.0 + pl.K * pl.K / 400.0);
+    double chunk = kp <= 16 ? 80.0 : kp == 32 ? 150.0 : kp == 48 ? 350.0 : kp == 64 ? 500.0 : 700.0, ns;
+    if (pl.sparse) ns = 0.3;
+    else if (pl.precision == HMM_PREC_FP32_SIMT) ns = kp <= 8 ? 0.05 : kp == 16 ? 0.25 : kp == 32 ? 2.0 : kp == 48 ? 10.0 : 14.0;
+    else ns = kp == 16 ? 0.2 : kp == 32 ? 0.27 : kp == 48 ? 0.7 : kp == 64 ? 1.3 : 2.5;
+    chunk += 1e-3 * ns * (double)steps * pl.n_prop;
+    const int wide = pl.strand_kp <= 32 ? 0 : pl.strand_kp <= 64 ? 1 : 2;
+    const double alone = wide == 0 ? 0.2 : wide == 1 ? 1.0 : 1.2, full = wide == 0 ? 0.15e-3 : wide == 1 ? 0.65e-3 : 1.1e-3;
+    const double join = pl.smooth ? 0.35 * scan : 0.5 * chunk;
+    pl.join_most = (int)std::min(2048.0, std::max(wide ? 256.0 : 320.0, join / alone)) / 32 * 32;
+    pl.join_budget = (int)std::min((double)(1 << 30), std::max((double)pl.join_most, join / (full * pl.n_prop)));
+    pl.rows_most = (int)std::min(16384.0, std::max(512.0, 0.35 * scan / (wide ? 0.2 : 0.1)));
+    pl.path_most = (int)std::min(16384.0, std::max(512.0, 0.3 * path / (wide ? 1.5 : 0.1 + 0.0175 * pl.K)));
+}
+
 static void build_strands(Plan &pl, bool sparse, int n_sms) {
     pl.strands.clear();
     pl.strand_order.clear();
@@ -427,6 +458,9 @@ static void build_strands(Plan &pl, bool sparse, int n_sms) {
     // (the few that have not run on one warp a piece, at a third of a strand's step)
     if (pl.smooth) L = std::max(L, 128);
     pl.strand_warm = pl.smooth ? 128 : strand_warm(pl.K, L, sparse, pl.strand_tensor);
+    int64_t all = 0;
+    for (int64_t m : steps) all += m;
+    strand_limits(pl, all);
     for (int s = 0; s < pl.n_seg; ++s) {
         // equal pieces of whole observation windows
         const int64_t wins = (steps[s] + OBS_WIN - 1) / OBS_WIN;
@@ -727,6 +761,9 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
         w->sp.desc = pl.d_strands;
         w->sp.order = pl.d_strand_order;
         w->sp.todo = w->obs_bad + 1;
+        w->sp.most = pl.join_most;
+        w->sp.budget = pl.join_budget;
+        w->sp.spent = cv.take<int>(n_prop);
         w->sp.route = cv.take<int>(n_prop);
         w->sp.vs = cv.take<float>(m * pl.strand_kp);
         w->sp.ve = cv.take<float>(m * pl.strand_kp);
@@ -879,6 +916,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         if (rc) return rc;
         carve(c->fb.p);
         sm.warm = pl.strand_warm;
+        sm.most = pl.rows_most;
         sm.gamma = out2->gamma;
         sm.stats = out2->stats;
         if (!out2->stats) {
@@ -1146,6 +1184,7 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
         bstate = cv.take<int32_t>(C + 1);
         bp = cv.take<uint8_t>(C * pl.L * KP);
         if (n) {
+            vp.most = pl.path_most;
             vp.lp = cv.take<float>(kp * kp);
             vp.lp64 = cv.take<double>(kp * kp);
             vp.em64 = cv.take<double>((size_t)K * 8);

@@ -102,6 +102,9 @@ struct StrandPtrs {
     int *jumps = nullptr;      // [n_prop] some piece's jump is not itself
     int *route = nullptr;      // [n_prop]
     int *todo = nullptr;       // [1 + n_prop]
+    int *spent = nullptr;      // [n_prop] steps that the proposal's joins have run on
+    int most = 0;              // how many a join may run on,
+    int budget = 0;            // and a proposal's together, before the chunk products are the quicker way
     bool bad_too = false;      // invalid parameters take the chunk products as well (they fill every output)
 };
 
@@ -110,6 +113,7 @@ struct StrandPtrs {
 constexpr int SMOOTH_PARTS = 456;  // partial sums of the E-step statistics
 struct SmoothPtrs {
     int warm = 0;              // warm-up steps of the backward strands
+    int most = 0;              // steps of the pieces that a chain of rows may pass
     float *alpha = nullptr;    // [T][KP] forward vectors, any scale (null: no posterior)
     float *gamma = nullptr;    // [T][K]
     float *u = nullptr;        // [T][KP] d o b / S of every step (null: no statistics)
@@ -124,6 +128,7 @@ struct SmoothPtrs {
 
 // The most probable path by strands (hmm_vit_strand.cu). Row i belongs to step i.
 struct VitPtrs {
+    int most = 0;              // steps of the pieces that a chain may pass
     float *lp = nullptr;       // [KP][KP] log2 P
     double *lp64 = nullptr;    // [KP][KP] log P
     double *em64 = nullptr;    // [K][8] emission constants of the score

@@ -4,17 +4,19 @@
 // tolerance in every entry, log r is noted. Otherwise both vectors run on
 // through the piece, with exact scaling, until they meet. Where the piece ends
 // first, a goes on against the strand of the next piece, and the pieces passed
-// over are taken from it (jump); after JOIN_MOST steps the proposal is sent to
-// the chunk products.
+// over are taken from it (jump). After sp.most steps of one piece, or sp.budget of
+// all of a proposal's, the proposal is sent to the chunk products, which would have
+// taken twice as long by then (strand_limits in hmm_api.cu).
 //
 // Most pieces meet at once (the warm-up covers the usual distance), so the
 // kernel reads 2 KP floats a piece; the rest are up to some hundred steps of one
 // warp each, bound by the latency of a step: 0.2 us with P's column in registers
 // (K <= 32), four steps between two looks and two renormalisations (0.3 us with a
 // look at every step). Beyond 32 states a CTA's four pieces are of one proposal
-// and share its P in shared memory, loaded where one of them has not met: @@ us a
-// step, 3.4 where every step fetched it through the cache (K = 48, 16 proposals,
-// T = 5000: 0.475 ms for the call, which chunk products make in 0.44; @@ now).
+// and share its P in shared memory, loaded where one of them has not met: 0.55 us
+// a step, eight rows' loads in flight (about 1 with four), 3.4 where every step
+// fetched it through the cache (K = 48, 16 proposals, T = 5000: 0.475 ms for the
+// call, which chunk products make in 0.44; 0.23 now).
 #include "hmm_strand.cuh"
 
 namespace hmm {
@@ -23,7 +25,6 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int JOIN_WARPS = 4;
-constexpr int JOIN_MOST = 2048;
 constexpr float JOIN_TOL = 3.0517578125e-5f;  // 2^-15: what FP32 vectors run on to
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -159,7 +160,7 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
                     acc[0][(i & 2) + 1] = fma2(x.y, pc[NC == 1 ? i + 1 : 0], acc[0][(i & 2) + 1]);
                 }
             } else {
-#pragma unroll 4
+#pragma unroll 8
                 for (int i = 0; i < KP; i += 2) {
                     const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&sag[warp][i]);
 #pragma unroll
@@ -202,7 +203,18 @@ join_kernel(int n_prop, int K, int KP, ConstLayout lay, bool round_tf32, float t
         };
         bool alive = true;
         int t0 = 0;
-        for (int done = 0; !ok && alive && done < JOIN_MOST; done += 32, t0 += 32) {
+        for (int done = 0; !ok && alive && done < sp.most; done += 32, t0 += 32) {
+            // Every 64 steps: what all joins of a proposal need is the same in any order, so whether it is
+            // above the budget is too. Another one may have given up: nothing to do here then.
+            if (done && done % 64 == 0) {
+                int sum = 0, route = ROUTE_STRANDS;
+                if (lane == 0) {
+                    sum = atomicAdd(&sp.spent[q], 64) + 64;
+                    route = *(volatile const int *)&sp.route[q];
+                }
+                if (__shfl_sync(FULL, route, 0) != ROUTE_STRANDS) return;
+                if (__shfl_sync(FULL, sum, 0) > sp.budget) break;
+            }
             if (t0 >= d.len) {
                 // this piece is over: on against the next one's strand
                 xa += off;

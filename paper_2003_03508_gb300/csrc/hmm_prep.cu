@@ -212,6 +212,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
                 const bool fits = !small && fabsf(mt) <= 1000.0f && fabsf(mn) <= 1000.0f;
                 sp.route[q] = bad ? ROUTE_BAD : ROUTE_STRANDS;
                 sp.jumps[q] = 0;
+                sp.spent[q] = 0;
                 if (bad ? sp.bad_too : !fits) {
                     sp.route[q] = ROUTE_CHUNKS;
                     sp.todo[1 + atomicAdd(&sp.todo[0], 1)] = q;

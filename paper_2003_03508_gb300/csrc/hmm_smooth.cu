@@ -234,9 +234,8 @@ strand_back_kernel(int K, int64_t steps, int warm, ConstLayout lay, const float 
 // c + 1. One warp per piece, one step after another with exact scaling. A piece
 // that ends first is noted with its true vector (unmet, carry), and a second
 // launch (`chain`) takes those on through the pieces that follow once every
-// piece has written its rows; after ROWS_MOST steps, or where two of them
+// piece has written its rows; after sm.most steps, or where two of them
 // touch, the sequence is left to the chunk products.
-constexpr int64_t ROWS_MOST = 16384;
 
 template <int NC, bool BACK>
 __global__ void __launch_bounds__(128)
@@ -461,7 +460,7 @@ rows_join_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__rest
     int64_t spent = 0;
     for (int x = x0 + 1; x < sp.n && how == 0; ++x) {
         // (all the rows that the piece's own run wrote, from a vector that was not the true one)
-        how = starts(x) || spent > ROWS_MOST ? -1 : run(piece(x), sm.unmet[piece(x)] >> 1);
+        how = starts(x) || spent > sm.most ? -1 : run(piece(x), sm.unmet[piece(x)] >> 1);
         spent += sp.desc[piece(x)].len;
         if (how == 1 && x + 1 < sp.n && (sm.unmet[piece(x)] & 1) && (sm.unmet[piece(x + 1)] & 1)) {
             ++x;

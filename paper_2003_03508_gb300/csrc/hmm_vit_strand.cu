@@ -30,7 +30,6 @@ constexpr unsigned FULL = 0xffffffffu;
 // (K = 4 to 64, scores to -3000). Those that have not may differ by any amount,
 // and a difference passed over is a path given up for a worse one.
 constexpr float VIT_TOL = 7.62939453125e-6f;  // 2^-17
-constexpr int64_t VIT_MOST = 16384;  // steps that a rejoin may run on
 
 // log2 P in FP32 for the recursion, and what the path's score takes in FP64:
 // log P and each state's emission constants
@@ -355,7 +354,7 @@ vit_rejoin_kernel(int K, int KP, bool chain, ConstLayout lay, const float *__res
     int how = 0;
     int64_t spent = 0;
     for (int x = c0 + 1; x < sp.n && how == 0; ++x) {
-        how = starts(x) || spent > VIT_MOST ? -1 : run(x, vp.unmet[x] >> 1);
+        how = starts(x) || spent > vp.most ? -1 : run(x, vp.unmet[x] >> 1);
         spent += sp.desc[x].len;
         if (how == 1 && x + 1 < sp.n && (vp.unmet[x] & 1) && (vp.unmet[x + 1] & 1)) {
             ++x;
