@@ -341,8 +341,10 @@ int hmm_tune_candidates(int32_t precision, int32_t n_prop, int32_t K, int64_t st
                         int32_t n_sms, int32_t *out, int32_t cap, int32_t *n_out);
 
 /*
- * Measures hmm_loglik_batched at every candidate chunk length for this
- * call's shape and stores the fastest. The arguments are those of
+ * Measures the chunk products of every proposal (hmm_loglik_batched as after
+ * hmm_set_strands(ctx, 0)) at every candidate chunk length for this call's
+ * shape and stores the fastest: the length matters to the proposals that
+ * vectors do not carry. The arguments are those of
  * hmm_loglik_batched (device pointers, host seg_offsets), with
  * opts->chunk_len = 0 (else HMM_EINVAL). Per candidate: one untimed call
  * (it builds the plan and grows the workspace), then `reps` (1..100) calls

@@ -207,8 +207,9 @@ static int choose_chunk_len(int precision, int n_prop, int KP, int64_t steps_tot
 
 // ---- chunk-length tuning ----
 //
-// The tuner measures a handful of chunk lengths around the cost model's
-// choice and remembers the fastest per shape. The tile shapes are fixed by
+// The tuner measures the chunk products of all proposals at a handful of chunk
+// lengths around the cost model's choice and remembers the fastest per shape; it is
+// what the proposals that vectors do not carry are given. The tile shapes are fixed by
 // the hardware mapping (M = 128 TMEM lanes, N = the padded state count), so
 // the chunk length is the schedule's free parameter: it sets the number of
 // work items, the waves the GPU runs them in, and the size of the tree.
@@ -1320,9 +1321,11 @@ int hmm_autotune_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi,
         if (e0) cudaEventDestroy(e0);
         return cuda_fail(c, e, "cudaEventCreate");
     }
-    // the tuner's own calls stay out of the phase profile
-    const bool prof_was = c->prof_on;
+    // the tuner's own calls stay out of the phase profile, and take the chunk
+    // products for every proposal: their length is what is tuned
+    const bool prof_was = c->prof_on, strands_were = c->strands_on;
     c->prof_on = false;
+    c->strands_on = false;
     int best_L = 0, rc = HMM_OK, last_rc = HMM_OK;
     double best_ms = 0.0;
     for (int L : cand) {
@@ -1356,6 +1359,7 @@ int hmm_autotune_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi,
         }
     }
     c->prof_on = prof_was;
+    c->strands_on = strands_were;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
