@@ -107,6 +107,9 @@ typedef struct {
  * input. hmm_last_chunk_proposals writes how many proposals of the context's
  * last call took the chunk products (for the one-sequence calls 0 or 1; for
  * hmm_viterbi, whether its path did). It synchronises the stream.
+ * A call whose vectors do not fit the device's memory beside the chunk products
+ * takes these alone, and so do its repeats until the shape changes or
+ * hmm_set_strands is called.
  */
 int hmm_set_strands(hmm_ctx *ctx, int on);
 int hmm_last_chunk_proposals(hmm_ctx *ctx, int32_t *n, void *stream);

@@ -28,6 +28,7 @@ namespace {
 struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
+    size_t no_room = SIZE_MAX;  // sizes from here on did not fit beside what else the device holds
 };
 
 struct Plan {
@@ -77,6 +78,7 @@ struct hmm_ctx {
     int last_L = 0;
     int n_sms = 0;
     bool strands_on = true;
+    bool work_strands = false;  // the workspace has room for the strands' vectors
     // who took chunk products in the last call: *last_todo proposals (device), or last_props where it is null
     const int *last_todo = nullptr;
     int last_props = 0;
@@ -153,6 +155,20 @@ static int ensure(hmm_ctx *c, DevBuf &b, size_t bytes) {
     }
     b.cap = want;
     return HMM_OK;
+}
+
+// A buffer of `full` bytes or, where there is no room for it, of `least` (`fits`
+// says which). A size that did not fit is not tried again: that would free and
+// allocate at every call.
+static int ensure_either(hmm_ctx *c, DevBuf &b, size_t full, size_t least, bool &fits) {
+    fits = full < b.no_room;
+    if (fits) {
+        const int rc = ensure(c, b, full);
+        if (rc != HMM_ENOMEM) return rc;
+        b.no_room = full;
+        fits = false;
+    }
+    return ensure(c, b, least);
 }
 
 // simple bump carve of an existing buffer
@@ -570,6 +586,7 @@ static bool plan_matches(const Plan &pl, int K, int n_prop, int n_seg, const int
 
 static int upload_plan(hmm_ctx *c, cudaStream_t st) {
     ++c->plan_version;
+    c->work.no_room = c->fb.no_room = SIZE_MAX;  // another shape: room is looked for again
     Plan &pl = c->plan;
     size_t bytes = 0;
     auto add = [&](size_t b) { bytes += (b + 255) & ~(size_t)255; };
@@ -671,6 +688,7 @@ int hmm_last_chunk_len(const hmm_ctx *c) { return c ? c->last_L : -1; }
 int hmm_set_strands(hmm_ctx *c, int on) {
     if (!c) return HMM_EINVAL;
     c->strands_on = on != 0;
+    c->work.no_room = c->fb.no_room = SIZE_MAX;
     return HMM_OK;
 }
 
@@ -748,7 +766,7 @@ struct WorkPtrs {
     LevelPtrs lv{};
 };
 
-static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &lay, const Plan &pl, WorkPtrs *w) {
+static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &lay, const Plan &pl, bool strands, WorkPtrs *w) {
     const int KP = lay.KP;
     Carve cv(base);
     w->cblock = cv.take<float>((size_t)n_prop * lay.stride);
@@ -756,7 +774,7 @@ static size_t carve_work(void *base, int n_prop, int n_seg, const ConstLayout &l
     // cleared together at the start of a call: obs_bad and the list's length
     w->obs_bad = cv.take<int>(2 + n_prop);
     w->sp = StrandPtrs{};
-    if (pl.strand_kp) {
+    if (strands) {
         const size_t n = pl.strands.size(), m = (size_t)n_prop * n;
         w->sp.n = (int)n;
         w->sp.desc = pl.d_strands;
@@ -865,14 +883,20 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     // ---- workspace ----
     const int KP = lay.KP;
     WorkPtrs wp;
-    const size_t main_bytes = (carve_work(nullptr, n_prop, n_seg, lay, pl, &wp) + 255) & ~(size_t)255;
+    auto carved = [&](bool strands) { return (carve_work(nullptr, n_prop, n_seg, lay, pl, strands, &wp) + 255) & ~(size_t)255; };
     // run-length table after the main carve (the other entry points never see it)
     const int nb = min_run ? rle_levels(L) : 0;
     const size_t qtab_bytes = ((size_t)n_prop * nb * KP * KP * sizeof(float) + 255) & ~(size_t)255;
     const size_t qexp_bytes = (size_t)n_prop * nb * KP * sizeof(int32_t);
-    int rc = ensure(c, c->work, main_bytes + qtab_bytes + qexp_bytes + 4096);
+    const size_t more = qtab_bytes + qexp_bytes + 4096;
+    // no room for the vectors beside the chunk products: those take every proposal
+    bool strands = pl.strand_kp && c->strands_on;
+    int rc = strands ? ensure_either(c, c->work, carved(true) + more, carved(false) + more, strands)
+                     : ensure(c, c->work, carved(false) + more);
     if (rc) return rc;
-    carve_work(c->work.p, n_prop, n_seg, lay, pl, &wp);
+    c->work_strands = strands;
+    const size_t main_bytes = carved(strands);
+    carve_work(c->work.p, n_prop, n_seg, lay, pl, strands, &wp);
     float *qtab = (float *)((char *)c->work.p + main_bytes);
     int32_t *qexp = (int32_t *)((char *)c->work.p + main_bytes + qtab_bytes);
     float *cblock = wp.cblock;
@@ -881,7 +905,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
     float2 *packed = wp.packed;
     float2 *head = wp.head;
     LevelPtrs lv = wp.lv;
-    StrandPtrs sp = c->strands_on ? wp.sp : StrandPtrs{};
+    StrandPtrs sp = wp.sp;
     sp.bad_too = mode == Mode::SMOOTH;
     SmoothPtrs sm;
     float *fvec = nullptr, *bvec = nullptr;
@@ -907,11 +931,15 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
             }
             return cv.off;
         };
-        rc = ensure(c, c->fb, carve(nullptr) + 256);
-        if (rc == HMM_ENOMEM && sp.n) {
-            // no room for two more rows a step: scans over the chunk products
+        if (sp.n) {
+            const size_t full = carve(nullptr) + 256;
+            const StrandPtrs kept = sp;
             sp = StrandPtrs{};
             sm = SmoothPtrs{};
+            bool fits = true;
+            rc = ensure_either(c, c->fb, full, carve(nullptr) + 256, fits);
+            if (fits) sp = kept;  // else no room for two more rows a step: scans over the chunk products
+        } else {
             rc = ensure(c, c->fb, carve(nullptr) + 256);
         }
         if (rc) return rc;
@@ -1169,9 +1197,9 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     const Plan &pl = c->plan;
     const int K = prm->K, KP = pl.lay.KP;
     const size_t C = std::max(1, pl.n_chunks), kp = (size_t)pl.strand_kp;
-    size_t n = pl.strand_kp && c->strands_on ? pl.strands.size() : 0;
+    size_t n = c->work_strands ? pl.strands.size() : 0;
     WorkPtrs wp;
-    carve_work(c->work.p, 1, 1, pl.lay, pl, &wp);
+    carve_work(c->work.p, 1, 1, pl.lay, pl, c->work_strands, &wp);
     VitPtrs vp;
     float *V = nullptr;
     double *voff = nullptr;
@@ -1201,11 +1229,14 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
         }
         return cv.off;
     };
-    rc = ensure(c, c->fb, carve(nullptr) + 1024);
-    if (rc == HMM_ENOMEM && n) {
-        // no room for the strands' back-pointers beside the chunks'
+    if (n) {
+        const size_t full = carve(nullptr) + 1024, kept = n;
         n = 0;
         vp = VitPtrs{};
+        bool fits = true;
+        rc = ensure_either(c, c->fb, full, carve(nullptr) + 1024, fits);
+        if (fits) n = kept;  // else no room for the strands' back-pointers beside the chunks'
+    } else {
         rc = ensure(c, c->fb, carve(nullptr) + 1024);
     }
     if (rc) return rc;
