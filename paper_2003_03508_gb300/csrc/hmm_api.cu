@@ -67,13 +67,13 @@ struct hmm_ctx {
     int device = 0;
     char err[512] = {0};
     DevBuf work;       // per-call workspace
-    DevBuf planbuf;    // plan tables
+    DevBuf planbuf[2]; // plan tables
     DevBuf stage;      // staging area for the _host entry point
     DevBuf fb;         // boundary vectors (and partial statistics) of hmm_posterior
     DevBuf gam;        // posterior vectors of hmm_expected_stats
     DevBuf stats;      // E-step statistics of hmm_loglik_grad / hmm_em_step
     unsigned *d_status = nullptr;
-    Plan plan;
+    Plan plan[2];      // of likelihoods, and of posteriors and paths: calls in turn keep both
     int last_launches = 0;
     int last_L = 0;
     int n_sms = 0;
@@ -96,7 +96,7 @@ struct hmm_ctx {
     std::vector<uint64_t> seen_key;     // the previous direct call's (a repeat is captured)
     int call_launches = 0;
     int last_graph = 0;                 // 0 direct, 1 captured and launched, 2 replayed
-    uint64_t plan_version = 0;          // advances whenever the plan tables are uploaded
+    uint64_t plan_version[2] = {};      // advances whenever the plan's tables are uploaded
 };
 
 static void drop_call_graph(hmm_ctx *c) {
@@ -584,10 +584,10 @@ static bool plan_matches(const Plan &pl, int K, int n_prop, int n_seg, const int
     return std::equal(pl.offsets.begin(), pl.offsets.end(), offs);
 }
 
-static int upload_plan(hmm_ctx *c, cudaStream_t st) {
-    ++c->plan_version;
+static int upload_plan(hmm_ctx *c, int which, cudaStream_t st) {
+    ++c->plan_version[which];
     c->work.no_room = c->fb.no_room = SIZE_MAX;  // another shape: room is looked for again
-    Plan &pl = c->plan;
+    Plan &pl = c->plan[which];
     size_t bytes = 0;
     auto add = [&](size_t b) { bytes += (b + 255) & ~(size_t)255; };
     add(sizeof(ChunkDesc) * std::max<size_t>(1, pl.chunks.size()));
@@ -597,9 +597,9 @@ static int upload_plan(hmm_ctx *c, cudaStream_t st) {
     add(sizeof(int64_t) * pl.pbase.size());
     add(sizeof(StrandDesc) * pl.strands.size());
     add(sizeof(int32_t) * pl.strand_order.size());
-    int rc = ensure(c, c->planbuf, bytes + 4096);
+    int rc = ensure(c, c->planbuf[which], bytes + 4096);
     if (rc) return rc;
-    Carve cv(c->planbuf.p);
+    Carve cv(c->planbuf[which].p);
     pl.d_chunks = cv.take<ChunkDesc>(std::max<size_t>(1, pl.chunks.size()));
     for (int l = 0; l < pl.n_levels; ++l) pl.d_groups[l] = cv.take<TreeGroup>(std::max<size_t>(1, pl.groups[l].size()));
     pl.d_segs = cv.take<SegFinal>(pl.segfinal.size());
@@ -665,7 +665,8 @@ int hmm_destroy(hmm_ctx *c) {
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     if (c->work.p) cudaFree(c->work.p);
-    if (c->planbuf.p) cudaFree(c->planbuf.p);
+    for (DevBuf &b : c->planbuf)
+        if (b.p) cudaFree(b.p);
     if (c->stage.p) cudaFree(c->stage.p);
     if (c->fb.p) cudaFree(c->fb.p);
     if (c->gam.p) cudaFree(c->gam.p);
@@ -868,16 +869,17 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         L = tune_get(key);
         if (!L) L = choose_chunk_len(prec, n_prop, lay.KP, steps_total, c->n_sms);
     }
-    if (!plan_matches(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode != Mode::LOGLIK)) {
-        build_plan(c->plan, K, n_prop, n_seg, offs, prec, L, min_run > 0, mode != Mode::LOGLIK, c->n_sms);
-        if (c->plan.n_levels + 1 > MAX_LEVELS) {
-            c->plan.valid = false;
+    const int which = mode != Mode::LOGLIK;
+    Plan &pl = c->plan[which];
+    if (!plan_matches(pl, K, n_prop, n_seg, offs, prec, L, min_run > 0, which)) {
+        build_plan(pl, K, n_prop, n_seg, offs, prec, L, min_run > 0, which, c->n_sms);
+        if (pl.n_levels + 1 > MAX_LEVELS) {
+            pl.valid = false;
             return fail(c, HMM_EINVAL, "too many chunks for the tree (raise chunk_len)");
         }
-        int rc = upload_plan(c, st);
+        int rc = upload_plan(c, which, st);
         if (rc) return rc;
     }
-    Plan &pl = c->plan;
     c->last_L = L;
 
     // ---- workspace ----
@@ -1024,7 +1026,7 @@ static int loglik_batched(hmm_ctx *c, int32_t n_prop, int32_t K, const float *pi
         const std::vector<uint64_t> key = {
             (uint64_t)(uintptr_t)pi, (uint64_t)(uintptr_t)P, (uint64_t)(uintptr_t)p, (uint64_t)(uintptr_t)mu,
             (uint64_t)(uintptr_t)cov, (uint64_t)(uintptr_t)xy, (uint64_t)(uintptr_t)tremor, (uint64_t)(uintptr_t)out,
-            (uint64_t)(uintptr_t)c->work.p, c->plan_version, (uint64_t)n_prop, (uint64_t)K, (uint64_t)n_seg,
+            (uint64_t)(uintptr_t)c->work.p, c->plan_version[which], (uint64_t)n_prop, (uint64_t)K, (uint64_t)n_seg,
             (uint64_t)prec, (uint64_t)opts.init_mode, (uint64_t)renorm, (uint64_t)min_run, (uint64_t)L,
             (uint64_t)T_total, (uint64_t)mode, (uint64_t)(todo != nullptr),
             (uint64_t)(uintptr_t)c->fb.p, (uint64_t)(uintptr_t)(out2 ? out2->gamma : nullptr),
@@ -1194,7 +1196,7 @@ int hmm_viterbi(hmm_ctx *c, const hmm_params *prm, const hmm_obs *obs, const hmm
     int rc = loglik_batched(c, 1, prm->K, prm->pi, prm->P, prm->p_tremor, prm->mu, prm->cov, 1, offs, obs->xy,
                                 obs->tremor, &o, loglik, Mode::PATH, nullptr, stream);
     if (rc) return rc;
-    const Plan &pl = c->plan;
+    const Plan &pl = c->plan[1];
     const int K = prm->K, KP = pl.lay.KP;
     const size_t C = std::max(1, pl.n_chunks), kp = (size_t)pl.strand_kp;
     size_t n = c->work_strands ? pl.strands.size() : 0;
