@@ -11,8 +11,7 @@
 // and w / S is what the expected transition counts need:
 //     N_ij = P_ij sum_t alpha_{t-1}(i) w_t(j) / S_t,
 // a K x T by T x K product taken over blocks of 64 steps in FP32 and summed in
-// FP64. The gamma-weighted moments are taken about each state's mean, so that
-// their FP32 block sums lose nothing to the coordinates' size.
+// FP64. The gamma-weighted moments keep what their FP32 products and sums drop.
 //
 // Vectors that have not met at a piece's edge run on from the true one, and the
 // rows passed are written again (rows_join_kernel).
@@ -482,7 +481,7 @@ __device__ __forceinline__ void add_kept(float &hi, float &lo, float x) {
 }
 
 // One CTA per range of steps: sum of alpha_i (x) u_i times P, and the gamma
-// moments about the states' means. Sums as in 64 bits: every term rounded to
+// moments. Sums as in 64 bits: every term of N rounded to
 // FP32, groups of SX_GROUP products in FP32 (a quiet stretch adds nearly the same
 // term again and again, whose rounding would repeat), what their additions drop
 // kept beside them for up to SX_FLUSH blocks of 64 steps, FP64 across those. FP64
@@ -506,25 +505,33 @@ stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__
     if (sp.route[0] != ROUTE_STRANDS) return;
     const int tid = threadIdx.x;
     const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(i0 + per, steps);
-    const float *em = cb + lay.off_emis;
     double *out = part + (size_t)blockIdx.x * (K * K + 7 * K);
 
     const int cq = tid % CQ, row = (tid / CQ) % (KP / NR), sl = tid / (CQ * (KP / NR));
     double acc[NR][4] = {};
     const int mk = tid % KP, msl = tid / KP;
-    const float mx = mk < K ? em[EM_MUX * lay.KP + mk] : 0.0f, my = mk < K ? em[EM_MUY * lay.KP + mk] : 0.0f;
     double mom[7] = {};
     // gamma rows: i + 1 for each of this CTA's steps i, and row 0 for the first CTA
+    // (products with what their rounding drops: a sum of squares near the origin
+    // by a mean far from it would be lost in squares about the mean)
     auto add = [&](float (&s)[7], float (&l)[7], float g, float2 o) {
         add_kept(s[0], l[0], g);
         if (!isnan(o.x)) {
-            const float dx = o.x - mx, dy = o.y - my;
+            const float gx = __fmul_rn(g, o.x), gy = __fmul_rn(g, o.y);
+            const float ex = fmaf(g, o.x, -gx), ey = fmaf(g, o.y, -gy);
+            auto square = [&](int c, float h, float e, float z) {
+                const float q = __fmul_rn(h, z);
+                add_kept(s[c], l[c], q);
+                l[c] += fmaf(e, z, fmaf(h, z, -q));
+            };
             add_kept(s[1], l[1], g);
-            add_kept(s[2], l[2], g * dx);
-            add_kept(s[3], l[3], g * dy);
-            add_kept(s[4], l[4], g * dx * dx);
-            add_kept(s[5], l[5], g * dx * dy);
-            add_kept(s[6], l[6], g * dy * dy);
+            add_kept(s[2], l[2], gx);
+            l[2] += ex;
+            add_kept(s[3], l[3], gy);
+            l[3] += ey;
+            square(4, gx, ex, o.x);
+            square(5, gx, ex, o.y);
+            square(6, gy, ey, o.y);
         }
     };
     float hi[NR][4] = {}, lo[NR][4] = {}, m[7] = {}, ml[7] = {};
@@ -614,13 +621,7 @@ stats_kernel(int K, int64_t steps, int64_t per, ConstLayout lay, const float *__
             for (int x = 0; x < MS; ++x) s[c] += red[tid + x * KP][0];
     }
     if (msl == 0 && mk < K) {
-        // back from the mean: S_x = sum g dx + mx sum g, and so on
-        const double ux = mx, uy = my;
-        const double v[7] = {s[0], s[1], s[2] + ux * s[1], s[3] + uy * s[1],
-                             s[4] + 2.0 * ux * s[2] + ux * ux * s[1],
-                             s[5] + ux * s[3] + uy * s[2] + ux * uy * s[1],
-                             s[6] + 2.0 * uy * s[3] + uy * uy * s[1]};
-        for (int c = 0; c < 7; ++c) out[K * K + c * K + mk] = v[c];
+        for (int c = 0; c < 7; ++c) out[K * K + c * K + mk] = s[c];
     }
 }
 
