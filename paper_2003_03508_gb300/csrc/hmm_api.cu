@@ -359,9 +359,9 @@ static StrandCost strand_cost(bool tensor, int KP, int precision) {
 }
 
 // Warm-up steps. Vectors on tremor data meet after 25 steps at the median and
-// 200 at most; the join carries those that have not met at less than the cost
-// of a longer warm-up for all (K=32, 64 segments, 64 proposals: 1273 us at 128,
-// 1365 at 256; K=25, T=2^20, one chain: 119 us at 64, 131 at 128). With the
+// 250 at most; the join carries those that have not met at less than the cost
+// of a longer warm-up for all (K=32, 64 segments, 64 proposals: 7% more at 256
+// than at 128; K=25, T=2^20, one chain: 10% more at 128 than at 64). With the
 // run-length option tremors are rare: 260 at the median, 800 at most.
 // (The join's step is dearer beyond 32 states: K=45, T=9000, 20 proposals 470 to
 // 1260 us at 512, 220 to 690 at 768.)
@@ -394,8 +394,8 @@ static int choose_strand_len(const StrandCost &c, int K, int n_prop, const std::
         const int64_t waves = std::max<int64_t>(1, (warps + cap - 1) / cap);
         const int64_t per_sched = (std::min(warps, cap) + 4 * n_sms - 1) / (4 * n_sms);
         const double step = (double)std::max<int64_t>(c.latency, per_sched * c.issue);
-        // and the joins that run on, 6 cycles a piece over the whole GPU (64 segments,
-        // 64 proposals: 1422 us for 1829 where short pieces were chosen without)
+        // and the joins that run on, 6 cycles a piece over the whole GPU (from two draws of
+        // 64 segments, 64 proposals: 1422 us for 1829 where short pieces were chosen without)
         const double joins = K <= 32 ? 6.0 * (double)n_prop * (double)n : 0.0;
         const double t = (double)waves * (double)(std::min<int64_t>(L, longest) + strand_warm(K, (int)L, sparse, c.tensor)) * step + joins;
         if (!best_L || t < best) {
@@ -413,25 +413,27 @@ static int choose_strand_len(const StrandCost &c, int K, int n_prop, const std::
 // the call would take, those of a posterior or path about a third of the scans' for
 // each kind (all of them ran to 2048 or 16384 steps before: K=80 BF16, 32
 // proposals 43 ms for 5.3, 10 now; a path of K=25, T=105,000 12.7 ms for 4.0, 5.4 now).
-// Tremor data needs 250 steps at most, which every join may have. Times in us,
-// measured at T = 10^4 to 2^17: chunk products a start (their tree) and a time a
-// proposal-step by padded count; a join's step 0.2, 1 and 1.2 alone (up to 32, 64, 80
-// states; 0.55 since), 0.15, 0.65 and 1.1 ns where the GPU is full of them; a scan's posterior
-// and path by T and K; a row's step 0.1 (0.2 beyond 32 states), a path's 0.1 + 0.0175 K
-// (1.5).
+// Tremor data needs 250 steps at most, rare tremors (the run-length option) 300
+// beyond the warm-up, which every join may have. Times in us, measured at T = 10^4
+// to 2^17: chunk products a start (their tree) and a time a proposal-step by padded
+// count; a join's step 0.2, 1 and 1.2 alone (up to 32, 64, 80 states; the latter 0.55
+// since), 0.15, 0.65 and 1.1 ns where the GPU is full of them; a scan's posterior and
+// path by T and K; a row's step 0.1 (0.2 beyond 32 states), a path's 0.1 + 0.0175 K (1.5).
 static void strand_limits(Plan &pl, int64_t steps) {
     const int kp = pl.lay.KP;
     const double root = std::sqrt((double)steps), scan = 4.5 * root * (1.0 + pl.K / 32.0);
     const double path = 4.0 * root * (1.0 + pl.K * pl.K / 400.0);
     double chunk = kp <= 16 ? 80.0 : kp == 32 ? 150.0 : kp == 48 ? 350.0 : kp == 64 ? 500.0 : 700.0, ns;
-    if (pl.sparse) ns = 0.3;
-    else if (pl.precision == HMM_PREC_FP32_SIMT) ns = kp <= 8 ? 0.05 : kp == 16 ? 0.25 : kp == 32 ? 2.0 : kp == 48 ? 10.0 : 14.0;
+    if (pl.sparse) {
+        chunk = kp <= 32 ? 200.0 : 1000.0;
+        ns = kp <= 32 ? 0.35 : 2.0;
+    } else if (pl.precision == HMM_PREC_FP32_SIMT) ns = kp <= 8 ? 0.05 : kp == 16 ? 0.25 : kp == 32 ? 2.0 : kp == 48 ? 10.0 : 14.0;
     else ns = kp == 16 ? 0.2 : kp == 32 ? 0.27 : kp == 48 ? 0.7 : kp == 64 ? 1.3 : 2.5;
     chunk += 1e-3 * ns * (double)steps * pl.n_prop;
     const int wide = pl.strand_kp <= 32 ? 0 : pl.strand_kp <= 64 ? 1 : 2;
     const double alone = wide == 0 ? 0.2 : wide == 1 ? 1.0 : 1.2, full = wide == 0 ? 0.15e-3 : wide == 1 ? 0.65e-3 : 1.1e-3;
     const double join = pl.smooth ? 0.35 * scan : 0.5 * chunk;
-    pl.join_most = (int)std::min(2048.0, std::max(wide ? 256.0 : 320.0, join / alone)) / 32 * 32;
+    pl.join_most = (int)std::min(2048.0, std::max(pl.sparse ? 640.0 : wide ? 256.0 : 320.0, join / alone)) / 32 * 32;
     pl.join_budget = (int)std::min((double)(1 << 30), std::max((double)pl.join_most, join / (full * pl.n_prop)));
     pl.rows_most = (int)std::min(16384.0, std::max(512.0, 0.35 * scan / (wide ? 0.2 : 0.1)));
     pl.path_most = (int)std::min(16384.0, std::max(512.0, 0.3 * path / (wide ? 1.5 : 0.1 + 0.0175 * pl.K)));

@@ -73,7 +73,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
     float *cb = cblock + (size_t)q * lay.stride;
     float *em = cb + lay.off_emis;
     __shared__ float s_ctr[80], s_cno[80], s_centre[2];
-    __shared__ double s_ctr64[80];
+    __shared__ double s_ctr64[80], s_quiet[80];
     const int lane = threadIdx.x & 31;
     bool bad = false, small = false, far = false;
 
@@ -124,6 +124,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
             const float v = use ? (float)log2(1.0 - pk) : -INFINITY;
             em[EM_CNO * KP + k] = v;
             s_cno[k] = v;
+            s_quiet[k] = use ? 1.0 - pk : 0.0;
         } else {
             // the quadratic form as two squares (Cholesky factor of the precision matrix)
             const double ux = use ? sqrt(0.5 * LOG2E * syy / det) : 0.0, wy = use ? sqrt(0.5 * LOG2E / syy) : 0.0;
@@ -195,7 +196,7 @@ __device__ __forceinline__ void prep_proposal(int q, int K, const ConstLayout &l
         constexpr double EX2_BIAS = 7.2e-8;
         for (int k = lane; k < KP; k += 32) {
             em[EM_SC * KP + k] = (float)((double)mt - s_ctr64[k] - EX2_BIAS);
-            em[EM_QF * KP + k] = s_cno[k] > -INFINITY ? (float)((1.0 - (double)p[k]) * (double)pow2f(-(int)mn)) : 0.0f;
+            em[EM_QF * KP + k] = (float)(s_quiet[k] * (double)pow2f(-(int)mn));
         }
         if (lane == 0) {
             em[EM_OFF * KP] = mt;

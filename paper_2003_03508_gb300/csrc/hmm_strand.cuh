@@ -4,7 +4,7 @@
 // such rows because the row entering the chunk is not known when the chunk
 // runs; but the products of a chain that mixes forget where they started: any
 // two positive vectors run through the same steps become proportional, after
-// some 25 steps at the median and 200 at most on tremor data (about 800 where
+// some 25 steps at the median and 250 at most on tremor data (about 800 where
 // tremors are rare). So every piece of a segment carries ONE vector, 2 K^2
 // flops a step in place of 2 K^3:
 //   * a strand starts `warm` steps before its piece from a flat vector, notes
@@ -16,9 +16,9 @@
 //     times the strand's for the rest of the chain: the piece contributes
 //     log r + its exponents, and the error is at most the tolerance, once per
 //     piece. If it is not, the join runs both vectors on until it is.
-//   * a piece whose two vectors do not meet before its end (a chain that does
-//     not mix: P = I), and a P with an entry below PMIN (next paragraph), send
-//     the whole proposal to the chunk products.
+//   * a proposal whose joins would run on for longer than its chunk products
+//     take (a chain that does not mix), or whose P has an entry below PMIN (next
+//     paragraph), goes to the chunk products as a whole.
 //
 // Range. Entries below 2^-126 flush to zero. The vector is renormalised every
 // four steps and the steps between are checked to shrink it by no more than
